@@ -293,7 +293,7 @@ __device__ __forceinline__ void node_velocity(const R (&g)[9], R alpha, R eps, R
 
 // Eq. 27 force, Eq. 30 equilibrium and Eq. 31 forcing (with the 1/eps on the
 // u.F term, the mass-conserving reading), then the BGK update of Eq. 29,
-// g* = g + (g_eq - g)/tau + F_i.
+// g* = g + (g_eq - g)/tau + F_i, for FP32 and FP64 storage.
 //
 // Rounding: at Darcy velocities every deviation is dominated by its density
 // carrier w_i (rho - 1), several decades above the velocity terms.  The update
@@ -301,76 +301,63 @@ __device__ __forceinline__ void node_velocity(const R (&g)[9], R alpha, R eps, R
 //     g* = w d + [ (1 - 1/tau)(g - w d) + w (even +- odd) ],   d = rho - 1,
 // where the bracket holds only small terms (g - w d is exact when g ~ w d),
 // so the carrier is rounded twice per population instead of at every term.
-// Opposite directions share the even part of f_eq and F_i (terms in 1,
-// (e.u)^2, (e.u)(e.F)) and flip the odd part (e.u, e.F).  g[] holds the
-// streamed deviations on entry and the post-collision deviations on exit.
+//
+// Operation count: with H = 1.5 u/tau + 3A F, J = 3 u/tau + 3A F and
+// A = 1 - 1/(2 tau) the direction sums of Eqs. 30 and 31 collapse to
+//     even = (3 rho/eps) [ (e.u)(e.H) - (u.H)/3 ],   odd = rho (e.J),
+// shared by opposite directions: 108 FP32 operations per node with the mass
+// closure below.  The form before it (separate f_eq and F_i terms, and TwoSum
+// sums of the populations before and after the collision) took 241 and was
+// bound by them where the lattice fits L2: 1024^2 FP32 10.8 -> 8.8 us a step.
+// The factor 3 sits in J, not in the weight, because fl(1/9) is 4x nearer to
+// its value than fl(1/3) or fl(1/6), and F, ten times u in shale, shows it:
+// with 1/6 in the weight the velocity error against FP64 was 5 % larger, as
+// written it is 1 % smaller than the separate terms' (192^2, 200 steps).
 template <typename R>
-__device__ __forceinline__ void collide_pair(R &gi, R &gj, R w, R wd, R eu, R eF, R k1, R om, R su, R a2,
-                                             R rho3, R fb, R f3, R f9) {
-    // even:  om [rho (9/(2 eps)(e.u)^2 - 3/(2 eps) u^2)] + rho A [9/eps (e.u)(e.F) - 3/eps u.F]
-    // odd :  om [3 rho e.u] + rho A [3 e.F]
-    const R ev = om * (a2 * eu * eu - su) + (fb + f9 * eu * eF);
-    const R od = om * rho3 * eu + f3 * eF;
-    gi = wd + (k1 * (gi - wd) + w * (ev + od));
-    gj = wd + (k1 * (gj - wd) + w * (ev - od));
-}
-
-// Error-free sum of g[first..8] as hi + lo (Knuth's TwoSum per addition,
-// explicitly rounded so nothing is reassociated or contracted).
-template <typename R>
-__device__ __forceinline__ void exact_sum(const R (&g)[9], int first, R &hi, R &lo) {
-    hi = g[first];
-    lo = R(0);
-#pragma unroll
-    for (int i = first + 1; i < 9; ++i) {
-        const R s = radd(hi, g[i]);
-        const R z = rsub(s, hi);
-        const R e = radd(rsub(hi, rsub(s, z)), rsub(g[i], z));
-        hi = s;
-        lo = radd(lo, e);
-    }
+__device__ __forceinline__ R collide_pair(R &gi, R &gj, R wd, R k1, R eu, R eH, R eJ, R q, R we, R wo) {
+    const R ev = rmul(we, rfma(eu, eH, -q));
+    const R ni = radd(wd, rfma(k1, rsub(gi, wd), rfma(wo, eJ, ev)));
+    const R nj = radd(wd, rfma(k1, rsub(gj, wd), rfma(-wo, eJ, ev)));
+    const R lost = radd(rsub(gi, ni), rsub(gj, nj));  // what this pair hands to the rest population
+    gi = ni;
+    gj = nj;
+    return lost;
 }
 
 template <typename R, bool FORCH>
 __device__ __forceinline__ void collide(R (&g)[9], R alpha, R eps, R beta,
                                         const Phys<R> &ph, R &ux, R &uy) {
-    // Mass closure: the collision conserves each node's mass exactly
-    // in arithmetic, but rounding the nine stored populations does not, and
-    // the slow pressure mode integrates that per-node error over thousands of
-    // steps.  The exact sum of the streamed populations is kept, and the rest
-    // population is stored as the exact remainder after the eight moving ones
-    // (one rounding per node instead of nine).
-    R in_hi, in_lo;
-    exact_sum<R>(g, 0, in_hi, in_lo);
     R drho;
     node_velocity<R, FORCH>(g, alpha, eps, beta, ph, drho, ux, uy);
-    const R rho = R(1) + drho;
-    R Fx = eps * ph.gx - alpha * ux;
-    R Fy = eps * ph.gy - alpha * uy;
-    if (FORCH) {
-        const R bu = beta * sqrt(ux * ux + uy * uy);
-        Fx -= bu * ux;
-        Fy -= bu * uy;
-    }
-    const R ie = rrcp(eps);
-    const R om = ph.omega, k1 = R(1) - ph.omega;
-    const R rho3 = R(3) * rho;
-    const R a2 = R(4.5) * ie * rho;
-    const R su = R(1.5) * ie * rho * (ux * ux + uy * uy);
-    const R rA = rho * ph.A;
-    const R f3 = R(3) * rA;
-    const R f9 = R(9) * ie * rA;
-    const R fb = R(-3) * ie * rA * (ux * Fx + uy * Fy);
-    const R w0 = wgt<R>(0), w1 = wgt<R>(1), w2 = wgt<R>(5);
-    const R wd0 = w0 * drho, wd1 = w1 * drho, wd2 = w2 * drho;
-    g[0] = wd0 + (k1 * (g[0] - wd0) + w0 * (fb - om * su));
-    collide_pair<R>(g[1], g[3], w1, wd1, ux, Fx, k1, om, su, a2, rho3, fb, f3, f9);
-    collide_pair<R>(g[2], g[4], w1, wd1, uy, Fy, k1, om, su, a2, rho3, fb, f3, f9);
-    collide_pair<R>(g[5], g[7], w2, wd2, ux + uy, Fx + Fy, k1, om, su, a2, rho3, fb, f3, f9);
-    collide_pair<R>(g[6], g[8], w2, wd2, uy - ux, Fy - Fx, k1, om, su, a2, rho3, fb, f3, f9);
-    R out_hi, out_lo;
-    exact_sum<R>(g, 1, out_hi, out_lo);
-    g[0] = radd(rsub(in_hi, out_hi), rsub(in_lo, out_lo));
+    const R rho = radd(R(1), drho);
+    R drag = alpha;
+    if (FORCH) drag = rfma(beta, rsqrt_(rfma(ux, ux, rmul(uy, uy))), alpha);
+    const R Fx = rfma(-drag, ux, rmul(eps, ph.gx));
+    const R Fy = rfma(-drag, uy, rmul(eps, ph.gy));
+    const R k1 = R(1) - ph.omega, omH = R(1.5) * ph.omega, omJ = R(3) * ph.omega, A3 = R(3) * ph.A;
+    const R AFx = rmul(A3, Fx), AFy = rmul(A3, Fy);
+    const R Hx = rfma(omH, ux, AFx), Hy = rfma(omH, uy, AFy);
+    const R Jx = rfma(omJ, ux, AFx), Jy = rfma(omJ, uy, AFy);
+    const R q = rmul(R(1.0 / 3.0), rfma(ux, Hx, rmul(uy, Hy)));
+    // weights of the axis class (w = 1/9) and the diagonal class (1/36)
+    const R we1 = rmul(R(1.0 / 3.0), rmul(rrcp(eps), rho)), we2 = rmul(R(0.25), we1);
+    const R wo1 = rmul(wgt<R>(1), rho), wo2 = rmul(R(0.25), wo1);
+    const R wd1 = rmul(wgt<R>(1), drho), wd2 = rmul(R(0.25), wd1);
+    // Mass closure: the collision conserves each node's mass exactly in
+    // arithmetic, but rounding the nine stored populations does not, and the
+    // slow pressure mode integrates that per-node error over thousands of
+    // steps.  The rest population therefore takes up exactly what the eight
+    // moving ones lose, g0* = g0 + sum_i (g_i - g_i*): each difference is of
+    // neighbouring densities (exact by Sterbenz's lemma once within a factor
+    // of two), so one rounding per node remains instead of nine.  Measured
+    // against FP64 over 10 000 steps (128^2; Darcy, clear and mixed media) the
+    // velocity and density errors equal those of TwoSum sums, 30x below the
+    // unclosed update's.
+    const R l1 = collide_pair<R>(g[1], g[3], wd1, k1, ux, Hx, Jx, q, we1, wo1);
+    const R l2 = collide_pair<R>(g[2], g[4], wd1, k1, uy, Hy, Jy, q, we1, wo1);
+    const R l5 = collide_pair<R>(g[5], g[7], wd2, k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), q, we2, wo2);
+    const R l6 = collide_pair<R>(g[6], g[8], wd2, k1, rsub(uy, ux), rsub(Hy, Hx), rsub(Jy, Jx), q, we2, wo2);
+    g[0] = radd(g[0], radd(radd(l1, l2), radd(l5, l6)));
 }
 
 // The same update for 16-bit storage, whose own rounding (2^-8 / 2^-11)
