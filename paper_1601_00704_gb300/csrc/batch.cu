@@ -37,6 +37,11 @@ struct BTile {
     int med, y, bx, pad;
 };
 
+// Segment of k_batch_pair: rows [y0, y1) of the strip at column xs.
+struct BSeg {
+    int med, xs, y0, y1;
+};
+
 struct BMed {
     long long off_f;  // element offset of the medium's plane 0 in the f buffers
     long long off_c;  // element offset in the coefficient planes
@@ -92,6 +97,41 @@ k_batch_step(const T *__restrict__ src_all, T *__restrict__ dst_all,
             if (atomicAdd(&clock->ticket, 1u) == gridDim.x - 1) {
                 clock->ticket = 0u;
                 clock->step += 1u;
+                __threadfence();
+            }
+        }
+    }
+}
+
+// Two steps in one pass over memory (march_strip), one warp per segment.
+template <typename T, bool WALLS>
+__global__ void __launch_bounds__(kPairThreads, kPairWarps<T>)
+k_batch_pair(const T *__restrict__ src_all, T *__restrict__ dst_all, const float *__restrict__ alpha,
+             const float *__restrict__ epsv, const BSeg *__restrict__ segs, const BMed *__restrict__ meds,
+             Phys<float> ph, const __grid_constant__ Pair2 c, StepClock *__restrict__ clock) {
+    extern __shared__ __align__(16) unsigned char strip_smem[];
+    pdl_enter();
+    const BSeg t = segs[blockIdx.x];
+    const BMed m = meds[t.med];
+    Geo geo;
+    geo.nx = m.nx;
+    geo.ny = m.ny;
+    geo.plane = m.plane;
+    geo.bpr = 0;
+    if (Store<T>::kSmall) {
+        ph.step_key = step_key_of(clock->step, clock->seed);
+        ph.step_key2 = step_key_of(clock->step + 1u, clock->seed);
+    }
+    march_strip<T, WALLS, false>(*reinterpret_cast<StripSmem<T, false> *>(strip_smem), src_all + m.off_f,
+                                 dst_all + m.off_f, alpha + m.off_c, epsv + m.off_c, nullptr, geo, ph, c, t.xs, t.y0,
+                                 t.y1);
+    if (Store<T>::kSmall) {
+        __syncwarp();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            if (atomicAdd(&clock->ticket, 1u) == gridDim.x - 1) {
+                clock->ticket = 0u;
+                clock->step += 2u;
                 __threadfence();
             }
         }
@@ -274,13 +314,14 @@ struct glbm_batch {
     std::vector<char> active;
     std::vector<int> parity_of;          // buffer of a stopped medium's state
     std::vector<long long> steps_of;     // steps of a stopped medium
-    long long off_f_total = 0, off_c_total = 0, max_tiles = 0;
+    long long off_f_total = 0, off_c_total = 0, max_tiles = 0, max_segs = 0;
     void *buf[2] = {nullptr, nullptr};
     float *coef[2] = {nullptr, nullptr};  // alpha, eps
     BMed *dmed = nullptr;
     BTile *dtiles = nullptr;
+    BSeg *dsegs = nullptr;    // segments of the two-step kernel (nsegs = 0: not used)
     int *dact = nullptr;
-    int ntiles = 0, nact = 0;
+    int ntiles = 0, nact = 0, nsegs = 0;
     double *partial = nullptr;
     DevStatus *dstat = nullptr, *hstat = nullptr;
     StepClock *dclock = nullptr;
@@ -299,7 +340,8 @@ struct glbm_batch {
     int *derr = nullptr;      // persistent kernel: grid-barrier timeout flag
     int nsm = 0;
     struct Graph {
-        int parity, chunk, test;
+        int parity, end_parity, chunk, test;
+        long long launches;
         cudaGraphExec_t exec;
     };
     std::vector<Graph> graphs;
@@ -325,6 +367,10 @@ glbm_status bfail(glbm_batch *h, glbm_status s, const char *fmt, ...) {
             return bfail((h), e_ == cudaErrorMemoryAllocation ? GLBM_ENOMEM : GLBM_ECUDA,     \
                          "%s: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__, __LINE__); \
     } while (0)
+
+// Rows of a segment of the two-step kernel: at least 4 (the table's size
+// counts on it), at most 32 (4 waves of the 24-medium sweep).
+constexpr int kBatchMinRows = 4, kBatchRows = 32;
 
 int vec_of(const glbm_batch *h) { return h->elem == 2 ? 4 : 4; }
 
@@ -375,6 +421,27 @@ glbm_status build_table(glbm_batch *h) {
             for (int bx = 0; bx < md.bpr; ++bx) tiles.push_back({m, y, bx, 0});
         md.ntiles = int(tiles.size()) - md.tile0;
     }
+    // segments of the two-step kernel: as long as one wave of resident warps
+    // allows, at most kBatchRows (beyond, several waves even out the media)
+    std::vector<BSeg> segs;
+    long long nodes = 0, strip_rows = 0;
+    for (int m : act) {
+        nodes += (long long)h->med[m].nx * h->med[m].ny;
+        strip_rows += (long long)((h->med[m].nx + kStripCols - 1) / kStripCols) * h->med[m].ny;
+    }
+    if (nodes >= kPairNodes) {
+        const long long slots = (long long)h->nsm * (h->elem == 2 ? kPairWarps<__half> : kPairWarps<float>);
+        const int rows = int(std::min<long long>(kBatchRows, std::max<long long>(kBatchMinRows, (strip_rows + slots - 1) / slots)));
+        for (int m : act) {
+            const BMed &md = h->med[m];
+            const int per = (md.ny + rows - 1) / rows, len = (md.ny + per - 1) / per;
+            for (int y = 0; y < md.ny; y += len)
+                for (int x = 0; x < md.nx; x += kStripCols) segs.push_back({m, x, y, std::min(y + len, md.ny)});
+        }
+    }
+    h->nsegs = int(segs.size());
+    if (h->nsegs > h->max_segs) return bfail(h, GLBM_EINVAL, "batch: segment table overflow");
+    if (h->nsegs) BCU(h, cudaMemcpyAsync(h->dsegs, segs.data(), sizeof(BSeg) * segs.size(), cudaMemcpyHostToDevice, h->stream));
     h->ntiles = int(tiles.size());
     h->nact = int(act.size());
     if (h->ntiles > h->max_tiles) return bfail(h, GLBM_EINVAL, "batch: tile table overflow");
@@ -386,18 +453,47 @@ glbm_status build_table(glbm_batch *h) {
     return GLBM_OK;
 }
 
-template <typename T, int THREADS, bool WALLS>
-cudaError_t launch_bstep_t(glbm_batch *h, bool reduce) {
-    using R = typename Store<T>::R;
-    Phys<R> ph;
-    ph.omega = R(1.0 / h->tau);
-    ph.A = R(1.0 - 0.5 / h->tau);
-    ph.gx = R(h->gx);
-    ph.gy = R(h->gy);
-    ph.scale = R(1);
-    ph.inv_scale = R(1);
+// Storage is FP32 or BF16: collisions in FP32, unscaled, stochastic rounding.
+Phys<float> batch_phys(const glbm_batch *h) {
+    Phys<float> ph;
+    ph.omega = float(1.0 / h->tau);
+    ph.A = float(1.0 - 0.5 / h->tau);
+    ph.gx = float(h->gx);
+    ph.gy = float(h->gy);
+    ph.scale = 1.0f;
+    ph.inv_scale = 1.0f;
     ph.step_key = 0;
     ph.sr = 1;
+    return ph;
+}
+
+template <typename T, bool WALLS>
+cudaError_t launch_bpair_t(glbm_batch *h) {
+    const Phys<float> ph = batch_phys(h);
+    // the test hook counts time steps
+    bool refused = glbm_injected_failure();
+    refused = glbm_injected_failure() || refused;
+    if (refused) return cudaErrorLaunchFailure;  // nothing is launched
+    const cudaError_t e = launch_kernel_smem(
+        k_batch_pair<T, WALLS>, dim3(unsigned(h->nsegs)), dim3(kPairThreads), sizeof(StripSmem<T, false>), h->stream,
+        h->stream != nullptr, static_cast<const T *>(h->buf[h->parity]), static_cast<T *>(h->buf[h->parity ^ 1]),
+        h->coef[0], h->coef[1], h->dsegs, h->dmed, ph, make_pair2(ph), h->dclock);
+    if (e != cudaSuccess) return e;
+    h->launches++;
+    h->parity ^= 1;
+    return cudaSuccess;
+}
+
+cudaError_t launch_bpair(glbm_batch *h) {
+    const bool walls = !(h->flags & GLBM_PERIODIC_Y);
+    if (h->storage == GLBM_BF16DEV)
+        return walls ? launch_bpair_t<__nv_bfloat16, true>(h) : launch_bpair_t<__nv_bfloat16, false>(h);
+    return walls ? launch_bpair_t<float, true>(h) : launch_bpair_t<float, false>(h);
+}
+
+template <typename T, int THREADS, bool WALLS>
+cudaError_t launch_bstep_t(glbm_batch *h, bool reduce) {
+    const Phys<float> ph = batch_phys(h);
     const T *src = static_cast<const T *>(h->buf[h->parity]);
     T *dst = static_cast<T *>(h->buf[h->parity ^ 1]);
     if (glbm_injected_failure()) return cudaErrorLaunchFailure;  // test hook: nothing is launched
@@ -434,15 +530,7 @@ cudaError_t launch_bstep(glbm_batch *h, bool reduce) {
 template <typename T, int THREADS, bool WALLS>
 cudaError_t launch_persist_t(glbm_batch *h, int chunk) {
     using R = typename Store<T>::R;
-    Phys<R> ph;
-    ph.omega = R(1.0 / h->tau);
-    ph.A = R(1.0 - 0.5 / h->tau);
-    ph.gx = R(h->gx);
-    ph.gy = R(h->gy);
-    ph.scale = R(1);
-    ph.inv_scale = R(1);
-    ph.step_key = 0;
-    ph.sr = 1;
+    const Phys<float> ph = batch_phys(h);
     auto kern = k_batch_persist<T, THREADS, WALLS>;
     int per_sm = 0;
     if (cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, THREADS, 0)) return e;
@@ -487,8 +575,12 @@ cudaError_t enqueue_chunk(glbm_batch *h, int chunk, double tol) {
                                                          : launch_persist_s<float>(h, chunk);
         if (e != cudaSuccess) return e;
     } else {
-        for (int s = 0; s < chunk; ++s)
-            if (cudaError_t e = launch_bstep(h, s == chunk - 1)) return e;
+        // the last step reduces, and the field export reads the state before it
+        for (int s = 0; s < chunk;) {
+            const bool pair = h->nsegs > 0 && s + 2 < chunk;
+            if (cudaError_t e = pair ? launch_bpair(h) : launch_bstep(h, s == chunk - 1)) return e;
+            s += pair ? 2 : 1;
+        }
     }
     if (glbm_injected_failure()) return cudaErrorLaunchFailure;
     k_batch_finalize<<<h->nact, 256, 0, h->stream>>>(h->partial, h->dmed, h->dact, tol, h->dstat, h->patience);
@@ -517,8 +609,8 @@ glbm_status run_chunk(glbm_batch *h, int chunk, double tol) {
     for (auto &g : h->graphs) {
         if (g.parity == h->parity && g.chunk == chunk && g.test == test) {
             BCU(h, cudaGraphLaunch(g.exec, h->stream));
-            h->launches += chunk + 1;
-            if (chunk % 2) h->parity ^= 1;
+            h->launches += g.launches;
+            h->parity = g.end_parity;
             return GLBM_OK;
         }
     }
@@ -548,7 +640,7 @@ glbm_status run_chunk(glbm_batch *h, int chunk, double tol) {
         h->launches = l0;
         return st;
     }
-    h->graphs.push_back({p0, chunk, test, exec});
+    h->graphs.push_back({p0, h->parity, chunk, test, h->launches - l0, exec});
     BCU(h, cudaGraphLaunch(exec, h->stream));
     return GLBM_OK;
 }
@@ -564,10 +656,11 @@ void brelease(glbm_batch *h) {
     drop_graphs(h);
     for (auto &p : h->buf) glbm_guard::release(h->guards, p), p = nullptr;
     for (auto &p : h->coef) glbm_guard::release(h->guards, p), p = nullptr;
-    void *ptrs[] = {h->dmed, h->dtiles, h->dact, h->partial, h->dstat, h->dclock, h->dflag, h->stage, h->dbar, h->derr};
+    void *ptrs[] = {h->dmed, h->dtiles, h->dsegs, h->dact, h->partial, h->dstat, h->dclock, h->dflag, h->stage, h->dbar, h->derr};
     for (void *p : ptrs) glbm_guard::release(h->guards, p);
     h->dmed = nullptr;
     h->dtiles = nullptr;
+    h->dsegs = nullptr;
     h->dact = nullptr;
     h->partial = nullptr;
     h->dstat = nullptr;
@@ -628,7 +721,7 @@ glbm_status glbm_batch_create(int count, const int *nx, const int *ny, double ta
     h->active.assign(count, 1);
     h->parity_of.assign(count, 0);
     h->steps_of.assign(count, 0);
-    long long offf = 0, offc = 0, maxt = 0, maxn = 0;
+    long long offf = 0, offc = 0, maxt = 0, maxs = 0, maxn = 0;
     for (int m = 0; m < count; ++m) {
         BMed &md = h->med[m];
         md.nx = nx[m];
@@ -640,11 +733,13 @@ glbm_status glbm_batch_create(int count, const int *nx, const int *ny, double ta
         offf += 9 * md.plane;
         offc += md.plane;
         maxt += (long long)((nx[m] / 4 + 63) / 64) * ny[m];  // 64 threads per block: most tiles
+        maxs += (long long)((nx[m] + kStripCols - 1) / kStripCols) * ((ny[m] + kBatchMinRows - 1) / kBatchMinRows + 1);
         maxn = std::max(maxn, N);
     }
     h->off_f_total = offf;
     h->off_c_total = offc;
     h->max_tiles = maxt;
+    h->max_segs = maxs;
     h->stage_n = maxn;
     cudaError_t e = cudaGetDevice(&h->dev);
     if (e == cudaSuccess && !stream) {
@@ -662,6 +757,7 @@ glbm_status glbm_batch_create(int count, const int *nx, const int *ny, double ta
     if (e == cudaSuccess) e = galloc(&h->coef[1], offc * sizeof(float));
     if (e == cudaSuccess) e = galloc(&h->dmed, sizeof(BMed) * count);
     if (e == cudaSuccess) e = galloc(&h->dtiles, sizeof(BTile) * maxt);
+    if (e == cudaSuccess) e = galloc(&h->dsegs, sizeof(BSeg) * maxs);
     if (e == cudaSuccess) e = galloc(&h->dact, sizeof(int) * count);
     if (e == cudaSuccess) e = galloc(&h->partial, sizeof(double) * 2 * maxt);
     if (e == cudaSuccess) e = galloc(&h->dstat, sizeof(DevStatus) * count);

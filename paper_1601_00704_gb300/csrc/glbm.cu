@@ -11,6 +11,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -81,9 +82,10 @@ struct glbm {
     // chunks replayed from captured CUDA graphs (any storage, on a
     // non-legacy stream): key = (buffer parity at start, steps, reduce at
     // end, test, tol, FP16 scale)
+    int nsm = 0;              // SMs of the device
     struct Graph {
-        int parity;
-        long long chunk;
+        int parity, end_parity;
+        long long launches, chunk;
         int reduce, test, patience;
         double tol, scale;
         cudaGraphExec_t exec;
@@ -137,6 +139,7 @@ Phys<R> make_phys(const glbm *h) {
     p.scale = R(h->scale);
     p.inv_scale = R(1.0 / h->scale);
     p.step_key = step_key_of(uint32_t(h->tstep), h->seed);
+    p.step_key2 = step_key_of(uint32_t(h->tstep + 1), h->seed);
     p.sr = h->sr ? 1 : 0;
     p.seed = h->seed;
     return p;
@@ -206,6 +209,70 @@ glbm_status do_step(glbm *h, bool reduce, long long clock_off = -1) {
     return GLBM_EINVAL;
 }
 
+// Two steps in one launch (k_pair), segments as long as one wave of resident
+// warps allows: the fewest rows are computed twice.
+template <typename T, bool WALLS, bool FORCH>
+glbm_status launch_pair_t(glbm *h, long long clock_off) {
+    const Geo geo = make_geo(h, 4);
+    Phys<float> ph = make_phys<float>(h);
+    if (Store<T>::kSmall && clock_off >= 0) {
+        ph.clock = h->dclock;
+        ph.step_off = uint32_t(clock_off);
+    }
+    // the test hook counts time steps
+    bool refused = injected_failure();
+    refused = injected_failure() || refused;
+    if (refused) return fail(h, GLBM_ECUDA, "step launch: injected failure (test hook)");
+    const int strips = (h->nx + kStripCols - 1) / kStripCols;
+    const int segs = std::max(1, h->nsm * kPairWarps<T> / strips);
+    const int rows = std::max(2, (h->ny + segs - 1) / segs);
+    const dim3 grid(unsigned(strips) * unsigned((h->ny + rows - 1) / rows));
+    const cudaError_t err = launch_kernel_smem(
+        k_pair<T, WALLS, FORCH>, grid, dim3(kPairThreads), sizeof(StripSmem<T, FORCH>), h->stream,
+        h->stream != nullptr, static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
+        static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
+        static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), strips, rows);
+    if (err != cudaSuccess) return fail(h, GLBM_ECUDA, "step launch: %s", cudaGetErrorString(err));
+    h->launches++;
+    h->tstep += 2;
+    h->cur ^= 1;
+    return GLBM_OK;
+}
+
+template <typename T>
+glbm_status launch_pair(glbm *h, long long co) {
+    if (!(h->flags & GLBM_PERIODIC_Y))
+        return h->forch ? launch_pair_t<T, true, true>(h, co) : launch_pair_t<T, true, false>(h, co);
+    return h->forch ? launch_pair_t<T, false, true>(h, co) : launch_pair_t<T, false, false>(h, co);
+}
+
+// Rows of whole vectors, a storage that k_pair knows (not FP64, not
+// round-to-nearest) and a lattice large enough for it.
+bool pair_eligible(const glbm *h) {
+    return h->nx % 4 == 0 && h->storage != GLBM_F64 && (h->elem == 4 || h->sr) && h->N >= kPairNodes;
+}
+
+glbm_status do_pair(glbm *h, long long clock_off = -1) {
+    switch (h->storage) {
+        case GLBM_F16DEV: return launch_pair<__half>(h, clock_off);
+        case GLBM_BF16DEV: return launch_pair<__nv_bfloat16>(h, clock_off);
+        default: return launch_pair<float>(h, clock_off);
+    }
+}
+
+// `chunk` steps, the last one reducing when `reduce`.  That one is a launch of
+// its own: the velocity export reads the state before it.
+glbm_status do_steps(glbm *h, long long chunk, bool reduce, bool clocked) {
+    const long long pairs_to = pair_eligible(h) ? chunk - (reduce ? 1 : 0) : 0;
+    for (long long s = 0; s < chunk;) {
+        const bool pair = s + 2 <= pairs_to;
+        const long long co = clocked ? s : -1;
+        if (glbm_status st = pair ? do_pair(h, co) : do_step(h, reduce && s == chunk - 1, co)) return st;
+        s += pair ? 2 : 1;
+    }
+    return GLBM_OK;
+}
+
 int nparts(const glbm *h) {
     const Geo g = make_geo(h, vec_width(h));
     return g.bpr * g.ny;
@@ -264,9 +331,9 @@ glbm_status run_chunk(glbm *h, long long chunk, bool reduce, double tol) {
             if (g.parity == h->cur && g.chunk == chunk && g.reduce == int(reduce) && g.test == test &&
                 g.tol == tol && g.scale == h->scale && g.patience == h->patience) {
                 CU(h, cudaGraphLaunch(g.exec, h->stream));
-                h->launches += chunk + (reduce ? 1 : 0) + (small ? 1 : 0);
+                h->launches += g.launches;
                 h->tstep += chunk;
-                if (chunk % 2) h->cur ^= 1;
+                h->cur = g.end_parity;
                 if (reduce) h->reduced = true;
                 return GLBM_OK;
             }
@@ -277,8 +344,7 @@ glbm_status run_chunk(glbm *h, long long chunk, bool reduce, double tol) {
         const bool r0 = h->reduced;
         cudaGraph_t graph = nullptr;
         CU(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-        glbm_status st = GLBM_OK;
-        for (long long s = 0; s < chunk && !st; ++s) st = do_step(h, reduce && s == chunk - 1, small ? s : -1);
+        glbm_status st = do_steps(h, chunk, reduce, small);
         if (!st && reduce) st = finalize(h, tol);
         if (!st) st = clock_op(h, chunk, true);
         cudaError_t e = cudaStreamEndCapture(h->stream, &graph);
@@ -299,12 +365,11 @@ glbm_status run_chunk(glbm *h, long long chunk, bool reduce, double tol) {
             h->reduced = r0;
             return st;
         }
-        h->graphs[h->ngraphs++] = {p0, chunk, int(reduce), test, h->patience, tol, h->scale, exec};
+        h->graphs[h->ngraphs++] = {p0, h->cur, h->launches - l0, chunk, int(reduce), test, h->patience, tol, h->scale, exec};
         CU(h, cudaGraphLaunch(exec, h->stream));
         return GLBM_OK;
     }
-    for (long long s = 0; s < chunk; ++s)
-        if (glbm_status st = do_step(h, reduce && s == chunk - 1)) return st;
+    if (glbm_status st = do_steps(h, chunk, reduce, false)) return st;
     if (reduce)
         if (glbm_status st = finalize(h, tol)) return st;
     // keep the device step counter in step for later graph replays
@@ -488,6 +553,7 @@ glbm_status glbm_create(int nx, int ny, double tau, glbm_storage storage, unsign
     h->celem = storage == GLBM_F64 ? 8 : 4;
     h->sr = !(flags & GLBM_NEAREST16);
     cudaError_t e = cudaGetDevice(&h->dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
     const size_t fbytes = size_t(9) * h->plane * h->elem;
     const size_t cbytes = size_t(h->plane) * h->celem;
     // the scalar grid has the most blocks

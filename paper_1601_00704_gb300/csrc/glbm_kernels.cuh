@@ -195,6 +195,7 @@ struct Phys {
     const unsigned *clock = nullptr;
     uint32_t step_off = 0;
     uint32_t seed = 0;
+    uint32_t step_key2 = 0;  // key of the following step, for k_pair
 };
 
 // Stochastic-rounding key of time step t (host and device agree).
@@ -400,6 +401,169 @@ __device__ __forceinline__ void collide_small(R (&g)[9], R alpha, R eps, R beta,
     pair(g[2], g[4], uy, Fy, R(1));
     pair(g[5], g[7], ux + uy, Fx + Fy, R(0.25));
     pair(g[6], g[8], uy - ux, Fy - Fx, R(0.25));
+}
+
+// ---------------------------------------------------------------------------
+// The same collisions for two nodes at once on packed FP32 pairs
+// (add/mul/fma.rn.f32x2): the lane rate is that of the scalar instructions,
+// but each pair takes one issue slot, and the multi-step kernels are bound by
+// issue.  Every operation and its rounding is that of the scalar functions
+// above (negated factors stand in for subtractions), so the bits are theirs.
+// ---------------------------------------------------------------------------
+struct f2 {
+    unsigned long long v;
+};
+__host__ __device__ __forceinline__ f2 mk2(float lo, float hi) {
+#ifdef __CUDA_ARCH__
+    f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+#else
+    uint32_t a, b;
+    memcpy(&a, &lo, 4);
+    memcpy(&b, &hi, 4);
+    return f2{(unsigned long long)b << 32 | a};
+#endif
+}
+__host__ __device__ __forceinline__ f2 bc2(float x) { return mk2(x, x); }
+__device__ __forceinline__ float lo2(f2 a) {
+    return __uint_as_float(uint32_t(a.v));
+}
+__device__ __forceinline__ float hi2(f2 a) {
+    return __uint_as_float(uint32_t(a.v >> 32));
+}
+__device__ __forceinline__ f2 radd(f2 a, f2 b) {
+    f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f2 rsub(f2 a, f2 b) {
+    f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f2 rmul(f2 a, f2 b) {
+    f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ f2 rfma(f2 a, f2 b, f2 c) {
+    f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ f2 rrcp(f2 a) { return mk2(rrcp(lo2(a)), rrcp(hi2(a))); }
+__device__ __forceinline__ f2 rsqrt_(f2 a) { return mk2(rsqrt_(lo2(a)), rsqrt_(hi2(a))); }
+
+// Launch constants as pairs, made on the host so that they sit in the
+// constant bank.
+struct Pair2 {
+    f2 one, half, quarter, hgx, hgy, ngx, ngy, k1;
+    f2 omH, omJ, nA3, nthird, third, w1, nw1;            // 32-bit storage
+    f2 cA, cO, ncO, w1om, four, cO3, ncA3, cO2, ncA;     // 16-bit storage
+    f2 scale, inv_s;
+};
+inline Pair2 make_pair2(const Phys<float> &p) {
+    Pair2 c;
+    const float w1 = 1.0f / 9.0f, om = p.omega, cA = (3.0f * w1) * p.A, cO = (1.5f * w1) * om;
+    c.one = bc2(1.0f), c.half = bc2(0.5f), c.quarter = bc2(0.25f);
+    c.hgx = bc2(0.5f * p.gx), c.hgy = bc2(0.5f * p.gy), c.ngx = bc2(-p.gx), c.ngy = bc2(-p.gy);
+    c.k1 = bc2(1.0f - om);
+    c.omH = bc2(1.5f * om), c.omJ = bc2(3.0f * om), c.nA3 = bc2(-(3.0f * p.A));
+    c.nthird = bc2(-(1.0f / 3.0f)), c.third = bc2(1.0f / 3.0f), c.w1 = bc2(w1), c.nw1 = bc2(-w1);
+    c.cA = bc2(cA), c.ncA = bc2(-cA), c.cO = bc2(cO), c.ncO = bc2(-cO), c.w1om = bc2(w1 * om), c.four = bc2(4.0f);
+    c.cO3 = bc2(3.0f * cO), c.ncA3 = bc2(-(3.0f * cA)), c.cO2 = bc2(2.0f * cO);
+    c.scale = bc2(p.scale), c.inv_s = bc2(p.inv_scale);
+    return c;
+}
+
+// node_velocity for a pair.
+template <bool FORCH>
+__device__ __forceinline__ void node_velocity2(const f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c, f2 &drho,
+                                               f2 &rho, f2 &ux, f2 &uy) {
+    drho = radd(radd(radd(g[0], radd(g[1], g[3])), radd(g[2], g[4])), radd(radd(g[5], g[7]), radd(g[6], g[8])));
+    const f2 d57 = rsub(g[5], g[7]), d86 = rsub(g[8], g[6]);
+    const f2 mx = radd(radd(rsub(g[1], g[3]), d57), d86);
+    const f2 my = rsub(radd(rsub(g[2], g[4]), d57), d86);
+    rho = radd(c.one, drho);
+    const f2 ir = rrcp(rho);
+    const f2 vx = rfma(mx, ir, rmul(eps, c.hgx)), vy = rfma(my, ir, rmul(eps, c.hgy));
+    f2 den;
+    if (FORCH) {
+        const f2 c0 = rfma(c.quarter, alpha, c.half), c1 = rmul(c.half, beta);
+        const f2 vmag = rsqrt_(rfma(vx, vx, rmul(vy, vy)));
+        den = radd(c0, rsqrt_(rfma(c1, vmag, rmul(c0, c0))));
+    } else {
+        den = rfma(c.half, alpha, c.one);
+    }
+    const f2 iden = rrcp(den);
+    ux = rmul(vx, iden);
+    uy = rmul(vy, iden);
+}
+
+__device__ __forceinline__ f2 collide_pair2(f2 &gi, f2 &gj, f2 wd, f2 k1, f2 eu, f2 eH, f2 eJ, f2 nq, f2 we, f2 wo,
+                                            f2 nwo) {
+    const f2 ev = rmul(we, rfma(eu, eH, nq));
+    const f2 ni = radd(wd, rfma(k1, rsub(gi, wd), rfma(wo, eJ, ev)));
+    const f2 nj = radd(wd, rfma(k1, rsub(gj, wd), rfma(nwo, eJ, ev)));
+    const f2 lost = radd(rsub(gi, ni), rsub(gj, nj));
+    gi = ni;
+    gj = nj;
+    return lost;
+}
+
+// collide for a pair.
+template <bool FORCH>
+__device__ __forceinline__ void collide2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c) {
+    f2 drho, rho, ux, uy;
+    node_velocity2<FORCH>(g, alpha, eps, beta, c, drho, rho, ux, uy);
+    f2 drag = alpha;
+    if (FORCH) drag = rfma(beta, rsqrt_(rfma(ux, ux, rmul(uy, uy))), alpha);
+    const f2 AFx = rmul(c.nA3, rfma(drag, ux, rmul(eps, c.ngx)));  // -3A (-F)
+    const f2 AFy = rmul(c.nA3, rfma(drag, uy, rmul(eps, c.ngy)));
+    const f2 Hx = rfma(c.omH, ux, AFx), Hy = rfma(c.omH, uy, AFy);
+    const f2 Jx = rfma(c.omJ, ux, AFx), Jy = rfma(c.omJ, uy, AFy);
+    const f2 nq = rmul(c.nthird, rfma(ux, Hx, rmul(uy, Hy)));
+    const f2 we1 = rmul(c.third, rmul(rrcp(eps), rho)), we2 = rmul(c.quarter, we1);
+    const f2 wo1 = rmul(c.w1, rho), wo2 = rmul(c.quarter, wo1);
+    const f2 nwo1 = rmul(c.nw1, rho), nwo2 = rmul(c.quarter, nwo1);
+    const f2 wd1 = rmul(c.w1, drho), wd2 = rmul(c.quarter, wd1);
+    const f2 l1 = collide_pair2(g[1], g[3], wd1, c.k1, ux, Hx, Jx, nq, we1, wo1, nwo1);
+    const f2 l2 = collide_pair2(g[2], g[4], wd1, c.k1, uy, Hy, Jy, nq, we1, wo1, nwo1);
+    const f2 l5 = collide_pair2(g[5], g[7], wd2, c.k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), nq, we2, wo2, nwo2);
+    const f2 l6 = collide_pair2(g[6], g[8], wd2, c.k1, rsub(uy, ux), rsub(Hy, Hx), rsub(Jy, Jx), nq, we2, wo2, nwo2);
+    g[0] = radd(g[0], radd(radd(l1, l2), radd(l5, l6)));
+}
+
+// collide_small for a pair.
+template <bool FORCH>
+__device__ __forceinline__ void collide_small2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c) {
+    f2 drho, rho, ux, uy;
+    node_velocity2<FORCH>(g, alpha, eps, beta, c, drho, rho, ux, uy);
+    f2 nFx = rfma(eps, c.ngx, rmul(alpha, ux)), nFy = rfma(eps, c.ngy, rmul(alpha, uy));  // -F
+    const f2 uu = rfma(ux, ux, rmul(uy, uy));
+    if (FORCH) {
+        const f2 bu = rmul(beta, rsqrt_(uu));
+        nFx = rfma(bu, ux, nFx);
+        nFy = rfma(bu, uy, nFy);
+    }
+    const f2 ier = rmul(rrcp(eps), rho);
+    const f2 nuF = rfma(ux, nFx, rmul(uy, nFy));
+    const f2 C1 = rfma(c.w1om, drho, rmul(ier, rfma(c.ncO, uu, rmul(c.cA, nuF))));
+    const f2 P1 = rmul(c.cO3, ier), Q1 = rmul(c.ncA3, ier);
+    const f2 T1 = rmul(c.cO2, rho), U1 = rmul(c.ncA, rho);
+    g[0] = rfma(c.k1, g[0], rmul(c.four, C1));
+    auto pair = [&](f2 &gi, f2 &gj, f2 eu, f2 neF, bool diag) {
+        f2 E = rfma(eu, rfma(P1, eu, rmul(Q1, neF)), C1);
+        f2 O = rfma(T1, eu, rmul(U1, neF));
+        if (diag) E = rmul(c.quarter, E), O = rmul(c.quarter, O);
+        gi = rfma(c.k1, gi, radd(E, O));
+        gj = rfma(c.k1, gj, rsub(E, O));
+    };
+    pair(g[1], g[3], ux, nFx, false);
+    pair(g[2], g[4], uy, nFy, false);
+    pair(g[5], g[7], radd(ux, uy), radd(nFx, nFy), true);
+    pair(g[6], g[8], rsub(uy, ux), rsub(nFy, nFx), true);
 }
 
 // Per-node coefficients of VEC consecutive nodes.
@@ -668,12 +832,12 @@ __device__ __forceinline__ void pdl_enter() {
 // Host: launch `kern` on `st`, with programmatic stream serialisation when
 // `pdl` (callers pass it for non-default streams).
 template <typename... P, typename... A>
-inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, bool pdl,
-                                 A &&...args) {
+inline cudaError_t launch_kernel_smem(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                                      bool pdl, A &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
-    cfg.dynamicSmemBytes = 0;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -681,6 +845,11 @@ inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, cuda
     cfg.attrs = pdl ? at : nullptr;
     cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, cudaStream_t st, bool pdl,
+                                 A &&...args) {
+    return launch_kernel_smem(kern, grid, block, 0, st, pdl, std::forward<A>(args)...);
 }
 
 // Grid: x = blocks of a row (geo.bpr), row y = blockIdx.y + kMaxGridY *
@@ -723,6 +892,309 @@ k_step(const T *__restrict__ src, T *__restrict__ dst, const typename Store<T>::
             if (threadIdx.x == 0) pmax[blk] = gm;
         }
     }
+}
+
+// ---------------------------------------------------------------------------
+// K2b: two time steps in one pass over memory.
+//
+// The one-step kernel is bound by HBM on large lattices (FP32: 80 B per node
+// and step at 1.03 of the copy bandwidth) while its arithmetic needs less than
+// half of that time, so two steps share one read and one write.  Each warp
+// marches up a strip of 128 columns (4 per lane), one row per iteration: it
+// gathers row r and collides it (first step), then streams and collides row
+// r - 1 (second step) from the first-step populations of rows r - 2, r - 1
+// and r.  Level ones stay in registers for a row, upward ones in shared memory
+// for two, downward ones are used at once.  x neighbours come by warp shuffle
+// as in gather(); the outermost lane on each side has none beyond it, so it
+// only is the halo of the next one and a strip stores 30 of its 32 lanes'
+// columns (6 %).  Rows y0 - 1 and y1 of a segment [y0, y1) are recomputed by
+// its neighbours' warps (2/rows).  One warp per block and no barriers.
+//
+// The arithmetic runs on packed pairs because issue, not HBM, is the next
+// bound (scalar: 147 instructions per node and step, packed: 107).  Registers
+// are what is scarce: with the upward rows and the next row's loads in
+// registers, or at 5 warps per scheduler, the loop spills and loses 20 %.
+// FP32 runs best at 12 warps per SM (fewer DRAM streams), 16-bit at 16;
+// cp.async.cg, a barrier per row and 128-thread blocks were slower.
+// 4096^2, us a step: FP32 195 -> 107, BF16 112 -> 86; 2048^2: FP32 49.6 -> 28.1,
+// FP16 29.6 -> 27.0.  FP32 then moves 0.9 of the copy bandwidth.
+//
+// Both steps round, and draw their stochastic-rounding words, exactly as the
+// one-step kernel does, so the results are its bits.
+// ---------------------------------------------------------------------------
+constexpr int kPairThreads = 32;
+template <typename T>
+constexpr int kPairWarps = sizeof(T) == 2 ? 16 : 12;  // resident warps per SM
+// Fewest nodes for which k_pair is used: below, the lattice stays in L2, there
+// is less than a warp's worth of rows per segment and the one-step kernel is
+// faster (1024^2: FP32 8.4 against 8.9 us a step, BF16 6.9 against 8.4; 1280^2:
+// 16.4 against 15.6 and 11.4 against 10.6).
+constexpr long long kPairNodes = 5ll << 18;
+constexpr int kStripLanes = 30;              // lanes of a strip that store
+constexpr int kStripCols = 4 * kStripLanes;  // columns of a strip
+
+template <typename F, size_t... I>
+__device__ __forceinline__ void for_pops_(F f, std::index_sequence<I...>) {
+    (f(std::integral_constant<int, int(I)>{}), ...);
+}
+template <typename F>
+__device__ __forceinline__ void for_pops(F f) {
+    for_pops_(f, std::make_index_sequence<9>{});
+}
+
+// Four nodes of a lane as two packed pairs.
+struct Quad {
+    f2 p[2];
+};
+
+// The LCG's state after n steps is a_n x + c_n: taken directly from the seed
+// the 18 words of a lane do not wait for one another.
+struct LcgStep {
+    uint32_t a, c;
+};
+__host__ __device__ constexpr LcgStep lcg_step(int n) {
+    LcgStep s{1u, 0u};
+    for (int i = 0; i < n; ++i) s = LcgStep{s.a * 0x2C1B3C6Du, s.c * 0x2C1B3C6Du + 0x297A2D39u};
+    return s;
+}
+
+// Stored form of 4 nodes' population I of 16-bit storage, stochastically
+// rounded with states 2I+1 and 2I+2 of the LCG as in step_body.
+template <typename T, int I>
+__device__ __forceinline__ uint2 round4(Quad q, f2 scale, uint32_t seed) {
+    constexpr LcgStep s0 = lcg_step(2 * I + 1), s1 = lcg_step(2 * I + 2);
+    if (Store<T>::kScaled) q.p[0] = rmul(q.p[0], scale), q.p[1] = rmul(q.p[1], scale);
+    return make_uint2(Store<T>::pack_sr(lo2(q.p[0]), hi2(q.p[0]), seed * s0.a + s0.c),
+                      Store<T>::pack_sr(lo2(q.p[1]), hi2(q.p[1]), seed * s1.a + s1.c));
+}
+// Loaded 4 nodes of storage T as pairs.
+template <typename T>
+__device__ __forceinline__ Quad unpack4(const T (&t)[4], f2 inv_s) {
+    Quad q;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        q.p[k] = mk2(Store<T>::ld(t[2 * k], 1.0f), Store<T>::ld(t[2 * k + 1], 1.0f));
+        if constexpr (Store<T>::kSmall)
+            if (Store<T>::kScaled) q.p[k] = rmul(q.p[k], inv_s);
+    }
+    return q;
+}
+
+// x shifts within a strip: RIGHT: node x takes x - 1; else node x takes x + 1.
+template <bool RIGHT>
+__device__ __forceinline__ Quad shift4(const Quad &r) {
+    Quad o;
+    if (RIGHT) {
+        const float n = __shfl_up_sync(0xffffffffu, hi2(r.p[1]), 1);
+        o.p[0] = mk2(n, lo2(r.p[0]));
+        o.p[1] = mk2(hi2(r.p[0]), lo2(r.p[1]));
+    } else {
+        const float n = __shfl_down_sync(0xffffffffu, lo2(r.p[0]), 1);
+        o.p[0] = mk2(hi2(r.p[0]), lo2(r.p[1]));
+        o.p[1] = mk2(hi2(r.p[1]), n);
+    }
+    return o;
+}
+
+template <typename T, bool FORCH>
+__device__ __forceinline__ void collide4(Quad (&g)[9], const Quad &a, const Quad &e, const Quad &b, const Pair2 &c) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+        f2 n[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) n[i] = g[i].p[k];
+        if constexpr (Store<T>::kSmall) collide_small2<FORCH>(n, a.p[k], e.p[k], b.p[k], c);
+        else collide2<FORCH>(n, a.p[k], e.p[k], b.p[k], c);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) g[i].p[k] = n[i];
+    }
+}
+
+// Shared memory of one warp.  Every lane reads back only what it wrote or
+// copied itself, so no barrier is needed.
+//  f, coef  row r + 1 travels here by cp.async while row r is computed; the
+//           coefficients stay for the second step of row r, a row later
+//  up       first-step upward populations of the last two rows
+template <typename T, bool FORCH>
+struct StripSmem {
+    struct Vec {
+        T v[4];
+    };
+    float4 coef[3][FORCH ? 3 : 2][32];
+    float4 up[2][3][32];
+    alignas(16) Vec f[9][32];
+};
+template <int B>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(unsigned(__cvta_generic_to_shared(smem))),
+                 "l"(gmem), "n"(B)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// Rows [y0, y1) of the strip whose stored columns begin at xs, two steps.
+// nx must be a multiple of 4; ph.step_key / step_key2 key the two steps;
+// `sm` is this warp's own.
+template <typename T, bool WALLS, bool FORCH>
+__device__ __forceinline__ void march_strip(StripSmem<T, FORCH> &sm, const T *__restrict__ src, T *__restrict__ dst,
+                                            const float *__restrict__ alpha, const float *__restrict__ epsv,
+                                            const float *__restrict__ betav, const Geo &geo, const Phys<float> &ph,
+                                            const Pair2 &c, int xs, int y0, int y1) {
+    const int nx = geo.nx, ny = geo.ny;
+    const int lane = threadIdx.x & 31;
+    const int groups = nx >> 2;
+    int grp = (xs >> 2) + lane - 1;  // this lane's column group, wrapped around the period
+    grp = grp < 0 ? grp + groups : grp;
+    grp = grp >= groups ? grp % groups : grp;
+    const int x0 = grp << 2;
+    const bool store = lane >= 1 && lane <= kStripLanes && xs + 4 * (lane - 1) < nx;
+    const bool at_lo = WALLS && y0 == 0, at_hi = WALLS && y1 == ny;
+
+    const Quad zero{{f2{0}, f2{0}}};
+    Quad c0 = zero, c1 = zero, c3 = zero;  // first-step rest and level populations of row r - 1 (x-shifted)
+    int slot = 0;                          // coefficient slot of row r
+    auto row_of = [&](int r) { return WALLS ? r : (r < 0 ? r + ny : (r >= ny ? r - ny : r)); };
+    // start the copies of row r: population i comes from row r - e_y, at a wall
+    // from its opposite in row r (halfway bounce-back)
+    auto fetch = [&](int r, int cs) {
+        const int rr = row_of(r);
+        const bool lo = WALLS && rr == 0, hi = WALLS && rr == ny - 1;
+        const long long row = (long long)rr * nx + x0;
+        const long long rm = !WALLS && rr == 0 ? (long long)(ny - 1) * nx + x0 : row - nx;
+        const long long rp = !WALLS && rr == ny - 1 ? x0 : row + nx;
+        cp_async<16>(&sm.coef[cs][0][lane], alpha + row);
+        cp_async<16>(&sm.coef[cs][1][lane], epsv + row);
+        if (FORCH) cp_async<16>(&sm.coef[cs][FORCH ? 2 : 0][lane], betav + row);
+        constexpr int B = 4 * sizeof(T);
+        const long long pl = geo.plane;
+        cp_async<B>(&sm.f[0][lane], src + row);
+        cp_async<B>(&sm.f[1][lane], src + pl + row);
+        cp_async<B>(&sm.f[3][lane], src + 3 * pl + row);
+        cp_async<B>(&sm.f[2][lane], src + (lo ? 4 * pl + row : 2 * pl + rm));
+        cp_async<B>(&sm.f[5][lane], src + (lo ? 7 * pl + row : 5 * pl + rm));
+        cp_async<B>(&sm.f[6][lane], src + (lo ? 8 * pl + row : 6 * pl + rm));
+        cp_async<B>(&sm.f[4][lane], src + (hi ? 2 * pl + row : 4 * pl + rp));
+        cp_async<B>(&sm.f[7][lane], src + (hi ? 5 * pl + row : 7 * pl + rp));
+        cp_async<B>(&sm.f[8][lane], src + (hi ? 6 * pl + row : 8 * pl + rp));
+    };
+    // row ny of a walled lattice is the upper wall's mirror, made from row ny - 1
+    const int r_first = at_lo ? 0 : y0 - 1, r_last = at_hi ? ny - 1 : y1;
+    fetch(r_first, 0);
+    cp_async_commit();
+    for (int r = r_first; r <= y1; ++r) {
+        const int next = slot == 2 ? 0 : slot + 1, prev = slot == 0 ? 2 : slot - 1;
+        Quad h0, h2, h4, s1, s3, s5, s6, s7, s8;
+        if (at_hi && r == ny) {
+            // halfway bounce-back: what left row ny - 1 upwards returns reversed
+            // to its own node (undo the x shift of 5 and 6)
+            Quad u5, u6;
+            memcpy(&h4, &sm.up[(r - 1) & 1][0][lane], 16);
+            memcpy(&u5, &sm.up[(r - 1) & 1][1][lane], 16);
+            memcpy(&u6, &sm.up[(r - 1) & 1][2][lane], 16);
+            s7 = shift4<false>(u5);
+            s8 = shift4<true>(u6);
+            h0 = s1 = s3 = h2 = s5 = s6 = zero;
+        } else {
+            const int rr = row_of(r);
+            const bool lo = WALLS && rr == 0, hi = WALLS && rr == ny - 1;
+            Quad h[9], a, e, b = zero;
+            cp_async_wait<0>();
+            memcpy(&a, &sm.coef[slot][0][lane], 16);
+            memcpy(&e, &sm.coef[slot][1][lane], 16);
+            if (FORCH) memcpy(&b, &sm.coef[slot][FORCH ? 2 : 0][lane], 16);
+            Quad f[9];
+#pragma unroll
+            for (int i = 0; i < 9; ++i) f[i] = unpack4<T>(sm.f[i][lane].v, c.inv_s);
+            h[0] = f[0], h[2] = f[2], h[4] = f[4];
+            h[1] = shift4<true>(f[1]);
+            h[3] = shift4<false>(f[3]);
+            h[5] = lo ? f[5] : shift4<true>(f[5]);
+            h[6] = lo ? f[6] : shift4<false>(f[6]);
+            h[7] = hi ? f[7] : shift4<false>(f[7]);
+            h[8] = hi ? f[8] : shift4<true>(f[8]);
+            if (r + 1 <= r_last) fetch(r + 1, next);  // row r is in registers by now
+            cp_async_commit();
+            collide4<T, FORCH>(h, a, e, b, c);
+            if constexpr (Store<T>::kSmall) {
+                const uint32_t seed = mix32(uint32_t((long long)rr * nx + x0) ^ ph.step_key);
+                for_pops([&](auto i) {
+                    const uint2 w = round4<T, i.value>(h[i.value], c.scale, seed);
+                    T t[4];
+                    memcpy(t, &w, 8);
+                    h[i.value] = unpack4<T>(t, c.inv_s);
+                });
+            }
+            h0 = h[0], h2 = h[2], h4 = h[4];
+            s1 = shift4<true>(h[1]);
+            s3 = shift4<false>(h[3]);
+            s5 = shift4<true>(h[5]);
+            s6 = shift4<false>(h[6]);
+            s7 = shift4<false>(h[7]);
+            s8 = shift4<true>(h[8]);
+            if (lo) {  // the lower wall returns row 0's own downward populations
+                memcpy(&sm.up[1][0][lane], &h[4], 16);
+                memcpy(&sm.up[1][1][lane], &h[7], 16);
+                memcpy(&sm.up[1][2][lane], &h[8], 16);
+            }
+        }
+        Quad g[9] = {c0, c1, zero, c3, h4, zero, zero, s7, s8};
+        if (r > y0) {
+            Quad a, e, b = zero;
+            memcpy(&g[2], &sm.up[r & 1][0][lane], 16);
+            memcpy(&g[5], &sm.up[r & 1][1][lane], 16);
+            memcpy(&g[6], &sm.up[r & 1][2][lane], 16);
+            memcpy(&a, &sm.coef[prev][0][lane], 16);
+            memcpy(&e, &sm.coef[prev][1][lane], 16);
+            if (FORCH) memcpy(&b, &sm.coef[prev][FORCH ? 2 : 0][lane], 16);
+            collide4<T, FORCH>(g, a, e, b, c);
+            const long long n0 = (long long)(r - 1) * nx + x0;
+            uint32_t seed = 0;
+            if constexpr (Store<T>::kSmall) seed = mix32(uint32_t(n0) ^ ph.step_key2);
+            for_pops([&](auto i) {
+                T *p = dst + (long long)i.value * geo.plane + n0;
+                if constexpr (Store<T>::kSmall) {
+                    const uint2 w = round4<T, i.value>(g[i.value], c.scale, seed);
+                    if (store) __stcs(reinterpret_cast<uint2 *>(p), w);
+                } else {
+                    uint4 w;
+                    memcpy(&w, &g[i.value], 16);
+                    if (store) __stcs(reinterpret_cast<uint4 *>(p), w);
+                }
+            });
+        }
+        memcpy(&sm.up[r & 1][0][lane], &h2, 16);
+        memcpy(&sm.up[r & 1][1][lane], &s5, 16);
+        memcpy(&sm.up[r & 1][2][lane], &s6, 16);
+        c0 = h0, c1 = s1, c3 = s3;
+        slot = next;
+    }
+}
+
+// One lattice: block w takes strip w % strips of segment w / strips
+// (neighbouring strips run side by side, so their shared columns hit L1 or L2).
+template <typename T, bool WALLS, bool FORCH>
+__global__ void __launch_bounds__(kPairThreads, kPairWarps<T>)
+k_pair(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__ alpha,
+       const float *__restrict__ epsv, const float *__restrict__ betav, Geo geo, Phys<float> ph,
+       const __grid_constant__ Pair2 c, int strips, int rows) {
+    extern __shared__ __align__(16) unsigned char strip_smem[];
+    pdl_enter();
+    if constexpr (Store<T>::kSmall) {
+        if (ph.clock) {
+            const uint32_t t = *ph.clock + ph.step_off;
+            ph.step_key = step_key_of(t, ph.seed);
+            ph.step_key2 = step_key_of(t + 1, ph.seed);
+        }
+    }
+    const int seg = blockIdx.x / strips;
+    const int y0 = seg * rows;
+    const int y1 = y0 + rows < geo.ny ? y0 + rows : geo.ny;
+    march_strip<T, WALLS, FORCH>(*reinterpret_cast<StripSmem<T, FORCH> *>(strip_smem), src, dst, alpha, epsv, betav,
+                                 geo, ph, c, (blockIdx.x - seg * strips) * kStripCols, y0, y1);
 }
 
 // Device step counter of 16-bit storage (see Phys::clock): set to a value
