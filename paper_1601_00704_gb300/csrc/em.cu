@@ -1,15 +1,19 @@
 // EM fit of a one-dimensional Gaussian mixture on the GPU (Sec. 2.2,
 // Eqs. 20-24): the pore-size statistics that the paper splits into organic
 // (OM) and inorganic (IOM) components before the DGM/GMS permeabilities are
-// assigned.  FP64 throughout.  One iteration is two passes over the samples:
-//   pass 1: E-step responsibilities w_j(i) (Eqs. 20-21, exponent with its
-//           minus sign) and the sums behind Phi_j (Eq. 22), mu_j (Eq. 23) and
-//           the log-likelihood;
-//   pass 2: the same responsibilities again and sum_i w_j(i)(x_i - mu_j)^2
-//           with the new mu_j (Eq. 24).
-// Each pass writes fixed per-block partials that one block adds in a fixed
+// assigned.  FP64 throughout.
+//
+// One iteration is one launch (k_em_step): the E-step responsibilities w_j(i)
+// (Eqs. 20-21, exponent with its minus sign) and, in the same pass, the sums
+// of w, w d and w d^2 with d = x - mu_j (the old mean), from which
+//   Phi_j = S0/m,  mu_j += S1/S0,  sigma_j^2 = S2/S0 - (S1/S0)^2   (Eqs. 22-24).
+// The subtraction is harmless while the mean moves by less than a few sigma.
+// Where it would cancel (a component collapsing onto few samples) the launch
+// leaves the estimate alone and asks for the two-pass iteration instead
+// (k_em_pass1/2: sums of w and w x, then of w (x - mu_new)^2).
+// Each launch writes per-block partials that the last block adds in a fixed
 // order, so a fit is bit-for-bit reproducible.
-
+//
 #include "glbm.h"
 
 #include <cuda_runtime.h>
@@ -23,13 +27,32 @@ extern __attribute__((visibility("hidden"))) thread_local char g_create_err[512]
 namespace {
 
 constexpr int KMAX = 8;
-constexpr int EM_THREADS = 256;
+constexpr int EM_THREADS = 256;   // two-pass kernels
+constexpr int STEP_THREADS = 128;  // k_em_step
+
+// Progress of a fit on the device.
+struct EmState {
+    double ll, prev;   // mean log-likelihood of this and the previous E-step
+    int it;            // iterations done
+    int done;          // converged: later launches return at once
+    int cancel;        // the next iteration needs the two passes; likewise
+    unsigned ticket;
+};
 
 struct EmParams {
     int k;
     double phi[KMAX], mu[KMAX], var[KMAX];  // current estimate (E-step uses these)
     double mu_new[KMAX];                    // pass-1 result used by pass 2
+    double amp[KMAX], hiv[KMAX];            // phi / sqrt(2 pi var), -1 / (2 var)
 };
+
+__host__ __device__ inline void em_factor(double phi, double var, double &amp, double &hiv) {
+    amp = phi * (0.39894228040143267794 / sqrt(var));
+    hiv = -0.5 / var;
+}
+__host__ __device__ inline void em_factors(EmParams &p) {
+    for (int j = 0; j < p.k; ++j) em_factor(p.phi[j], p.var[j], p.amp[j], p.hiv[j]);
+}
 
 __device__ __forceinline__ void responsibilities(double x, const EmParams &p, double (&w)[KMAX], double &den) {
     const double inv_sqrt_2pi = 0.39894228040143267794;
@@ -68,6 +91,155 @@ __device__ __forceinline__ void block_sums(double (&v)[CNT], int cnt, double *__
             for (int w = 0; w < EM_THREADS / 32; ++w) s += sh[w][c];
             out[c] = s;
         }
+    }
+}
+
+// Sum of logarithms as a running product: mantissas multiply (relative error
+// 2^-53 each, as small as a log's), exponents add, and one log at the very end
+// replaces one per sample.  Factors that are zero, subnormal, infinite or NaN
+// go through log().
+__device__ __forceinline__ double split_exponent(double f, long long &exps) {  // f normal, positive
+    const long long b = __double_as_longlong(f);
+    exps += (b >> 52) - 1023;
+    return __longlong_as_double((b & 0x000fffffffffffffll) | 0x3ff0000000000000ll);  // in [1, 2)
+}
+struct LogSum {
+    double prod = 1.0, rest = 0.0;
+    long long exps = 0;
+    int n = 0;
+    __device__ __forceinline__ void add(double f) {
+        const int e = int(__double_as_longlong(f) >> 52);  // sign and exponent: 1 .. 2046 for normal positive
+        if (e < 1 || e > 2046) {
+            rest += log(f);
+            return;
+        }
+        prod *= split_exponent(f, exps);
+        if (++n == 1000) prod = split_exponent(prod, exps), n = 0;  // stays below 2^1001
+    }
+};
+
+// One EM iteration.  Bound by FP64 issue (GB300 has two FP64 lanes per SM):
+// about 45 operations per sample and component for the exponential, the
+// shared reciprocal and the three sums, so everything that is not per sample
+// is kept off it: the component factors are formed once per iteration by the
+// last block, logarithms are one product, and block sums go through shared
+// memory (8 FP64 instructions per sum and block of 4 warps instead of 20 by
+// shuffles).  4 blocks per SM.  10^6 samples, 2 components, us an iteration:
+// two passes with a one-thread sum of the block partials 1154, this form with
+// a log per thread and shuffled block sums 190, as written 131.
+// part: 3K sums, product, rest (doubles) and exponents, [3K + 3][blocks].
+template <int K>
+__global__ void __launch_bounds__(STEP_THREADS)
+k_em_step(const double *__restrict__ x, long long m, EmParams *__restrict__ pp, EmState *__restrict__ st, double tol,
+          double *__restrict__ part) {
+    if (st->done || st->cancel) return;
+    constexpr int W = 3 * K + 3, PROD = 3 * K, REST = 3 * K + 1, EXPS = 3 * K + 2, NW = STEP_THREADS / 32;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int nb = gridDim.x;
+    double mu[K], amp[K], hiv[K], v[3 * K];
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+        mu[j] = pp->mu[j];
+        amp[j] = pp->amp[j];
+        hiv[j] = pp->hiv[j];
+        v[j] = v[K + j] = v[2 * K + j] = 0.0;
+    }
+    LogSum ls;
+    for (long long i = blockIdx.x * (long long)STEP_THREADS + threadIdx.x; i < m; i += (long long)nb * STEP_THREADS) {
+        const double xi = x[i];
+        double d[K], w[K], den = 0.0;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            d[j] = xi - mu[j];
+            w[j] = amp[j] * exp(hiv[j] * (d[j] * d[j]));
+            den += w[j];
+        }
+        const double inv = 1.0 / den;
+#pragma unroll
+        for (int j = 0; j < K; ++j) {
+            const double r = w[j] * inv, rd = r * d[j];
+            v[j] += r;
+            v[K + j] += rd;
+            v[2 * K + j] += rd * d[j];
+        }
+        ls.add(den);
+    }
+    // sums of the block, then of all blocks by the last one, in fixed order
+    __shared__ double sh[W][STEP_THREADS];
+    __shared__ bool last;
+#pragma unroll
+    for (int c = 0; c < 3 * K; ++c) sh[c][threadIdx.x] = v[c];
+    sh[PROD][threadIdx.x] = split_exponent(ls.prod, ls.exps);
+    sh[REST][threadIdx.x] = ls.rest;
+    sh[EXPS][threadIdx.x] = __longlong_as_double(ls.exps);
+    __syncthreads();
+    // column c of n values: sum, product or integer sum, in lane 0
+    auto column = [&](int c, auto value, int n) {
+        if (c == EXPS) {
+            long long t = 0;
+            for (int q = lane; q < n; q += 32) t += __double_as_longlong(value(q));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+            return __longlong_as_double(t);
+        }
+        double t = c == PROD ? 1.0 : 0.0;
+        for (int q = lane; q < n; q += 32) t = c == PROD ? t * value(q) : t + value(q);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double u = __shfl_down_sync(0xffffffffu, t, o);
+            t = c == PROD ? t * u : t + u;
+        }
+        return t;
+    };
+    for (int c = warp; c < W; c += NW) {
+        const double t = column(c, [&](int q) { return sh[c][q]; }, STEP_THREADS);  // product: 128 factors below 2
+        if (lane == 0) {
+            __stcg(part + (long long)c * nb + blockIdx.x, t);
+            __threadfence();
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&st->ticket, 1u) == unsigned(nb) - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    long long moved = 0;  // exponents taken off the blocks' products (then 2^nb bounds theirs, nb <= 608)
+    for (int c = warp; c < W; c += NW) {
+        const double *p = part + (long long)c * nb;
+        const double t = column(
+            c, [&](int q) { return c == PROD ? split_exponent(__ldcg(p + q), moved) : __ldcg(p + q); }, nb);
+        if (lane == 0) sh[0][c] = t;
+        if (c == PROD) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) moved += __shfl_down_sync(0xffffffffu, moved, o);
+            if (lane == 0) sh[0][W] = __longlong_as_double(moved);
+        }
+    }
+    __syncthreads();
+    if (warp != 0) return;
+    // lane j finishes component j, lane K the log-likelihood
+    const double *tot = sh[0];
+    const int j = lane < K ? lane : 0;
+    const double s0 = tot[j], shift = tot[K + j] / s0, second = tot[2 * K + j] / s0;
+    const bool cancel = __any_sync(0xffffffffu, second - shift * shift < second * (1.0 / 64.0));
+    if (lane == 0) {
+        st->ticket = 0u;
+        if (cancel) st->cancel = 1;
+    }
+    if (cancel) return;
+    if (lane < K) {
+        const double phi = s0 / double(m), var = second - shift * shift;
+        pp->phi[j] = phi;
+        pp->mu[j] += shift;
+        pp->var[j] = var;
+        em_factor(phi, var, pp->amp[j], pp->hiv[j]);
+    } else if (lane == K) {
+        const long long exps = __double_as_longlong(tot[EXPS]) + __double_as_longlong(tot[W]);
+        const double ll = (tot[REST] + (log(tot[PROD]) + double(exps) * 0.693147180559945309417)) / double(m);
+        st->it++;
+        st->ll = ll;
+        if (tol > 0.0 && fabs(ll - st->prev) < tol) st->done = 1;
+        st->prev = ll;
     }
 }
 
@@ -116,35 +288,50 @@ k_em_pass2(const double *__restrict__ x, long long m, const EmParams *__restrict
     block_sums<KMAX>(v, KMAX, part + (long long)blockIdx.x * KMAX);
 }
 
-// Fixed-order totals of the block partials; pass 1 sets phi, mu_new and the
-// log-likelihood, pass 2 the variances and moves mu_new into mu.
-__global__ void k_em_finalize(const double *__restrict__ part, int nblocks, long long m, int pass,
-                              EmParams *__restrict__ pp, double *__restrict__ sw_keep, double *__restrict__ ll) {
+// Fixed-order totals of the block partials, one warp per sum; pass 1 sets
+// mu_new and the log-likelihood, pass 2 phi and the variances, moves mu_new
+// into mu and ends the iteration.
+__global__ void __launch_bounds__(EM_THREADS)
+k_em_finalize(const double *__restrict__ part, int nblocks, long long m, int pass, double tol,
+              EmParams *__restrict__ pp, EmState *__restrict__ st, double *__restrict__ sw_keep) {
+    __shared__ double tot[2 * KMAX + 1];
+    const int W = pass == 1 ? 2 * KMAX + 1 : KMAX;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int c = warp; c < W; c += EM_THREADS / 32) {
+        double s = 0.0;
+        for (int b = lane; b < nblocks; b += 32) s += part[(long long)b * W + c];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) tot[c] = s;
+    }
+    __syncthreads();
     if (threadIdx.x != 0) return;
     EmParams &p = *pp;
     if (pass == 1) {
-        const int W = 2 * KMAX + 1;
         for (int j = 0; j < p.k; ++j) {
-            double sw = 0.0, swx = 0.0;
-            for (int b = 0; b < nblocks; ++b) {
-                sw += part[(long long)b * W + j];
-                swx += part[(long long)b * W + KMAX + j];
-            }
-            sw_keep[j] = sw;
-            p.mu_new[j] = swx / sw;
+            sw_keep[j] = tot[j];
+            p.mu_new[j] = tot[KMAX + j] / tot[j];
         }
-        double s = 0.0;
-        for (int b = 0; b < nblocks; ++b) s += part[(long long)b * W + 2 * KMAX];
-        *ll = s / double(m);
+        st->ll = tot[2 * KMAX] / double(m);
     } else {
         for (int j = 0; j < p.k; ++j) {
-            double sd = 0.0;
-            for (int b = 0; b < nblocks; ++b) sd += part[(long long)b * KMAX + j];
             p.phi[j] = sw_keep[j] / double(m);
             p.mu[j] = p.mu_new[j];
-            p.var[j] = sd / sw_keep[j];
+            p.var[j] = tot[j] / sw_keep[j];
         }
+        em_factors(p);
+        st->it++;
+        st->cancel = 0;
+        if (tol > 0.0 && fabs(st->ll - st->prev) < tol) st->done = 1;
+        st->prev = st->ll;
     }
+}
+
+template <int K>
+void launch_em_step(int k, int nb, cudaStream_t s, const double *x, long long m, EmParams *pp, EmState *st, double tol,
+                    double *part) {
+    if (k == K) k_em_step<K><<<nb, STEP_THREADS, 0, s>>>(x, m, pp, st, tol, part);
+    else if constexpr (K < KMAX) launch_em_step<K + 1>(k, nb, s, x, m, pp, st, tol, part);
 }
 
 glbm_status emfail(glbm_status s, const char *fmt, const char *detail) {
@@ -174,43 +361,51 @@ extern "C" glbm_status glbm_em_gmm1d(const double *x, long long m, int k, double
     for (int j = 0; j < k; ++j) hp.phi[j] /= fsum;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nb = int(std::min<long long>((m + EM_THREADS - 1) / EM_THREADS, 152LL * 8));
-    double *dx = nullptr, *part = nullptr, *sw = nullptr, *dll = nullptr;
-    EmParams *dp = nullptr;
+    const int nbs = int(std::min<long long>((m + STEP_THREADS - 1) / STEP_THREADS, 152LL * 4));
+    // one workspace: estimate, progress, Phi sums, block partials of either form
+    const size_t parts = std::max(size_t(nbs) * (3 * k + 3), size_t(nb) * (2 * KMAX + 1));
+    em_factors(hp);
+    struct Head {
+        EmParams p;
+        EmState s;
+        double sw[KMAX];
+    };
+    EmState hs{};
+    hs.ll = hs.prev = -INFINITY;
+    Head head{hp, hs, {}};
+    double *dx = nullptr;
+    Head *dh = nullptr;
     cudaError_t e = cudaSuccess;
     if (!device_ptrs) {
         e = cudaMalloc(&dx, sizeof(double) * m);
         if (e == cudaSuccess) e = cudaMemcpyAsync(dx, x, sizeof(double) * m, cudaMemcpyHostToDevice, st);
     }
-    if (e == cudaSuccess) e = cudaMalloc(&part, sizeof(double) * nb * (2 * KMAX + 1));
-    if (e == cudaSuccess) e = cudaMalloc(&sw, sizeof(double) * KMAX);
-    if (e == cudaSuccess) e = cudaMalloc(&dll, sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&dp, sizeof(EmParams));
-    if (e == cudaSuccess) e = cudaMemcpyAsync(dp, &hp, sizeof(EmParams), cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = cudaMalloc(&dh, sizeof(Head) + sizeof(double) * parts);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(dh, &head, sizeof(Head), cudaMemcpyHostToDevice, st);
+    double *part = reinterpret_cast<double *>(dh + 1);
     const double *xs = device_ptrs ? x : dx;
-    double prev = -INFINITY, ll = -INFINITY;
-    int it = 0;
-    for (; e == cudaSuccess && it < max_iter; ++it) {
-        k_em_pass1<<<nb, EM_THREADS, 0, st>>>(xs, m, dp, part);
-        k_em_finalize<<<1, 32, 0, st>>>(part, nb, m, 1, dp, sw, dll);
-        k_em_pass2<<<nb, EM_THREADS, 0, st>>>(xs, m, dp, part);
-        k_em_finalize<<<1, 32, 0, st>>>(part, nb, m, 2, dp, sw, dll);
-        e = cudaGetLastError();
-        if (e == cudaSuccess && tol > 0.0) {
-            e = cudaMemcpyAsync(&ll, dll, sizeof(double), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-            if (e == cudaSuccess && std::fabs(ll - prev) < tol) {
-                ++it;
-                break;
-            }
-            prev = ll;
+    // Iterations are enqueued in batches; the launches after one that
+    // converged, or that asks for the two-pass form, return at once.
+    int batch = tol > 0.0 ? 2 : max_iter;
+    while (e == cudaSuccess && hs.it < max_iter && !hs.done) {
+        const int n = std::min(batch, max_iter - hs.it);
+        if (hs.cancel) {
+            k_em_pass1<<<nb, EM_THREADS, 0, st>>>(xs, m, &dh->p, part);
+            k_em_finalize<<<1, EM_THREADS, 0, st>>>(part, nb, m, 1, tol, &dh->p, &dh->s, dh->sw);
+            k_em_pass2<<<nb, EM_THREADS, 0, st>>>(xs, m, &dh->p, part);
+            k_em_finalize<<<1, EM_THREADS, 0, st>>>(part, nb, m, 2, tol, &dh->p, &dh->s, dh->sw);
+        } else {
+            for (int i = 0; i < n; ++i) launch_em_step<1>(k, nbs, st, xs, m, &dh->p, &dh->s, tol, part);
+            batch = std::min(2 * batch, 16);
         }
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, &dh->s, sizeof(EmState), cudaMemcpyDeviceToHost, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&hp, dp, sizeof(EmParams), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&ll, dll, sizeof(double), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&hp, &dh->p, sizeof(EmParams), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    void *ptrs[] = {dx, part, sw, dll, dp};
-    for (void *p : ptrs)
-        if (p) cudaFree(p);
+    if (dx) cudaFree(dx);
+    if (dh) cudaFree(dh);
     if (e != cudaSuccess) return emfail(GLBM_ECUDA, "em_gmm1d: %s", cudaGetErrorString(e));
     bool finite = true;
     for (int j = 0; j < k; ++j) {
@@ -219,8 +414,8 @@ extern "C" glbm_status glbm_em_gmm1d(const double *x, long long m, int k, double
         var[j] = hp.var[j];
         finite = finite && std::isfinite(phi[j]) && std::isfinite(mu[j]) && std::isfinite(var[j]);
     }
-    if (iters) *iters = it;
-    if (loglik) *loglik = max_iter > 0 ? ll : NAN;
+    if (iters) *iters = hs.it;
+    if (loglik) *loglik = max_iter > 0 ? hs.ll : NAN;
     // a component that collapses onto a single sample has zero variance and
     // the next E-step is undefined
     if (!finite) return emfail(GLBM_ENAN, "em_gmm1d: %s", "estimate not finite (a component collapsed)");
