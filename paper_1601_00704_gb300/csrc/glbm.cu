@@ -83,6 +83,7 @@ struct glbm {
     // non-legacy stream): key = (buffer parity at start, steps, reduce at
     // end, test, tol, FP16 scale)
     int nsm = 0;              // SMs of the device
+    TilePlan tile{};          // multi-step tiles of small or odd lattices
     struct Graph {
         int parity, end_parity;
         long long launches, chunk;
@@ -140,12 +141,69 @@ Phys<R> make_phys(const glbm *h) {
     p.inv_scale = R(1.0 / h->scale);
     p.step_key = step_key_of(uint32_t(h->tstep), h->seed);
     p.step_key2 = step_key_of(uint32_t(h->tstep + 1), h->seed);
+    p.tstep = uint32_t(h->tstep);
     p.sr = h->sr ? 1 : 0;
     p.seed = h->seed;
     return p;
 }
 
 bool injected_failure() { return glbm_injected_failure(); }
+
+// Tile shape for k_tile: the one with the fewest microseconds a step, if that
+// beats the one-step kernel.  A launch takes
+//     A + rounds (blocks in turn on an SM) x T (B + C x warps per scheduler),
+// fitted to 900 launches over lattices of 64^2 to 768^2, tiles of 32 and 64
+// columns and T = 2 .. 12 (median error 5 %): A = 1.85 us launch, loads and
+// stores, B = 0.28 us the latency of a step, C = 0.37 us its issue.  The
+// one-step kernel takes max(1.7, 1.3 + 7e-6 N) us from a graph; on the legacy
+// stream, where nothing is captured, no launch takes less than about 5 us.
+//   FP32, us a step before / after: 128^2 1.74 / 0.97 (T = 8), 256^2 2.22 / 1.33
+//   (T = 4), 512 x 384 2.96 / 2.17, 640^2 5.16 / 3.99, 768^2 5.78 / 5.4;
+//   BF16: 128^2 1.85 / 1.02, 512 x 384 2.57 / 2.18.
+// Above kTileNodes a wave of blocks no longer covers the lattice and the halo
+// is pure loss: 1024^2 8.4 / 8.8.  Odd row lengths keep gaining in FP32, whose
+// one-step kernel loads one node per thread (2221 x 2000: 57.7 / 44.9, best with
+// two blocks per SM that overlap loads and steps); in 16-bit storage rounding
+// node by node dominates and large lattices stay on it (61.4 / 61.9).
+TilePlan plan_tiles(const glbm *h) {
+    constexpr long long kTileNodes = 600000;
+    TilePlan best{};
+    const bool small = h->elem == 2, odd = h->nx % 4 != 0;
+    if (h->storage == GLBM_F64 || (small && !h->sr)) return best;
+    auto shape = [&](int T, int q, int R) {
+        TilePlan p;
+        p.steps = T;
+        p.q_log2 = q;
+        p.rows = R;
+        p.hx = (T + 3) / 4 * 4;
+        p.hy = T - 1;
+        const int w = (4 << q) - 2 * p.hx, l = R - 2 * p.hy;
+        p.nx_tiles = (h->nx + w - 1) / w;
+        p.ny_tiles = (h->ny + l - 1) / l;
+        return p;
+    };
+    if (h->N > kTileNodes) return odd && !small ? shape(4, 4, 20) : best;
+    const double A = small ? 1.71 : 1.85, B = small ? 0.31 : 0.28, C = small ? 0.405 : 0.37;
+    const double launch = h->stream ? 0.0 : 5.0;
+    double least = std::max(launch, std::max(1.7, small ? 1.2 + 7.4e-6 * double(h->N) : 1.3 + 7e-6 * double(h->N)));
+    for (int T : {2, 3, 4, 6, 8})
+        for (int q : {3, 4}) {
+            const int Q = 1 << q;
+            for (int R = 2 * (T - 1) + 1; R * Q <= kTileThreads; ++R) {
+                if (R * Q % 32) continue;
+                const TilePlan p = shape(T, q, R);
+                const int fit = std::min(65536 / (96 * R * Q), 227 * 1024 / (192 * (R + 2) * Q + 1024));
+                const long long tiles = (long long)p.nx_tiles * p.ny_tiles;
+                const long long per_sm = (tiles + h->nsm - 1) / h->nsm, side = std::min<long long>(per_sm, std::max(1, fit));
+                const long long rounds = (per_sm + side - 1) / side;
+                // rows of the halo drop out as their reach shrinks
+                const double warps = double(side) * R * Q / 128.0 * (R - (T - 1)) / R;
+                const double t = std::max(launch, A + double(rounds) * T * (B + C * warps)) / T;
+                if (t < least) least = t, best = p;
+            }
+        }
+    return best;
+}
 
 int grid_1d(long long N) {
     long long b = (N + 255) / 256;
@@ -260,15 +318,71 @@ glbm_status do_pair(glbm *h, long long clock_off = -1) {
     }
 }
 
+// Several steps of every tile in one launch (k_tile), `n` <= plan.steps.
+template <typename T, bool WALLS, bool FORCH, bool ODD>
+glbm_status launch_tile_t(glbm *h, int n, long long clock_off) {
+    const TilePlan &pl = h->tile;
+    const Geo geo = make_geo(h, 4);
+    Phys<float> ph = make_phys<float>(h);
+    if (Store<T>::kSmall && clock_off >= 0) {
+        ph.clock = h->dclock;
+        ph.step_off = uint32_t(clock_off);
+    }
+    bool refused = false;
+    for (int i = 0; i < n; ++i) refused = injected_failure() || refused;  // the test hook counts time steps
+    if (refused) return fail(h, GLBM_ECUDA, "step launch: injected failure (test hook)");
+    const int Q = 1 << pl.q_log2;
+    const size_t smem = sizeof(float4) * 2 * 6 * (pl.rows + 2) * Q;
+    cudaError_t err = cudaSuccess;
+    if (smem > 48 * 1024)
+        err = cudaFuncSetAttribute(k_tile<T, WALLS, FORCH, ODD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   int(smem));
+    if (err == cudaSuccess)
+        err = launch_kernel_smem(
+            k_tile<T, WALLS, FORCH, ODD>, dim3(unsigned(pl.nx_tiles) * unsigned(pl.ny_tiles)),
+            dim3(unsigned(Q * pl.rows)), smem, h->stream, h->stream != nullptr,
+            static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
+            static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
+            static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), pl, n);
+    if (err != cudaSuccess) return fail(h, GLBM_ECUDA, "step launch: %s", cudaGetErrorString(err));
+    h->launches++;
+    h->tstep += n;
+    h->cur ^= 1;
+    return GLBM_OK;
+}
+
+template <typename T, bool ODD>
+glbm_status launch_tile(glbm *h, int n, long long co) {
+    if (!(h->flags & GLBM_PERIODIC_Y))
+        return h->forch ? launch_tile_t<T, true, true, ODD>(h, n, co) : launch_tile_t<T, true, false, ODD>(h, n, co);
+    return h->forch ? launch_tile_t<T, false, true, ODD>(h, n, co) : launch_tile_t<T, false, false, ODD>(h, n, co);
+}
+
+glbm_status do_tile(glbm *h, int n, long long co) {
+    const bool odd = h->nx % 4 != 0;
+    switch (h->storage) {
+        case GLBM_F16DEV: return odd ? launch_tile<__half, true>(h, n, co) : launch_tile<__half, false>(h, n, co);
+        case GLBM_BF16DEV:
+            return odd ? launch_tile<__nv_bfloat16, true>(h, n, co) : launch_tile<__nv_bfloat16, false>(h, n, co);
+        default: return odd ? launch_tile<float, true>(h, n, co) : launch_tile<float, false>(h, n, co);
+    }
+}
+
 // `chunk` steps, the last one reducing when `reduce`.  That one is a launch of
 // its own: the velocity export reads the state before it.
 glbm_status do_steps(glbm *h, long long chunk, bool reduce, bool clocked) {
-    const long long pairs_to = pair_eligible(h) ? chunk - (reduce ? 1 : 0) : 0;
+    const long long plain = chunk - (reduce ? 1 : 0);
+    const bool pairs = pair_eligible(h);
     for (long long s = 0; s < chunk;) {
-        const bool pair = s + 2 <= pairs_to;
         const long long co = clocked ? s : -1;
-        if (glbm_status st = pair ? do_pair(h, co) : do_step(h, reduce && s == chunk - 1, co)) return st;
-        s += pair ? 2 : 1;
+        const int n = pairs ? 2 : int(std::min<long long>(h->tile.steps, plain - s));
+        glbm_status st;
+        int done = n;
+        if (pairs && s + 2 <= plain) st = do_pair(h, co);
+        else if (!pairs && n >= 2) st = do_tile(h, n, co);
+        else st = do_step(h, reduce && s == chunk - 1, co), done = 1;
+        if (st) return st;
+        s += done;
     }
     return GLBM_OK;
 }
@@ -554,6 +668,7 @@ glbm_status glbm_create(int nx, int ny, double tau, glbm_storage storage, unsign
     h->sr = !(flags & GLBM_NEAREST16);
     cudaError_t e = cudaGetDevice(&h->dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
+    if (e == cudaSuccess) h->tile = plan_tiles(h);
     const size_t fbytes = size_t(9) * h->plane * h->elem;
     const size_t cbytes = size_t(h->plane) * h->celem;
     // the scalar grid has the most blocks

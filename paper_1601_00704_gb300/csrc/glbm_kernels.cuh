@@ -196,6 +196,7 @@ struct Phys {
     uint32_t step_off = 0;
     uint32_t seed = 0;
     uint32_t step_key2 = 0;  // key of the following step, for k_pair
+    uint32_t tstep = 0;      // the step itself, for kernels that form several keys
 };
 
 // Stochastic-rounding key of time step t (host and device agree).
@@ -300,13 +301,14 @@ __device__ __forceinline__ void node_velocity(const R (&g)[9], R alpha, R eps, R
 // carrier w_i (rho - 1), several decades above the velocity terms.  The update
 // is therefore regrouped as
 //     g* = w d + [ (1 - 1/tau)(g - w d) + w (even +- odd) ],   d = rho - 1,
-// where the bracket holds only small terms (g - w d is exact when g ~ w d),
-// so the carrier is rounded twice per population instead of at every term.
+// where the bracket holds only small terms and w d enters by fused
+// multiply-add, so the carrier is rounded once per population instead of at
+// every term.
 //
 // Operation count: with H = 1.5 u/tau + 3A F, J = 3 u/tau + 3A F and
 // A = 1 - 1/(2 tau) the direction sums of Eqs. 30 and 31 collapse to
 //     even = (3 rho/eps) [ (e.u)(e.H) - (u.H)/3 ],   odd = rho (e.J),
-// shared by opposite directions: 108 FP32 operations per node with the mass
+// shared by opposite directions: 106 FP32 operations per node with the mass
 // closure below.  The form before it (separate f_eq and F_i terms, and TwoSum
 // sums of the populations before and after the collision) took 241 and was
 // bound by them where the lattice fits L2: 1024^2 FP32 10.8 -> 8.8 us a step.
@@ -315,10 +317,10 @@ __device__ __forceinline__ void node_velocity(const R (&g)[9], R alpha, R eps, R
 // with 1/6 in the weight the velocity error against FP64 was 5 % larger, as
 // written it is 1 % smaller than the separate terms' (192^2, 200 steps).
 template <typename R>
-__device__ __forceinline__ R collide_pair(R &gi, R &gj, R wd, R k1, R eu, R eH, R eJ, R q, R we, R wo) {
+__device__ __forceinline__ R collide_pair(R &gi, R &gj, R w, R d, R k1, R eu, R eH, R eJ, R q, R we, R wo) {
     const R ev = rmul(we, rfma(eu, eH, -q));
-    const R ni = radd(wd, rfma(k1, rsub(gi, wd), rfma(wo, eJ, ev)));
-    const R nj = radd(wd, rfma(k1, rsub(gj, wd), rfma(-wo, eJ, ev)));
+    const R ni = rfma(w, d, rfma(k1, rfma(-w, d, gi), rfma(wo, eJ, ev)));
+    const R nj = rfma(w, d, rfma(k1, rfma(-w, d, gj), rfma(-wo, eJ, ev)));
     const R lost = radd(rsub(gi, ni), rsub(gj, nj));  // what this pair hands to the rest population
     gi = ni;
     gj = nj;
@@ -343,7 +345,7 @@ __device__ __forceinline__ void collide(R (&g)[9], R alpha, R eps, R beta,
     // weights of the axis class (w = 1/9) and the diagonal class (1/36)
     const R we1 = rmul(R(1.0 / 3.0), rmul(rrcp(eps), rho)), we2 = rmul(R(0.25), we1);
     const R wo1 = rmul(wgt<R>(1), rho), wo2 = rmul(R(0.25), wo1);
-    const R wd1 = rmul(wgt<R>(1), drho), wd2 = rmul(R(0.25), wd1);
+    const R w1 = wgt<R>(1), w2 = R(0.25) * wgt<R>(1);
     // Mass closure: the collision conserves each node's mass exactly in
     // arithmetic, but rounding the nine stored populations does not, and the
     // slow pressure mode integrates that per-node error over thousands of
@@ -354,10 +356,10 @@ __device__ __forceinline__ void collide(R (&g)[9], R alpha, R eps, R beta,
     // against FP64 over 10 000 steps (128^2; Darcy, clear and mixed media) the
     // velocity and density errors equal those of TwoSum sums, 30x below the
     // unclosed update's.
-    const R l1 = collide_pair<R>(g[1], g[3], wd1, k1, ux, Hx, Jx, q, we1, wo1);
-    const R l2 = collide_pair<R>(g[2], g[4], wd1, k1, uy, Hy, Jy, q, we1, wo1);
-    const R l5 = collide_pair<R>(g[5], g[7], wd2, k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), q, we2, wo2);
-    const R l6 = collide_pair<R>(g[6], g[8], wd2, k1, rsub(uy, ux), rsub(Hy, Hx), rsub(Jy, Jx), q, we2, wo2);
+    const R l1 = collide_pair<R>(g[1], g[3], w1, drho, k1, ux, Hx, Jx, q, we1, wo1);
+    const R l2 = collide_pair<R>(g[2], g[4], w1, drho, k1, uy, Hy, Jy, q, we1, wo1);
+    const R l5 = collide_pair<R>(g[5], g[7], w2, drho, k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), q, we2, wo2);
+    const R l6 = collide_pair<R>(g[6], g[8], w2, drho, k1, rsub(uy, ux), rsub(Hy, Hx), rsub(Jy, Jx), q, we2, wo2);
     g[0] = radd(g[0], radd(radd(l1, l2), radd(l5, l6)));
 }
 
@@ -459,7 +461,7 @@ __device__ __forceinline__ f2 rsqrt_(f2 a) { return mk2(rsqrt_(lo2(a)), rsqrt_(h
 // constant bank.
 struct Pair2 {
     f2 one, half, quarter, hgx, hgy, ngx, ngy, k1;
-    f2 omH, omJ, nA3, nthird, third, w1, nw1;            // 32-bit storage
+    f2 omH, omJ, nA3, nthird, third, w1, nw1, w2, nw2;   // 32-bit storage
     f2 cA, cO, ncO, w1om, four, cO3, ncA3, cO2, ncA;     // 16-bit storage
     f2 scale, inv_s;
 };
@@ -471,6 +473,7 @@ inline Pair2 make_pair2(const Phys<float> &p) {
     c.k1 = bc2(1.0f - om);
     c.omH = bc2(1.5f * om), c.omJ = bc2(3.0f * om), c.nA3 = bc2(-(3.0f * p.A));
     c.nthird = bc2(-(1.0f / 3.0f)), c.third = bc2(1.0f / 3.0f), c.w1 = bc2(w1), c.nw1 = bc2(-w1);
+    c.w2 = bc2(0.25f * w1), c.nw2 = bc2(-0.25f * w1);
     c.cA = bc2(cA), c.ncA = bc2(-cA), c.cO = bc2(cO), c.ncO = bc2(-cO), c.w1om = bc2(w1 * om), c.four = bc2(4.0f);
     c.cO3 = bc2(3.0f * cO), c.ncA3 = bc2(-(3.0f * cA)), c.cO2 = bc2(2.0f * cO);
     c.scale = bc2(p.scale), c.inv_s = bc2(p.inv_scale);
@@ -501,11 +504,11 @@ __device__ __forceinline__ void node_velocity2(const f2 (&g)[9], f2 alpha, f2 ep
     uy = rmul(vy, iden);
 }
 
-__device__ __forceinline__ f2 collide_pair2(f2 &gi, f2 &gj, f2 wd, f2 k1, f2 eu, f2 eH, f2 eJ, f2 nq, f2 we, f2 wo,
-                                            f2 nwo) {
+__device__ __forceinline__ f2 collide_pair2(f2 &gi, f2 &gj, f2 w, f2 nw, f2 d, f2 k1, f2 eu, f2 eH, f2 eJ, f2 nq,
+                                            f2 we, f2 wo, f2 nwo) {
     const f2 ev = rmul(we, rfma(eu, eH, nq));
-    const f2 ni = radd(wd, rfma(k1, rsub(gi, wd), rfma(wo, eJ, ev)));
-    const f2 nj = radd(wd, rfma(k1, rsub(gj, wd), rfma(nwo, eJ, ev)));
+    const f2 ni = rfma(w, d, rfma(k1, rfma(nw, d, gi), rfma(wo, eJ, ev)));
+    const f2 nj = rfma(w, d, rfma(k1, rfma(nw, d, gj), rfma(nwo, eJ, ev)));
     const f2 lost = radd(rsub(gi, ni), rsub(gj, nj));
     gi = ni;
     gj = nj;
@@ -527,11 +530,12 @@ __device__ __forceinline__ void collide2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, 
     const f2 we1 = rmul(c.third, rmul(rrcp(eps), rho)), we2 = rmul(c.quarter, we1);
     const f2 wo1 = rmul(c.w1, rho), wo2 = rmul(c.quarter, wo1);
     const f2 nwo1 = rmul(c.nw1, rho), nwo2 = rmul(c.quarter, nwo1);
-    const f2 wd1 = rmul(c.w1, drho), wd2 = rmul(c.quarter, wd1);
-    const f2 l1 = collide_pair2(g[1], g[3], wd1, c.k1, ux, Hx, Jx, nq, we1, wo1, nwo1);
-    const f2 l2 = collide_pair2(g[2], g[4], wd1, c.k1, uy, Hy, Jy, nq, we1, wo1, nwo1);
-    const f2 l5 = collide_pair2(g[5], g[7], wd2, c.k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), nq, we2, wo2, nwo2);
-    const f2 l6 = collide_pair2(g[6], g[8], wd2, c.k1, rsub(uy, ux), rsub(Hy, Hx), rsub(Jy, Jx), nq, we2, wo2, nwo2);
+    const f2 l1 = collide_pair2(g[1], g[3], c.w1, c.nw1, drho, c.k1, ux, Hx, Jx, nq, we1, wo1, nwo1);
+    const f2 l2 = collide_pair2(g[2], g[4], c.w1, c.nw1, drho, c.k1, uy, Hy, Jy, nq, we1, wo1, nwo1);
+    const f2 l5 = collide_pair2(g[5], g[7], c.w2, c.nw2, drho, c.k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), nq, we2,
+                                wo2, nwo2);
+    const f2 l6 = collide_pair2(g[6], g[8], c.w2, c.nw2, drho, c.k1, rsub(uy, ux), rsub(Hy, Hx), rsub(Jy, Jx), nq, we2,
+                                wo2, nwo2);
     g[0] = radd(g[0], radd(radd(l1, l2), radd(l5, l6)));
 }
 
@@ -1195,6 +1199,222 @@ k_pair(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__
     const int y1 = y0 + rows < geo.ny ? y0 + rows : geo.ny;
     march_strip<T, WALLS, FORCH>(*reinterpret_cast<StripSmem<T, FORCH> *>(strip_smem), src, dst, alpha, epsv, betav,
                                  geo, ph, c, (blockIdx.x - seg * strips) * kStripCols, y0, y1);
+}
+
+// ---------------------------------------------------------------------------
+// K2c: several time steps of a tile per launch, for lattices that one wave of
+// blocks covers and for row lengths that are not a multiple of the vector.
+//
+// Small lattices are bound by the latency of a launch (a 128^2 step is 0.2 us
+// of arithmetic in a 2 us launch), odd row lengths by scalar loads.  A block
+// loads a tile with a halo, advances it `nsteps` steps and stores the inside.
+// A thread keeps 4 nodes of a row: rest and level populations stay in its
+// registers (x neighbours by shuffle among the Q lanes of the row), the six
+// that move in y go through shared memory, two buffers, one barrier per step.
+// The first step gathers from memory itself, so rows need a halo of
+// nsteps - 1; columns lose one per step, rounded up to 4.  Values beyond the
+// halo's reach are computed from stale neighbours and never stored.  Wall
+// rows write what the wall returns into the shared row beyond it.
+// Columns of an odd-length row are fetched one by one, each wrapped around
+// the period; everything after that is the same.
+// Rounding and stochastic-rounding words are the one-step kernel's (per lane
+// of 4 for whole vectors, per node otherwise), so the results are its bits.
+// ---------------------------------------------------------------------------
+constexpr int kTileThreads = 640;  // most per block: 96 registers a thread
+
+struct TilePlan {
+    int steps;     // T: most steps per launch; 0: not used
+    int q_log2;    // lanes per row, Q = 1 << q_log2
+    int rows;      // rows per block with halo
+    int hx, hy;    // halo
+    int nx_tiles, ny_tiles;
+};
+
+// Stored 16-bit form of one node as the one-step kernel with one node per
+// thread rounds it.
+template <typename T, int I>
+__device__ __forceinline__ T round1(float v, float scale, uint32_t hash) {
+    uint32_t r = (hash ^ (uint32_t(I >> 1) * 0x9E3779B9u)) * 0x2C1B3C6Du;
+    r ^= r >> 15;
+    return Store<T>::st_sr(v, scale, (I & 1) ? (r >> 16) : r);
+}
+
+template <typename T, bool WALLS, bool FORCH, bool ODD>
+__global__ void __launch_bounds__(kTileThreads, 1)
+k_tile(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__ alpha,
+       const float *__restrict__ epsv, const float *__restrict__ betav, Geo geo, Phys<float> ph,
+       const __grid_constant__ Pair2 c, TilePlan pl, int nsteps) {
+    extern __shared__ __align__(16) float4 tile_smem[];
+    const int Q = 1 << pl.q_log2, R = pl.rows;
+    const int qx = threadIdx.x & (Q - 1), ly = threadIdx.x >> pl.q_log2;
+    const int ty = blockIdx.x / pl.nx_tiles, tx = blockIdx.x - ty * pl.nx_tiles;
+    const int nx = geo.nx, ny = geo.ny;
+    const int gx = tx * (4 * Q - 2 * pl.hx) - pl.hx + 4 * qx;  // unwrapped
+    const int gy = ty * (R - 2 * pl.hy) - pl.hy + ly;
+    const bool inside = !WALLS || (gy >= 0 && gy < ny);
+    int row = gy;  // wrapped; rows outside a walled lattice compute row 0 to no effect
+    if (WALLS) row = inside ? gy : 0;
+    else {
+        row %= ny;
+        row = row < 0 ? row + ny : row;
+    }
+    int col[ODD ? 4 : 1];  // this lane's columns, wrapped (whole vectors: the first)
+#pragma unroll
+    for (int k = 0; k < (ODD ? 4 : 1); ++k) {
+        const int x = (gx + k) % nx;
+        col[k] = x < 0 ? x + nx : x;
+    }
+    const bool lo = WALLS && inside && row == 0, hi = WALLS && inside && row == ny - 1;
+    const bool out = inside && ly >= pl.hy && ly < R - pl.hy && gy < ny && 4 * qx >= pl.hx &&
+                     4 * qx < 4 * Q - pl.hx && gx < nx;
+    // rows of this warp (first and last), to skip those that do not matter
+    const int wy0 = int(threadIdx.x & ~31u) >> pl.q_log2, wy1 = int(threadIdx.x | 31u) >> pl.q_log2;
+    const bool beyond = WALLS && (gy - ly + wy1 < 0 || gy - ly + wy0 >= ny);
+
+    const long long base = (long long)row * nx;
+    auto coef = [&](const float *p) {
+        Quad q;
+        if constexpr (ODD) {
+            q.p[0] = mk2(p[base + col[0]], p[base + col[1]]);
+            q.p[1] = mk2(p[base + col[2]], p[base + col[3]]);
+        } else {
+            const uint4 w = *reinterpret_cast<const uint4 *>(p + base + col[0]);
+            memcpy(&q, &w, 16);
+        }
+        return q;
+    };
+    const Quad zero{{f2{0}, f2{0}}};
+    // no step kernel writes the coefficients: they load while the one before drains
+    const Quad a = coef(alpha), e = coef(epsv), b = FORCH ? coef(betav) : zero;
+    pdl_enter();
+    uint32_t t0 = ph.tstep;
+    if constexpr (Store<T>::kSmall) {
+        if (ph.clock) t0 = *ph.clock + ph.step_off;
+    }
+    auto right = [&](const Quad &r) {  // node x takes x - 1 within the row's lanes
+        const float n = __shfl_up_sync(0xffffffffu, hi2(r.p[1]), 1, Q);
+        return Quad{{mk2(n, lo2(r.p[0])), mk2(hi2(r.p[0]), lo2(r.p[1]))}};
+    };
+    auto left = [&](const Quad &r) {
+        const float n = __shfl_down_sync(0xffffffffu, lo2(r.p[0]), 1, Q);
+        return Quad{{mk2(hi2(r.p[0]), lo2(r.p[1])), mk2(hi2(r.p[1]), n)}};
+    };
+
+    Quad g[9];
+    {
+        const int rm = row == 0 ? ny - 1 : row - 1, rp = row == ny - 1 ? 0 : row + 1;
+        // at a wall the opposite population that left the node returns to it
+        const int rlo = lo ? row : rm, rhi = hi ? row : rp;
+        const int plane[9] = {0, 1, lo ? 4 : 2, 3, hi ? 2 : 4, lo ? 7 : 5, lo ? 8 : 6, hi ? 5 : 7, hi ? 6 : 8};
+        const int from[9] = {row, row, rlo, row, rhi, rlo, rlo, rhi, rhi};
+        Quad f[9];
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const T *p = src + (long long)plane[i] * geo.plane + (long long)from[i] * nx;
+            T t[4];
+            if constexpr (ODD) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) t[k] = p[col[ODD ? k : 0]];
+            } else {
+                ld16<T, 4>(p + col[0], t);
+            }
+            f[i] = unpack4<T>(t, c.inv_s);
+        }
+        g[0] = f[0], g[2] = f[2], g[4] = f[4];
+        g[1] = right(f[1]), g[3] = left(f[3]);
+        const Quad s5 = right(f[5]), s6 = left(f[6]), s7 = left(f[7]), s8 = right(f[8]);
+        auto pick = [](bool first, const Quad &p, const Quad &q) {
+            return Quad{{f2{first ? p.p[0].v : q.p[0].v}, f2{first ? p.p[1].v : q.p[1].v}}};
+        };
+        g[5] = pick(lo, f[5], s5), g[6] = pick(lo, f[6], s6);
+        g[7] = pick(hi, f[7], s7), g[8] = pick(hi, f[8], s8);
+    }
+    for (int s = 0; s < nsteps; ++s) {
+        const int reach = nsteps - 1 - s;  // rows beyond the inside that still matter
+        const bool work = !beyond && wy1 >= pl.hy - reach && wy0 < R - pl.hy + reach;
+        if (work) {
+            collide4<T, FORCH>(g, a, e, b, c);
+            T stored[9][4];
+            if constexpr (Store<T>::kSmall) {
+                const uint32_t key = step_key_of(t0 + uint32_t(s), ph.seed);
+                if constexpr (ODD) {
+                    uint32_t hash[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) hash[k] = mix32(uint32_t(base + col[ODD ? k : 0]) ^ key);
+                    for_pops([&](auto i) {
+                        const Quad &q = g[i.value];
+                        const float v[4] = {lo2(q.p[0]), hi2(q.p[0]), lo2(q.p[1]), hi2(q.p[1])};
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) stored[i.value][k] = round1<T, i.value>(v[k], ph.scale, hash[k]);
+                    });
+                } else {
+                    const uint32_t seed = mix32(uint32_t(base + col[0]) ^ key);
+                    for_pops([&](auto i) {
+                        const uint2 w = round4<T, i.value>(g[i.value], c.scale, seed);
+                        memcpy(stored[i.value], &w, 8);
+                    });
+                }
+            } else {
+                memcpy(stored, g, sizeof(stored));
+            }
+            if (reach == 0) {
+                if (out) {
+#pragma unroll
+                    for (int i = 0; i < 9; ++i) {
+                        T *p = dst + (long long)i * geo.plane + base + gx;
+                        if constexpr (ODD) {
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+                                if (gx + k < nx) p[k] = stored[i][k];
+                        } else {
+                            st16<T, 4>(p, stored[i]);
+                        }
+                    }
+                }
+                break;
+            }
+            if constexpr (Store<T>::kSmall) {
+#pragma unroll
+                for (int i = 0; i < 9; ++i) g[i] = unpack4<T>(stored[i], c.inv_s);
+            }
+            // slots: population set {2, 5, 6 | 4, 7, 8}, row + 1, lane
+            float4 *buf = tile_smem + (s & 1) * 6 * (R + 2) * Q + qx;
+            auto slot = [&](int set, int r) { return buf + (set * (R + 2) + r + 1) * Q; };
+            if (inside) {
+                if (lo) {
+                    memcpy(slot(0, ly - 1), &g[4], 16);
+                    memcpy(slot(1, ly - 1), &g[7], 16);
+                    memcpy(slot(2, ly - 1), &g[8], 16);
+                }
+                if (hi) {
+                    memcpy(slot(3, ly + 1), &g[2], 16);
+                    memcpy(slot(4, ly + 1), &g[5], 16);
+                    memcpy(slot(5, ly + 1), &g[6], 16);
+                }
+            }
+            g[1] = right(g[1]), g[3] = left(g[3]);
+            g[5] = right(g[5]), g[6] = left(g[6]), g[7] = left(g[7]), g[8] = right(g[8]);
+            if (inside) {
+                memcpy(slot(0, ly), &g[2], 16);
+                memcpy(slot(1, ly), &g[5], 16);
+                memcpy(slot(2, ly), &g[6], 16);
+                memcpy(slot(3, ly), &g[4], 16);
+                memcpy(slot(4, ly), &g[7], 16);
+                memcpy(slot(5, ly), &g[8], 16);
+            }
+        } else if (reach == 0) {
+            break;
+        }
+        __syncthreads();
+        const float4 *buf = tile_smem + (s & 1) * 6 * (R + 2) * Q + qx;
+        auto slot = [&](int set, int r) { return buf + (set * (R + 2) + r + 1) * Q; };
+        memcpy(&g[2], slot(0, ly - 1), 16);
+        memcpy(&g[5], slot(1, ly - 1), 16);
+        memcpy(&g[6], slot(2, ly - 1), 16);
+        memcpy(&g[4], slot(3, ly + 1), 16);
+        memcpy(&g[7], slot(4, ly + 1), 16);
+        memcpy(&g[8], slot(5, ly + 1), 16);
+    }
 }
 
 // Device step counter of 16-bit storage (see Phys::clock): set to a value
