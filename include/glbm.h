@@ -563,8 +563,9 @@ void glbm_nn_tc_debug_starve(int stage);
 /* Choice of tensor-core convolution kernel for glbm_nn_tc_conv and
  * glbm_nn_tc_conv_fused (process-wide):
  * 0 (default) = per layer: 3x3 layers with BF16 output, rows of >= 128
- * pixels and 32 or 64 output channels where one CTA per (image, 128-pixel
- * strip) leaves segments of >= 16 rows per SM run the streaming kernel (each
+ * pixels and 32, 64, 128, 192 or 256 output channels (in groups of 64) where
+ * one CTA per (image, 128-pixel strip, group) leaves segments of >= 16 rows
+ * per SM run the streaming kernel (each
  * CTA walks down its strip, each input row multiplied once into a ring of
  * row accumulators in tensor memory; the three vertical taps stacked into
  * one MMA of 96 or 192 columns where the weights fit shared memory with

@@ -548,7 +548,7 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
     }
 }
 
-// ---- Streaming variant for 32 and 64 output channels --------------------------
+// ---- Streaming variant for 32, 64 and groups of 64 output channels --------------------------
 // The band kernel above clears and drains its accumulator per band of R = 4
 // rows: the stacked MMA of each of the band's R + 2 halo rows also feeds the
 // two rows above and below the band, 1.5x the MMAs the outputs need, and the
@@ -577,7 +577,15 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // Where the weights do not fit in shared memory (wstream), each stage brings
 // the nine weight tiles of its chunk along with its input rows (stacked: in
 // the 17-tile layout with its zero tiles; else four-row groups, so that each
-// weight tile serves four rows per load).  With up2 the epilogue writes the
+// weight tile serves four rows per load).
+// Layers with 128, 192 or 256 output channels run as groups of 64, one CTA per
+// group, strip and segment: a ring of 128-column slots would hold only two row
+// pairs, and reading the input once per group from L2 costs less than the tile
+// kernel's nine loads of every pixel.  512^2: 256 -> 128 channels 192 us (tile
+// kernel, 804 TFLOP/s) -> 158 us (977), 128 -> 128 115 -> 92, 64 -> 128 71 -> 48;
+// 1024^2 128 -> 128 374 -> 326.  Segments below 16 rows stay on the tile kernel
+// (256^2: 54 us against 58).
+// With up2 the epilogue writes the
 // output 2x nearest-upsampled by TMA stores from a staged row pair.
 // Roles: warp 0 TMA (G input rows of one 32-channel chunk per stage: boxes
 // of G rows, as tall as the band kernel's, keep the TMA engine streaming),
@@ -590,6 +598,7 @@ constexpr int ST_SMAX = 12;
 
 struct StreamArgs {
     int n, h, w, nchunk0, nchunk, nbx, nseg, L, stages;
+    int groups;  // groups of COUT output channels, one CTA each (1, or cout / 64)
     int starve;  // test hook: stage number + 1 the first CTA leaves unloaded
     int nblk;              // 8-channel blocks per chunk: 4, or 2 for a 16-channel input
     uint32_t blk_stride;   // bytes between the 8-channel blocks of a stage (LBO)
@@ -646,7 +655,8 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
     const int S = a.stages;
     const int seg = int(blockIdx.x % unsigned(a.nseg));
     const int rest = int(blockIdx.x / unsigned(a.nseg));
-    const int bx = rest % a.nbx, img = rest / a.nbx;
+    const int o0 = rest % a.groups * COUT;  // first output channel
+    const int bx = rest / a.groups % a.nbx, img = rest / a.groups / a.nbx;
     const int ya = seg * a.L;
     const int Lseg = min(a.L, a.h - ya);
     // input rows ya - 1 .. ya + Lseg (local index ir = 0 .. Lseg + 1), G per
@@ -657,7 +667,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
     constexpr int hg = G / 2;
     const int ngroups = (Lseg + 2 + G - 1) / G;
     const int npairs = (Lseg + 1) / 2;
-    if (threadIdx.x < COUT) sbias[threadIdx.x] = a.bias[threadIdx.x];
+    if (threadIdx.x < COUT) sbias[threadIdx.x] = a.bias[o0 + threadIdx.x];
     // head weights, zero for the outputs beyond head_out (computed, never stored)
     if (threadIdx.x < 4 * 32)
         shead[threadIdx.x] =
@@ -709,7 +719,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                         tma_load_3d(
                             sW + size_t(STACK ? 2 + 5 * (ch * 3 + tap % 3) + (2 - tap / 3) : tap * a.nchunk + ch) *
                                      a.wtile,
-                            &mapB, &wfull, ch * TC_KC, 0, tap);
+                            &mapB, &wfull, ch * TC_KC, o0, tap);
             }
             long long i = 0;
             bool go = true;
@@ -733,7 +743,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                         for (int tap = 0; tap < 9; ++tap)
                             tma_load_3d(dst + a.wofs +
                                             size_t(STACK ? 2 + 5 * (tap % 3) + (2 - tap / 3) : tap) * a.wtile,
-                                        &mapB, &full[s], ch * TC_KC, 0, tap);
+                                        &mapB, &full[s], ch * TC_KC, o0, tap);
                 }
             if (!a.wstream) mbar_drain(&wfull, 0);
             drain_ring(full, S, i);
@@ -920,7 +930,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                         if (r0 + u >= Lseg) break;
                         uint4 *dst = reinterpret_cast<uint4 *>(
                             static_cast<__nv_bfloat16 *>(a.y) + (((long long)img * a.h + ya + r0 + u) * a.w + px) * a.ys +
-                            cg * 32);
+                            o0 + cg * 32);
 #pragma unroll
                         for (int j4 = 0; j4 < 4; ++j4)
                             dst[j4] = make_uint4(pk[u][4 * j4], pk[u][4 * j4 + 1], pk[u][4 * j4 + 2], pk[u][4 * j4 + 3]);
@@ -1304,10 +1314,18 @@ struct StreamPlan {
     bool wstream;        // weights travel with each stage (too many to keep resident)
     uint32_t wofs;       // wstream: byte offset of the weight tiles in a stage
     size_t stage_bytes;
+    int groups;          // CTAs per strip and segment, 64 output channels each
 };
 
-bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p, bool up2 = false) {
+// grouped: cout may be 128, 192 or 256, split into groups of 64.
+bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p, bool up2 = false,
+                 bool grouped = false) {
     if (w < TC_M || g_tc_variant == 1 || g_tc_variant == 3 || g_tc_variant == 4) return false;
+    p->groups = 1;
+    if (grouped && cout > 64 && cout % 64 == 0 && cin % TC_KC == 0) {
+        p->groups = cout / 64;
+        cout = 64;
+    }
     if (cout != 32 && cout != 64) return false;
     const bool resident = size_t(9) * kchunks(cin) * TC_KC * cout * 2 <= kBandMaxWeights;
     // 32 output channels: resident weights only (the stacked tiles with
@@ -1328,7 +1346,7 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     const size_t wbytes = !resident ? 0 : stack ? wstack : size_t(9) * kchunks(cin) * cout * TC_KC * 2;
     // the 227 KB per block less this kernel's ~5 KB of static shared memory
     constexpr size_t kStreamSmemLimit = 221 * 1024;
-    const long long units = (long long)n * ((w + TC_M - 1) / TC_M);
+    const long long units = (long long)n * ((w + TC_M - 1) / TC_M) * p->groups;
     if (units > nsm) return false;
     int segs = int(nsm / units);
     int l = (h + segs - 1) / segs;
@@ -1367,6 +1385,7 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
                           const StreamPlan &pl, void *pool_y = nullptr, const void *head_w = nullptr,
                           const float *head_b = nullptr, float *head_y = nullptr, int head_out = 0,
                           bool up2 = false) {
+    cout /= pl.groups;  // output channels of a CTA
     const int L = pl.L, nseg = pl.nseg, G = pl.G, stages = pl.stages;
     const size_t smem = pl.smem;
     CUtensorMap mA0, mA1, mY0, mY1;
@@ -1399,6 +1418,7 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
     a.nblk = c0 % TC_KC ? 2 : 4;
     a.nbx = (w + TC_M - 1) / TC_M;
     a.nseg = nseg;
+    a.groups = pl.groups;
     a.L = L;
     a.stages = stages;
     a.blk_stride = uint32_t((size_t(G) * BAND_PX * 16 + 127) / 128 * 128);
@@ -1432,7 +1452,7 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
                              : (G == 4 ? k_tc_conv_stream<4, 32, true> : k_tc_conv_stream<2, 32, true>));
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv: shared memory attribute (streaming)");
-    const unsigned grid = unsigned((long long)n * a.nbx * nseg);
+    const unsigned grid = unsigned((long long)n * a.nbx * pl.groups * nseg);
     kern<<<grid, ST_THREADS, smem, st>>>(mA0, mA1, mB, mY0, mY1, a);
     e = cudaGetLastError();
     return e == cudaSuccess ? GLBM_OK : tccuda(e, "nn_tc_conv launch (streaming)");
@@ -1481,23 +1501,24 @@ extern "C" glbm_status glbm_nn_tc_conv(const void *x0, int c0, const void *x1, i
     if (!map_act(&mA0, x0, c0, w, h, n, tw, th) || !map_act(&mA1, c1 > 0 ? x1 : x0, c1 > 0 ? c1 : c0, w, h, n, tw, th))
         return tcfail(GLBM_EINVAL, "nn_tc_conv: activation tensor map rejected");
     const int cin = c0 + c1, taps = k * k;
+    int nsm = 0;
+    if (sm_count(&nsm)) return tcfail(GLBM_ECUDA, "nn_tc_conv: device query failed");
+    StreamPlan pl;
+    const bool streams = k == 3 && !f32_nchw && stream_plan(w, h, n, cin, cout, nsm, &pl, false, true);
     {
         const cuuint64_t dims[3] = {cuuint64_t(cin), cuuint64_t(cout), cuuint64_t(taps)};
         const cuuint64_t strides[2] = {cuuint64_t(cin) * 2, cuuint64_t(cin) * 2 * cout};
-        const cuuint32_t box[3] = {TC_KC, cuuint32_t(cout), 1};
+        const cuuint32_t box[3] = {TC_KC, cuuint32_t(streams ? cout / pl.groups : cout), 1};
         const cuuint32_t es[3] = {1, 1, 1};
         if (encode_fn()(&mB, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(wt), dims, strides, box, es,
                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return tcfail(GLBM_EINVAL, "nn_tc_conv: weight tensor map rejected");
     }
-    int nsm = 0;
-    if (sm_count(&nsm)) return tcfail(GLBM_ECUDA, "nn_tc_conv: device query failed");
     int R = 0, stages = 0;
     size_t bsmem = 0;
     int stack = 0;
-    StreamPlan pl;
-    if (k == 3 && !f32_nchw && stream_plan(w, h, n, cin, cout, nsm, &pl))
+    if (streams)
         return launch_stream(x0, c0, x1, c1, n, h, w, mB, bias, cout, y, ys, relu, err,
                              static_cast<cudaStream_t>(stream), pl);
     if (g_tc_variant != 1 && band_plan(k, f32_nchw, w, cin, cout, h, &R, &stages, &bsmem, &stack))
