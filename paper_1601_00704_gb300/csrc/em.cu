@@ -14,6 +14,7 @@
 // Each launch writes per-block partials that the last block adds in a fixed
 // order, so a fit is bit-for-bit reproducible.
 //
+#include "fixed.cuh"
 #include "glbm.h"
 
 #include <cuda_runtime.h>
@@ -29,6 +30,7 @@ namespace {
 constexpr int KMAX = 8;
 constexpr int EM_THREADS = 256;   // two-pass kernels
 constexpr int STEP_THREADS = 128;  // k_em_step
+constexpr int STEP_BLOCKS = 4;     // of it per SM
 
 // Progress of a fit on the device.
 struct EmState {
@@ -94,39 +96,35 @@ __device__ __forceinline__ void block_sums(double (&v)[CNT], int cnt, double *__
     }
 }
 
-// Sum of logarithms as a running product: mantissas multiply (relative error
-// 2^-53 each, as small as a log's), exponents add, and one log at the very end
-// replaces one per sample.  Factors that are zero, subnormal, infinite or NaN
-// go through log().
+// Sum of logarithms as a running product: significands multiply, exponents
+// add, and one log at the very end replaces one per sample.  Factors that are
+// zero, subnormal, infinite or NaN go through log().
 __device__ __forceinline__ double split_exponent(double f, long long &exps) {  // f normal, positive
     const long long b = __double_as_longlong(f);
     exps += (b >> 52) - 1023;
     return __longlong_as_double((b & 0x000fffffffffffffll) | 0x3ff0000000000000ll);  // in [1, 2)
 }
-struct LogSum {
-    double prod = 1.0, rest = 0.0;
-    long long exps = 0;
-    int n = 0;
-    __device__ __forceinline__ void add(double f) {
-        const int e = int(__double_as_longlong(f) >> 52);  // sign and exponent: 1 .. 2046 for normal positive
-        if (e < 1 || e > 2046) {
-            rest += log(f);
-            return;
-        }
-        prod *= split_exponent(f, exps);
-        if (++n == 1000) prod = split_exponent(prod, exps), n = 0;  // stays below 2^1001
-    }
-};
 
-// One EM iteration.  Bound by FP64 issue (GB300 has two FP64 lanes per SM):
-// about 45 operations per sample and component for the exponential, the
-// shared reciprocal and the three sums, so everything that is not per sample
-// is kept off it: the component factors are formed once per iteration by the
-// last block, logarithms are one product, and block sums go through shared
-// memory (8 FP64 instructions per sum and block of 4 warps instead of 20 by
-// shuffles).  4 blocks per SM.  10^6 samples, 2 components, us an iteration:
-// two passes with a one-thread sum of the block partials 1154, this form with
-// a log per thread and shuffled block sums 190, as written 131.
+// A number beyond FP64's normal range, or one whose products with others of
+// its kind might leave it, is handled in FP64 instructions.
+__device__ __forceinline__ bool tame(double x) {
+    const int f = fx::field(x);
+    return f >= 1 && f <= 2046;
+}
+constexpr int kNever = 1 << 16;  // exponent that no product brings back into range
+
+__device__ const fx::Table g_exp_table = fx::make_table();
+
+// One EM iteration.  Bound by FP64 issue (GB300 has two FP64 lanes per SM), so
+// what is not a sum runs on the integer units, which issue 64 instructions for
+// one of FP64 (fixed.cuh): exponent, exponential, weight, reciprocal and the
+// product under the logarithm.  FP64 keeps d, the sum of the weights, w d and
+// the three sums: 6 instructions per sample and component instead of 38.
+// Component factors are formed once per iteration by the last block, and block
+// sums go through shared memory (8 FP64 instructions per sum and block of 4
+// warps instead of 20 by shuffles).  4 blocks per SM.  10^6 samples, 2
+// components, us an iteration: two passes with a one-thread sum of the block
+// partials 1154, one pass in FP64 instructions 131, as written 68.
 // part: 3K sums, product, rest (doubles) and exponents, [3K + 3][blocks].
 template <int K>
 __global__ void __launch_bounds__(STEP_THREADS)
@@ -136,42 +134,65 @@ k_em_step(const double *__restrict__ x, long long m, EmParams *__restrict__ pp, 
     constexpr int W = 3 * K + 3, PROD = 3 * K, REST = 3 * K + 1, EXPS = 3 * K + 2, NW = STEP_THREADS / 32;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nb = gridDim.x;
-    double mu[K], amp[K], hiv[K], v[3 * K];
+    __shared__ uint64_t table[128];
+    static_assert(STEP_THREADS >= 128, "one table entry per thread");
+    if (threadIdx.x < 128) table[threadIdx.x] = g_exp_table.t[threadIdx.x];
+    double mu[K], v[3 * K];
+    fx::Num amp[K], rate[K];  // weight is amp 2^(-rate d^2)
 #pragma unroll
     for (int j = 0; j < K; ++j) {
         mu[j] = pp->mu[j];
-        amp[j] = pp->amp[j];
-        hiv[j] = pp->hiv[j];
+        amp[j] = fx::unpack(pp->amp[j]);
+        rate[j] = fx::mul(fx::unpack(pp->hiv[j]), fx::Num{fx::kLog2e, 0});
+        if (!tame(pp->amp[j]) || !tame(pp->hiv[j])) rate[j].e = kNever;
         v[j] = v[K + j] = v[2 * K + j] = 0.0;
     }
-    LogSum ls;
+    __syncthreads();
+    fx::Num prod{1ull << 63, 0};
+    double rest = 0.0;
+    long long exps = 0;
     for (long long i = blockIdx.x * (long long)STEP_THREADS + threadIdx.x; i < m; i += (long long)nb * STEP_THREADS) {
         const double xi = x[i];
         double d[K], w[K], den = 0.0;
 #pragma unroll
         for (int j = 0; j < K; ++j) {
             d[j] = xi - mu[j];
-            w[j] = amp[j] * exp(hiv[j] * (d[j] * d[j]));
-            den += w[j];
+            const fx::Num a = fx::unpack(d[j]), t = fx::mul(fx::mul(a, a), rate[j]);
+            fx::Num n{0, kNever};
+            if (t.e <= 9) n = fx::mul(fx::exp2_neg(t, table), amp[j]);
+            if (n.e >= -1022 && n.e <= 1000) w[j] = fx::pack(n);
+            else w[j] = pp->amp[j] * exp(pp->hiv[j] * (d[j] * d[j]));
+            den = j ? den + w[j] : w[0];
         }
-        const double inv = 1.0 / den;
+        const bool normal = tame(den) && den > 0.0;
+        const fx::Num dn = fx::unpack(den), inv = fx::reciprocal(dn);
+        if (normal) {
+            prod = fx::mul(prod, dn);
+            exps += prod.e;
+            prod.e = 0;
+        } else {
+            rest += log(den);
+        }
 #pragma unroll
         for (int j = 0; j < K; ++j) {
-            const double r = w[j] * inv, rd = r * d[j];
+            const fx::Num n = fx::mul(fx::unpack(w[j]), inv);
+            double r;
+            if (normal && tame(w[j]) && n.e >= -1022) r = fx::pack(n);
+            else r = w[j] * (1.0 / den);
+            const double rd = r * d[j];
             v[j] += r;
             v[K + j] += rd;
             v[2 * K + j] += rd * d[j];
         }
-        ls.add(den);
     }
     // sums of the block, then of all blocks by the last one, in fixed order
     __shared__ double sh[W][STEP_THREADS];
     __shared__ bool last;
 #pragma unroll
     for (int c = 0; c < 3 * K; ++c) sh[c][threadIdx.x] = v[c];
-    sh[PROD][threadIdx.x] = split_exponent(ls.prod, ls.exps);
-    sh[REST][threadIdx.x] = ls.rest;
-    sh[EXPS][threadIdx.x] = __longlong_as_double(ls.exps);
+    sh[PROD][threadIdx.x] = fx::pack(prod);
+    sh[REST][threadIdx.x] = rest;
+    sh[EXPS][threadIdx.x] = __longlong_as_double(exps);
     __syncthreads();
     // column c of n values: sum, product or integer sum, in lane 0
     auto column = [&](int c, auto value, int n) {
@@ -192,7 +213,7 @@ k_em_step(const double *__restrict__ x, long long m, EmParams *__restrict__ pp, 
         return t;
     };
     for (int c = warp; c < W; c += NW) {
-        const double t = column(c, [&](int q) { return sh[c][q]; }, STEP_THREADS);  // product: 128 factors below 2
+        const double t = column(c, [&](int q) { return sh[c][q]; }, STEP_THREADS);  // product: 128 factors up to 2
         if (lane == 0) {
             __stcg(part + (long long)c * nb + blockIdx.x, t);
             __threadfence();
@@ -361,7 +382,7 @@ extern "C" glbm_status glbm_em_gmm1d(const double *x, long long m, int k, double
     for (int j = 0; j < k; ++j) hp.phi[j] /= fsum;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int nb = int(std::min<long long>((m + EM_THREADS - 1) / EM_THREADS, 152LL * 8));
-    const int nbs = int(std::min<long long>((m + STEP_THREADS - 1) / STEP_THREADS, 152LL * 4));
+    const int nbs = int(std::min<long long>((m + STEP_THREADS - 1) / STEP_THREADS, 152LL * STEP_BLOCKS));
     // one workspace: estimate, progress, Phi sums, block partials of either form
     const size_t parts = std::max(size_t(nbs) * (3 * k + 3), size_t(nb) * (2 * KMAX + 1));
     em_factors(hp);
