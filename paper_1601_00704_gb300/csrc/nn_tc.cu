@@ -74,7 +74,7 @@ k_tc_conv(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUt
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int x0 = blockIdx.x * a.tw, y0 = blockIdx.y * (MT * a.th), img = blockIdx.z;
     const int iters = a.taps * a.nchunk;
 
@@ -96,16 +96,15 @@ k_tc_conv(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUt
     if (warp == 0) {
         if (lane == 0) {
             const uint32_t bytes = uint32_t(MT * a.tw * a.th * TC_KC * 2 + stage_b);
-            int i = 0;
+            int i = 0, tap = 0, ch = 0;
             for (; i < iters; ++i) {
                 const int s = i % S, use = i / S;
                 if (use > 0 && !mbar_wait(&empty[s], (use - 1) & 1, &abort_flag, a.err, 1)) break;
-                const int tap = i / a.nchunk, ch = i - tap * a.nchunk;
                 const int dy = a.taps == 9 ? tap / 3 - 1 : 0, dx = a.taps == 9 ? tap % 3 - 1 : 0;
                 mbar_expect_tx(&full[s], bytes);
-                if (a.starve == i + 1 && blockIdx.x + blockIdx.y + blockIdx.z == 0) continue;
+                const bool starved = a.starve == i + 1 && blockIdx.x + blockIdx.y + blockIdx.z == 0;
 #pragma unroll
-                for (int t = 0; t < MT; ++t) {
+                for (int t = 0; t < MT && !starved; ++t) {
                     uint8_t *dst = sA + (s * MT + t) * TC_STAGE_A;
                     const int yt = y0 + t * a.th + dy;
                     if (ch < a.nchunk0)
@@ -113,12 +112,14 @@ k_tc_conv(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUt
                     else
                         tma_load_4d(dst, &mapA1, &full[s], (ch - a.nchunk0) * TC_KC, x0 + dx, yt, img);
                 }
-                tma_load_3d(sB + s * stage_b, &mapB, &full[s], ch * TC_KC, 0, tap);
+                if (!starved) tma_load_3d(sB + s * stage_b, &mapB, &full[s], ch * TC_KC, 0, tap);
+                if (++ch == a.nchunk) ch = 0, ++tap;
             }
             drain_ring(full, S, i);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
+            const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
             const uint32_t idesc = idesc_bf16(a.cout);
             for (int i = 0; i < iters; ++i) {
                 const int s = i % S, use = i / S;
@@ -130,12 +131,12 @@ k_tc_conv(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUt
                     const uint64_t ad = sdesc_k64(sA + (s * MT + t) * TC_STAGE_A);
 #pragma unroll
                     for (int kk = 0; kk < TC_KC / 16; ++kk)  // K = 16 per MMA: 32 bytes along the row
-                        umma_bf16(tmem + uint32_t(t) * a.acc_cols, ad + uint64_t((kk * 32) >> 4),
+                        umma_bf16_if(one, tmem + uint32_t(t) * a.acc_cols, ad + uint64_t((kk * 32) >> 4),
                                   bd + uint64_t((kk * 32) >> 4), idesc, (i > 0 || kk > 0) ? 1u : 0u);
                 }
-                umma_commit(&empty[s]);
+                umma_commit_if(one, &empty[s]);
             }
-            umma_commit(&done);  // after a timeout too: the wait below retires every MMA issued
+            umma_commit_if(one, &done);  // after a timeout too: the wait below retires every MMA issued
             mbar_drain(&done, 0);
         }
     } else {
@@ -571,8 +572,8 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // stacked weights with their zero tiles fit in shared memory (STK), each
 // input row takes one N = 192 MMA per tap and K step as above; otherwise
 // three N = 64 MMAs, one per output row (no stacking, so no ring wrap inside
-// an MMA).  A single thread issues MMAs no faster than about one per 46
-// cycles whatever their size, so fewer, larger MMAs win.  Groups of two
+// an MMA).  Issue has a cost per MMA whatever its size, so fewer, larger MMAs
+// win.  Groups of two
 // input rows leave the epilogue two groups of slack in the 4 pair slots.
 // Where the weights do not fit in shared memory (wstream), each stage brings
 // the nine weight tiles of its chunk along with its input rows (stacked: in
@@ -581,10 +582,25 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // Layers with 128, 192 or 256 output channels run as groups of 64, one CTA per
 // group, strip and segment: a ring of 128-column slots would hold only two row
 // pairs, and reading the input once per group from L2 costs less than the tile
-// kernel's nine loads of every pixel.  512^2: 256 -> 128 channels 192 us (tile
-// kernel, 804 TFLOP/s) -> 158 us (977), 128 -> 128 115 -> 92, 64 -> 128 71 -> 48;
-// 1024^2 128 -> 128 374 -> 326.  Segments below 16 rows stay on the tile kernel
-// (256^2: 54 us against 58).
+// kernel's nine loads of every pixel.  Where a group's weights stay resident
+// beside two input rows (32 to 128 input channels) a stage holds one row of
+// one chunk, and once a row's chunks are there they are multiplied tap by tap
+// (rowwise).  Every output is then summed in the tile kernel's order and has
+// its bits: an early layer of other rounding would move a whole network's
+// BF16 output by 1 %.  Rows whose three slots wrap the ring take two MMAs of
+// 64 and 128 columns, so no zero tiles are needed.
+//
+// Input rows lie in shared memory as [row][130 pixels][32 channels] in the
+// 64-byte swizzle: the A operand of a tap starts dx pixels (64 dx bytes) in,
+// and one TMA box of 64-byte pieces brings a stage.  (Unswizzled 8-channel
+// blocks took four boxes of 16-byte pieces.)  The control path is what bounds
+// these layers most: the MMA warp runs as a whole with one lane issuing, so
+// that descriptors stay in uniform registers, and counts its ring position
+// instead of dividing 64-bit stage numbers.
+// us before (16-byte pieces, divisions, one-lane branch) / now, tile kernel in
+// brackets: 512^2 64 -> 128 48 / 46 (78), 128 -> 128 92 / 70 (117), 256 -> 128
+// 158 / 131 (192); 1024^2 128 -> 128 326 / 240 (375), 64 -> 64 85 / 72,
+// 192 -> 64 210 / 195; 2048^2 32 -> 32 137 / 103, 96 -> 32 310 / 240.
 // With up2 the epilogue writes the
 // output 2x nearest-upsampled by TMA stores from a staged row pair.
 // Roles: warp 0 TMA (G input rows of one 32-channel chunk per stage: boxes
@@ -599,11 +615,11 @@ constexpr int ST_SMAX = 12;
 struct StreamArgs {
     int n, h, w, nchunk0, nchunk, nbx, nseg, L, stages;
     int groups;  // groups of COUT output channels, one CTA each (1, or cout / 64)
+    int rowwise;  // 1 (64 channels, stacked): stages of one row, a row's chunks multiplied tap by tap
     int starve;  // test hook: stage number + 1 the first CTA leaves unloaded
-    int nblk;              // 8-channel blocks per chunk: 4, or 2 for a 16-channel input
-    uint32_t blk_stride;   // bytes between the 8-channel blocks of a stage (LBO)
-    uint32_t stage_bytes;  // 4 blocks
-    uint32_t tx_bytes;     // bytes the 4 TMA loads of a stage deliver
+    int kks;               // K steps of 16 channels per chunk: 2, or 1 for a 16-channel input
+    uint32_t stage_bytes;
+    uint32_t tx_bytes;     // bytes the TMA loads of a stage deliver
     uint32_t wtile;        // bytes of one weight slice (32 rows x 64 B)
     const float *bias;
     void *y;  // BF16 NHWC output, or NULL (only the fused outputs)
@@ -626,6 +642,17 @@ struct StreamArgs {
     uint32_t wofs;
 };
 
+// Position in a ring of S stages: slot and the parity of its use.  Counted up,
+// not divided out of a stage number: 64-bit divisions by the runtime S in the
+// thread that issues MMAs took longer than the MMAs.
+struct RingPos {
+    int s = 0;
+    uint32_t parity = 0;
+    __device__ __forceinline__ void next(int S) {
+        if (++s == S) s = 0, parity ^= 1u;
+    }
+};
+
 template <int G, int COUT, bool STK>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
@@ -637,7 +664,8 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int ntile_w = 9 * a.nchunk;
-    const int nslot_w = a.wstream ? 0 : (STACK ? 15 * a.nchunk + 2 : ntile_w);  // stacked: with zero tiles
+    const bool rowwise = STACK && COUT == 64 && a.rowwise;
+    const int nslot_w = a.wstream ? 0 : (STACK && !rowwise ? 15 * a.nchunk + 2 : ntile_w);  // stacked: with zero tiles
     uint8_t *sW = smem;
     uint8_t *sA = smem + size_t(nslot_w) * a.wtile;
     // up2: two buffers of a staged row pair after the stages
@@ -651,7 +679,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
     __shared__ float shead_b[4];
     __shared__ __align__(128) uint8_t szero[4096];  // all-zero A (128 rows x 16 K, unswizzled)
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int S = a.stages;
     const int seg = int(blockIdx.x % unsigned(a.nseg));
     const int rest = int(blockIdx.x / unsigned(a.nseg));
@@ -674,7 +702,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
             a.head_y && threadIdx.x < a.head_out * 32 ? __bfloat162float(a.head_w[threadIdx.x]) : 0.0f;
     if (a.head_y && threadIdx.x < a.head_out) shead_b[threadIdx.x] = a.head_b[threadIdx.x];
     for (int j = threadIdx.x; j < 4096 / 16; j += blockDim.x) reinterpret_cast<uint4 *>(szero)[j] = make_uint4(0, 0, 0, 0);
-    if (STACK) {
+    if (STACK && !rowwise) {
         // the zero tiles: 0, 1 and 5 + 5k, 6 + 5k around (chunk, dx) group k,
         // in the resident weights or, with wstream, in every stage's 17 tiles
         const int per = int(a.wtile / 16);
@@ -717,17 +745,20 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                 for (int tap = 0; tap < 9; ++tap)
                     for (int ch = 0; ch < a.nchunk; ++ch)
                         tma_load_3d(
-                            sW + size_t(STACK ? 2 + 5 * (ch * 3 + tap % 3) + (2 - tap / 3) : tap * a.nchunk + ch) *
+                            sW + size_t(rowwise ? 3 * (ch * 3 + tap % 3) + (2 - tap / 3)
+                                        : STACK ? 2 + 5 * (ch * 3 + tap % 3) + (2 - tap / 3)
+                                                : tap * a.nchunk + ch) *
                                      a.wtile,
                             &mapB, &wfull, ch * TC_KC, o0, tap);
             }
-            long long i = 0;
+            int i = 0;
+            RingPos at;
             bool go = true;
-            for (int g = 0; g < ngroups && go; ++g)
-                for (int ch = 0; ch < a.nchunk; ++ch, ++i) {
-                    const int s = int(i % S);
-                    const long long use = i / S;
-                    if (use > 0 && !mbar_wait_idle(&empty[s], uint32_t(use - 1) & 1u, &abort_flag, a.err, 21)) {
+            const int rows = rowwise ? 1 : G;  // of a stage
+            for (int y = ya - 1; y < ya - 1 + G * ngroups && go; y += rows)
+                for (int ch = 0; ch < a.nchunk; ++ch, ++i, at.next(S)) {
+                    const int s = at.s;
+                    if (i >= S && !mbar_wait_idle(&empty[s], at.parity ^ 1u, &abort_flag, a.err, 21)) {
                         go = false;
                         break;
                     }
@@ -736,9 +767,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                     uint8_t *dst = sA + size_t(s) * a.stage_bytes;
                     const bool first = ch < a.nchunk0;
                     const int c0 = (first ? ch : ch - a.nchunk0) * TC_KC;
-                    for (int blk = 0; blk < a.nblk; ++blk)
-                        tma_load_4d(dst + blk * a.blk_stride, first ? &mapA0 : &mapA1, &full[s], c0 + blk * 8,
-                                    x0 - 1, ya - 1 + G * g, img);
+                    tma_load_4d(dst, first ? &mapA0 : &mapA1, &full[s], c0, x0 - 1, y, img);
                     if (a.wstream)
                         for (int tap = 0; tap < 9; ++tap)
                             tma_load_3d(dst + a.wofs +
@@ -749,7 +778,8 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
             drain_ring(full, S, i);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
+            const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
             // MMA shapes: the main N (3 COUT stacked, else COUT) and the clearing
             // of a row pair's two slots
             const uint32_t idN = idesc_bf16(STACK ? 3 * COUT : COUT), idZ = idesc_bf16(STACK ? 2 * COUT : COUT);
@@ -757,10 +787,12 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
             tc_fence_after();
             const uint64_t zdesc = sdesc_nosw(smem_u32(szero), 2048u, 128u);
             const uint64_t wdesc = sdesc_k64(sW);
-            const uint32_t wt16 = a.wtile >> 4, kstep = (2 * a.blk_stride) >> 4;
-            const int kks = a.nblk / 2;  // K steps of 16 channels per chunk
+            const uint32_t wt16 = a.wtile >> 4;
+            const int kks = a.kks;
+            // A in 16-byte units: a pixel is 4, a K step of 16 channels 2
+            constexpr uint32_t kRow = BAND_PX * 4, kPx = 4, kStep = 2;
             const uint32_t d13 = uint32_t((NS - 3) * COUT);
-            long long i = 0;
+            RingPos at;
             for (int g = 0; g < ngroups && ok; ++g) {
                 // pairs hg g + 1 .. hg g + hg enter their slots: wait until the
                 // epilogue has drained each one's last stored occupant, then
@@ -774,27 +806,54 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                     }
                     tc_fence_after();
                     if (STACK) {
-                        umma_bf16(tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
+                        umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
                     } else {
-                        umma_bf16(tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
-                        umma_bf16(tmem + uint32_t((2 * ps + 1) * COUT), zdesc, zdesc, idZ, 0u);
+                        umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
+                        umma_bf16_if(one, tmem + uint32_t((2 * ps + 1) * COUT), zdesc, zdesc, idZ, 0u);
                     }
                 }
-                for (int ch = 0; ch < a.nchunk && ok; ++ch, ++i) {
-                    const int s = int(i % S);
-                    if (!mbar_wait(&full[s], uint32_t(i / S) & 1u, &abort_flag, a.err, 24)) {
+                for (int ri = 0; ri < G && ok && rowwise; ++ri) {
+                    const int row = G * g + ri, s0 = row % NS, st0 = at.s;
+                    RingPos w = at;
+                    for (int ch = 0; ch < a.nchunk && ok; ++ch, w.next(S))
+                        ok = mbar_wait(&full[w.s], w.parity, &abort_flag, a.err, 24);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t a0 = sdesc_k64(sA);
+                    // slots s0 .. s0 + 2, or those up to the ring's end and then the rest
+                    const int head = min(3, NS - s0);
+                    for (int part = 0; part < (head < 3 ? 2 : 1); ++part) {
+                        const uint32_t d = tmem + uint32_t(part ? 0 : s0 * COUT);
+                        const uint32_t id = idesc_bf16((part ? 3 - head : head) * COUT);
+                        const uint64_t b0 = wdesc + uint64_t((part ? head : 0) * wt16);
+#pragma unroll 1
+                        for (int dxi = 0; dxi < 3; ++dxi)
+#pragma unroll 1
+                            for (int ch = 0; ch < a.nchunk; ++ch) {
+                                const int s = st0 + ch < S ? st0 + ch : st0 + ch - S;
+                                const uint64_t ar = a0 + uint64_t(uint32_t(s) * (a.stage_bytes >> 4) + uint32_t(dxi) * kPx);
+                                const uint64_t br = b0 + uint64_t(uint32_t(3 * (3 * ch + dxi)) * wt16);
+                                umma_bf16_if(one, d, ar, br, id, 1u);
+                                umma_bf16_if(one, d, ar + kStep, br + 2, id, 1u);
+                            }
+                    }
+                    for (int ch = 0; ch < a.nchunk; ++ch, at.next(S)) umma_commit_if(one, &empty[at.s]);
+                }
+                for (int ch = 0; ch < a.nchunk && ok && !rowwise; ++ch, at.next(S)) {
+                    const int s = at.s;
+                    if (!mbar_wait(&full[s], at.parity, &abort_flag, a.err, 24)) {
                         ok = false;
                         break;
                     }
                     tc_fence_after();
-                    const uint64_t a0 = sdesc_nosw(smem_u32(sA + size_t(s) * a.stage_bytes), a.blk_stride, 128u);
+                    const uint64_t a0 = sdesc_k64(sA + size_t(s) * a.stage_bytes);
                     if (!STACK) {
                         // input row G g + ri adds W(dy) to output row G g + ri + 1 - dy; the
                         // weight tile of (tap, chunk) is resident or in this stage
                         const uint64_t wbase = a.wstream ? sdesc_k64(sA + size_t(s) * a.stage_bytes + a.wofs) : wdesc;
 #pragma unroll 1
                         for (int ri = 0; ri < G; ++ri) {
-                            const uint64_t arow = a0 + uint64_t(ri * BAND_PX);  // 16-byte units
+                            const uint64_t arow = a0 + uint64_t(ri * kRow);
 #pragma unroll
                             for (int o = 0; o < 3; ++o) {
                                 const uint32_t d = tmem + uint32_t(((G * g + ri + o) % NS) * COUT);
@@ -806,12 +865,12 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
 #pragma unroll
                                     for (int kk = 0; kk < 2; ++kk)
                                         if (kk < kks)
-                                            umma_bf16(d, arow + uint64_t(dxi + kk * kstep), bt + uint64_t(kk * 2),
+                                            umma_bf16_if(one, d, arow + uint64_t(dxi * kPx + kk * kStep), bt + uint64_t(kk * 2),
                                                       idN, 1u);
                                 }
                             }
                         }
-                        umma_commit(&empty[s]);
+                        umma_commit_if(one, &empty[s]);
                         continue;
                     }
                     // B of (chunk, dx) group k starts at tile 2 + 5k: [W(+1) W(0) W(-1)];
@@ -823,7 +882,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                     for (int ri = 0; ri < G; ++ri) {
                         // input row G g + ri feeds the slots of rows G g + ri .. + 2
                         const int s0 = (G * g + ri) % NS;
-                        const uint64_t arow = a0 + uint64_t(ri * BAND_PX);  // 16-byte units
+                        const uint64_t arow = a0 + uint64_t(ri * kRow);
                         if (s0 <= NS - 3) {
                             const uint32_t d0 = tmem + uint32_t(s0 * COUT);
 #pragma unroll
@@ -831,7 +890,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
 #pragma unroll
                                 for (int kk = 0; kk < 2; ++kk)
                                     if (kk < kks)
-                                        umma_bf16(d0, arow + uint64_t(dxi + kk * kstep),
+                                        umma_bf16_if(one, d0, arow + uint64_t(dxi * kPx + kk * kStep),
                                                   b0 + uint64_t(5 * dxi * wt16 + kk * 2), idN, 1u);
                         } else {
                             // slots 13-15 take B shifted by 1 (s0 = 14: [0 W(+1) W(0)]) or
@@ -843,19 +902,19 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
 #pragma unroll
                                 for (int kk = 0; kk < 2; ++kk) {
                                     if (kk >= kks) break;
-                                    const uint64_t ad = arow + uint64_t(dxi + kk * kstep);
+                                    const uint64_t ad = arow + uint64_t(dxi * kPx + kk * kStep);
                                     const uint64_t bk = b0 + uint64_t(5 * dxi * wt16 + kk * 2);
-                                    umma_bf16(tmem + d13, ad, bk - uint64_t(sh * wt16), idN, 1u);
-                                    umma_bf16(tmem, ad, bk + uint64_t((3 - sh) * wt16), idN, 1u);
+                                    umma_bf16_if(one, tmem + d13, ad, bk - uint64_t(sh * wt16), idN, 1u);
+                                    umma_bf16_if(one, tmem, ad, bk + uint64_t((3 - sh) * wt16), idN, 1u);
                                 }
                         }
                     }
-                    umma_commit(&empty[s]);
+                    umma_commit_if(one, &empty[s]);
                 }
                 for (int pc = hg * g; pc < hg * g + hg && ok; ++pc)
-                    if (pc >= 1 && pc <= npairs) umma_commit(&pfull[pc % NP]);
+                    if (pc >= 1 && pc <= npairs) umma_commit_if(one, &pfull[pc % NP]);
             }
-            umma_commit(&drainbar);  // retire every MMA issued, also after a timeout
+            umma_commit_if(one, &drainbar);  // retire every MMA issued, also after a timeout
             mbar_drain(&drainbar, 0);
         }
     } else if (warp >= 4) {
@@ -1315,6 +1374,7 @@ struct StreamPlan {
     uint32_t wofs;       // wstream: byte offset of the weight tiles in a stage
     size_t stage_bytes;
     int groups;          // CTAs per strip and segment, 64 output channels each
+    bool rowwise;        // stages of one row; every output summed in the tile kernel's order
 };
 
 // grouped: cout may be 128, 192 or 256, split into groups of 64.
@@ -1327,7 +1387,14 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
         cout = 64;
     }
     if (cout != 32 && cout != 64) return false;
-    const bool resident = size_t(9) * kchunks(cin) * TC_KC * cout * 2 <= kBandMaxWeights;
+    // groups whose weights stay resident beside two rows of input sum in the
+    // tile kernel's order (one chunk: they do so anyway)
+    constexpr size_t kStreamSmemLimit = 221 * 1024;  // the 227 KB per block less ~5 KB of static shared memory
+    auto stage_rows = [](int g) { return (size_t(g) * BAND_PX * TC_KC * 2 + 1023) / 1024 * 1024; };  // bytes
+    const size_t row1 = stage_rows(1);
+    const size_t wplain = size_t(9) * kchunks(cin) * TC_KC * cout * 2;
+    p->rowwise = p->groups > 1 && kchunks(cin) > 1 && 1024 + wplain + 2 * kchunks(cin) * row1 <= kStreamSmemLimit;
+    const bool resident = p->rowwise || wplain <= kBandMaxWeights;
     // 32 output channels: resident weights only (the stacked tiles with
     // their zero tiles); 64: resident, or nine tiles per stage
     if (!resident && cout == 32) return false;
@@ -1338,14 +1405,12 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     // the plain tiles; weights carried in each stage stack too (17 tiles per
     // stage)
     const size_t wstack = size_t(15 * kchunks(cin) + 2) * cout * TC_KC * 2;
-    const size_t stage2 = 4 * ((size_t(2) * BAND_PX * 16 + 127) / 128 * 128);
+    const size_t stage2 = stage_rows(2);
     const size_t pair_y = size_t(2) * TC_M * cout * 2;
     const int ystages = up2 ? 2 : 0;
-    const bool stack = cout == 32 || !resident || 1024 + wstack + ystages * pair_y + 2 * stage2 <= 221 * 1024;
+    const bool stack = cout == 32 || !resident || p->rowwise || 1024 + wstack + ystages * pair_y + 2 * stage2 <= 221 * 1024;
     const size_t staged = size_t(ystages) * pair_y;
-    const size_t wbytes = !resident ? 0 : stack ? wstack : size_t(9) * kchunks(cin) * cout * TC_KC * 2;
-    // the 227 KB per block less this kernel's ~5 KB of static shared memory
-    constexpr size_t kStreamSmemLimit = 221 * 1024;
+    const size_t wbytes = !resident ? 0 : stack && !p->rowwise ? wstack : wplain;
     const long long units = (long long)n * ((w + TC_M - 1) / TC_M) * p->groups;
     if (units > nsm) return false;
     int segs = int(nsm / units);
@@ -1361,9 +1426,16 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     // output channels; 2 rows with 64 (the 4 pair slots need two groups of
     // slack), 4 when each stage carries the weights (amortised over 4 rows)
     const int g0 = cout == 32 ? 6 : (resident || stack ? 2 : 4);
+    if (p->rowwise) {
+        p->G = 2;
+        p->stages = std::min(int((kStreamSmemLimit - 1024 - wbytes) / row1), ST_SMAX);
+        p->wofs = 0;
+        p->stage_bytes = row1;
+        p->smem = 1024 + wbytes + size_t(p->stages) * row1;
+        return true;
+    }
     for (int g = g0; g >= 2; g -= 2) {
-        const size_t blk = (size_t(g) * BAND_PX * 16 + 127) / 128 * 128;
-        const size_t arows = resident ? 4 * blk : (4 * blk + 1023) / 1024 * 1024;
+        const size_t arows = stage_rows(g);
         const size_t stage = arows + (resident ? 0 : size_t(stack ? 17 : 9) * cout * TC_KC * 2);
         if (1024 + wbytes + staged + 2 * stage > kStreamSmemLimit) continue;
         const size_t room = kStreamSmemLimit - 1024 - wbytes - staged;
@@ -1404,8 +1476,9 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
                 return tcfail(GLBM_EINVAL, "nn_tc_conv_up2: output tensor map rejected");
         }
     }
-    if (!map_act_band(&mA0, x0, c0, w, h, n, G - 2) ||
-        !map_act_band(&mA1, c1 > 0 ? x1 : x0, c1 > 0 ? c1 : c0, w, h, n, G - 2))
+    const int rows = pl.rowwise ? 1 : G;  // of a stage
+    if (!map_act(&mA0, x0, c0, w, h, n, BAND_PX, rows) ||
+        !map_act(&mA1, c1 > 0 ? x1 : x0, c1 > 0 ? c1 : c0, w, h, n, BAND_PX, rows))
         return tcfail(GLBM_EINVAL, "nn_tc_conv: streaming activation tensor map rejected");
     StreamArgs a;
     a.starve = take_starve();
@@ -1414,19 +1487,18 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
     a.w = w;
     a.nchunk0 = kchunks(c0);
     a.nchunk = a.nchunk0 + c1 / TC_KC;
-    // 16 input channels: two 8-channel blocks and one K step per tap
-    a.nblk = c0 % TC_KC ? 2 : 4;
+    a.kks = c0 % TC_KC ? 1 : 2;  // 16 input channels: one K step per tap
     a.nbx = (w + TC_M - 1) / TC_M;
     a.nseg = nseg;
     a.groups = pl.groups;
+    a.rowwise = pl.rowwise ? 1 : 0;
     a.L = L;
     a.stages = stages;
-    a.blk_stride = uint32_t((size_t(G) * BAND_PX * 16 + 127) / 128 * 128);
     a.wtile = uint32_t(cout * TC_KC * 2);
     a.wstream = pl.wstream ? 1 : 0;
     a.wofs = pl.wofs;
     a.stage_bytes = uint32_t(pl.stage_bytes);
-    a.tx_bytes = uint32_t(a.nblk * G * BAND_PX * 16) + (pl.wstream ? 9 * a.wtile : 0u);
+    a.tx_bytes = uint32_t(rows * BAND_PX * TC_KC * 2) + (pl.wstream ? 9 * a.wtile : 0u);
     a.bias = bias;
     a.y = y;
     a.ys = ys;

@@ -53,3 +53,38 @@ def test_grouped_streaming_layer(lib, n, h, w, c0, c1, cout, variant):
     # the BF16 output rounding (half an ulp = 2^-9 relative) plus FP32 accumulation
     assert bool(((got - ref).abs() <= 2.0 ** -8 * ref.abs() + 1e-6 * ref.abs().max()).all())
     assert bool((y[..., cout:] == -7.0).all())
+
+
+@pytest.mark.parametrize("n,h,w,c0,c1,cout,variant", [
+    (1, 640, 256, 128, 0, 128, 0), (1, 611, 130, 64, 0, 128, 0), (1, 37, 200, 32, 64, 192, 5),
+    (2, 2, 128, 64, 64, 256, 5), (1, 65, 129, 32, 0, 128, 5)])
+def test_resident_groups_sum_in_the_tile_kernels_order(lib, n, h, w, c0, c1, cout, variant):
+    """Up to 128 input channels the groups add taps and channels in the order of
+    the tile kernel (variant 1): the outputs are its bits."""
+    import torch
+    g = torch.Generator(device="cuda").manual_seed(h * w + cout)
+    cin = c0 + c1
+
+    def vp(t):
+        return C.c_void_p(t.data_ptr()) if t is not None else None
+
+    x0 = torch.randn((n, h, w, c0), generator=g, device="cuda").to(torch.bfloat16)
+    x1 = torch.randn((n, h, w, c1), generator=g, device="cuda").to(torch.bfloat16) if c1 else None
+    wf = torch.randn((cout, cin, 3, 3), generator=g, device="cuda").contiguous()
+    b = torch.randn(cout, generator=g, device="cuda")
+    wt = torch.empty(9 * cout * cin, dtype=torch.bfloat16, device="cuda")
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert lib.glbm_nn_tc_pack_weights(vp(wf), cout, cin, 3, cout, cin, vp(wt), st) == 0
+    err = torch.zeros(1, dtype=torch.int32, device="cuda")
+    out = []
+    for v in (1, variant):
+        y = torch.full((n, h, w, cout), -7.0, dtype=torch.bfloat16, device="cuda")
+        lib.glbm_nn_tc_set_variant(v)
+        rc = lib.glbm_nn_tc_conv(vp(x0), c0, vp(x1), c1, n, h, w, 3, vp(wt), vp(b), cout, vp(y), cout, 0, 0, 0, vp(err),
+                                 st)
+        lib.glbm_nn_tc_set_variant(0)
+        assert rc == 0
+        torch.cuda.synchronize()
+        assert int(err) == 0
+        out.append(y)
+    assert torch.equal(*out)
