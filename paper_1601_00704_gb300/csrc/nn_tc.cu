@@ -642,17 +642,6 @@ struct StreamArgs {
     uint32_t wofs;
 };
 
-// Position in a ring of S stages: slot and the parity of its use.  Counted up,
-// not divided out of a stage number: 64-bit divisions by the runtime S in the
-// thread that issues MMAs took longer than the MMAs.
-struct RingPos {
-    int s = 0;
-    uint32_t parity = 0;
-    __device__ __forceinline__ void next(int S) {
-        if (++s == S) s = 0, parity ^= 1u;
-    }
-};
-
 template <int G, int COUT, bool STK>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,

@@ -186,6 +186,12 @@ k_tc_wgrad(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUt
 // A work unit is a band of R dy rows (and the R + 2 x rows they meet) of
 // one kp-pixel strip of one image, loaded once per stage.  Each CTA owns a
 // group of input and output chunks and a contiguous range of units.
+// Bound by the latency of loads and issue: its MMAs (48 cycles each) are
+// issued by a whole warp with one lane active, and unit and ring positions are
+// counted.  Batch 8, us before (one-lane branch, 64-bit divisions) / now:
+// 96 -> 32 at 256^2 63.8 / 51.5, 32 -> 32 at 256^2 30.1 / 27.2, 192 -> 64 at
+// 128^2 57.9 / 50.2, 256 -> 128 at 64^2 43.3 / 37.3; 128 -> 128 at 16^2 and
+// below stay at 12.5, a launch and one unit per CTA.
 constexpr int WB_MAX_STAGES = 4;
 
 struct WgradBandArgs {
@@ -213,7 +219,7 @@ k_tc_wgrad_band(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
     __shared__ uint32_t tmem_base;
     __shared__ volatile int abort_flag;
     __shared__ volatile int s_bad;  // the epilogue warps' joint verdict on the accumulator
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const int xg = blockIdx.x % a.ngx, og = blockIdx.x / a.ngx;
     const int cx0 = xg * a.nxc, co0 = og * a.nob;
     const int nx = min(a.nxc, a.nchunk - cx0), no = min(a.nob, a.nobt - co0);
@@ -242,51 +248,54 @@ k_tc_wgrad_band(const __grid_constant__ CUtensorMap mapX, const __grid_constant_
 
     if (warp == 0) {
         if (lane == 0) {
-            int i = 0;
-            for (; i < iters; ++i) {
-                const int s = i % S, use = i / S;
-                if (use > 0 && !mbar_wait(&empty[s], (use - 1) & 1, &abort_flag, a.err, 21)) break;
-                const long long u = u0 + i;
-                const int x0 = int(u % a.xsteps) * a.kp;
-                const long long band = u / a.xsteps;
-                const int img = int(band / a.ybands), yb = int(band % a.ybands) * a.R;
+            // strip, band and image of the unit, counted up (64-bit divisions cost
+            // this thread as much as its loads)
+            int i = 0, xs = int(u0 % a.xsteps), band = int(u0 / a.xsteps % a.ybands), img = int(u0 / a.xsteps / a.ybands);
+            RingPos at;
+            for (; i < iters; ++i, at.next(S)) {
+                const int s = at.s;
+                if (i >= S && !mbar_wait(&empty[s], at.parity ^ 1u, &abort_flag, a.err, 21)) break;
+                const int x0 = xs * a.kp, yb = band * a.R, im = img;
+                if (++xs == a.xsteps) {
+                    xs = 0;
+                    if (++band == a.ybands) band = 0, ++img;
+                }
                 uint8_t *st = smem + size_t(s) * a.stage_bytes;
                 mbar_expect_tx(&full[s], uint32_t(nx) * uint32_t(a.R + 2) * uint32_t(a.kp * 64) +
                                              uint32_t(no) * uint32_t(a.R) * uint32_t((a.kp + 2) * 64));
                 if (a.starve == i + 1 && blockIdx.x + blockIdx.y == 0) continue;
                 for (int xi = 0; xi < nx; ++xi)
                     for (int t = 0; t < a.R + 2; ++t)
-                        tma_load_4d(st + xi * xblk + t * a.xrow, &mapX, &full[s], (cx0 + xi) * 32, x0, yb - 1 + t, img);
+                        tma_load_4d(st + xi * xblk + t * a.xrow, &mapX, &full[s], (cx0 + xi) * 32, x0, yb - 1 + t, im);
                 for (int ob = 0; ob < no; ++ob)
                     for (int t = 0; t < a.R; ++t)
                         tma_load_4d(st + a.dy_off + ob * dyblk + t * a.dyrow, &mapDY, &full[s], (co0 + ob) * 32, x0 - 1,
-                                    yb + t, img);
+                                    yb + t, im);
             }
             drain_ring(full, S, i);
         }
     } else if (warp == 1) {
-        if (lane == 0) {
-            const uint32_t idesc = idesc_bf16_mn(128, 96);
-            for (int i = 0; i < iters; ++i) {
-                const int s = i % S, use = i / S;
-                if (!mbar_wait(&full[s], use & 1, &abort_flag, a.err, 22)) break;
-                tc_fence_after();
-                uint8_t *st = smem + size_t(s) * a.stage_bytes;
-                for (int t = 0; t < a.R; ++t)
-                    for (int kk = 0; kk < a.kp / 16; ++kk)  // K = 16 pixels per MMA
-                        for (int ob = 0; ob < no; ++ob) {
-                            const uint64_t bd = sdesc_mn64(st + a.dy_off + ob * dyblk + t * a.dyrow + kk * 1024, 64, 512);
-                            for (int xi = 0; xi < nx; ++xi) {
-                                const uint64_t ad = sdesc_mn64(st + xi * xblk + t * a.xrow + kk * 1024, a.xrow, 512);
-                                umma_bf16(tmem + uint32_t(xi * a.nob + ob) * 96u, ad, bd, idesc,
-                                          (i > 0 || t > 0 || kk > 0) ? 1u : 0u);
-                            }
+        const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
+        const uint32_t idesc = idesc_bf16_mn(128, 96);
+        RingPos at;
+        for (int i = 0; i < iters; ++i, at.next(S)) {
+            if (!mbar_wait(&full[at.s], at.parity, &abort_flag, a.err, 22)) break;
+            tc_fence_after();
+            uint8_t *st = smem + size_t(at.s) * a.stage_bytes;
+            for (int t = 0; t < a.R; ++t)
+                for (int kk = 0; kk < a.kp / 16; ++kk)  // K = 16 pixels per MMA
+                    for (int ob = 0; ob < no; ++ob) {
+                        const uint64_t bd = sdesc_mn64(st + a.dy_off + ob * dyblk + t * a.dyrow + kk * 1024, 64, 512);
+                        for (int xi = 0; xi < nx; ++xi) {
+                            const uint64_t ad = sdesc_mn64(st + xi * xblk + t * a.xrow + kk * 1024, a.xrow, 512);
+                            umma_bf16_if(one, tmem + uint32_t(xi * a.nob + ob) * 96u, ad, bd, idesc,
+                                         (i > 0 || t > 0 || kk > 0) ? 1u : 0u);
                         }
-                umma_commit(&empty[s]);
-            }
-            umma_commit(&done);  // after a timeout too: the wait below retires every MMA issued
-            mbar_drain(&done, 0);
+                    }
+            umma_commit_if(one, &empty[at.s]);
         }
+        umma_commit_if(one, &done);  // after a timeout too: the wait below retires every MMA issued
+        mbar_drain(&done, 0);
     } else if (iters > 0) {
         // warps 2-5 (TMEM lanes 32r..: x row y + r - 1, i.e. ky = r; r = 3 holds no
         // tap).  Per (x chunk, dy chunk) the three tap rows are gathered in the

@@ -112,6 +112,17 @@ __device__ void drain_ring(uint64_t *full, int S, long long issued) {
     for (long long u = issued > S ? issued - S : 0; u < issued; ++u) mbar_drain(&full[u % S], uint32_t(u / S) & 1u);
 }
 
+// Position in a ring of S stages: slot and the parity of its use.  Counted up,
+// not divided out of a stage number: 64-bit divisions by the runtime S in the
+// thread that issues MMAs took longer than the MMAs.
+struct RingPos {
+    int s = 0;
+    uint32_t parity = 0;
+    __device__ __forceinline__ void next(int S) {
+        if (++s == S) s = 0, parity ^= 1u;
+    }
+};
+
 // Test hook (glbm_nn_tc_debug_starve): stage number + 1 whose copies the
 // first CTA of the next tensor-core launch leaves unissued, 0 for none.
 inline int take_starve() {
