@@ -29,8 +29,8 @@ namespace {
 
 constexpr int KMAX = 8;
 constexpr int EM_THREADS = 256;   // two-pass kernels
-constexpr int STEP_THREADS = 128;  // k_em_step
-constexpr int STEP_BLOCKS = 4;     // of it per SM
+constexpr int STEP_THREADS = 256;  // k_em_step
+constexpr int STEP_BLOCKS = 2;     // of it per SM
 
 // Progress of a fit on the device.
 struct EmState {
@@ -121,10 +121,12 @@ __device__ const fx::Table g_exp_table = fx::make_table();
 // product under the logarithm.  FP64 keeps d, the sum of the weights, w d and
 // the three sums: 6 instructions per sample and component instead of 38.
 // Component factors are formed once per iteration by the last block, and block
-// sums go through shared memory (8 FP64 instructions per sum and block of 4
-// warps instead of 20 by shuffles).  4 blocks per SM.  10^6 samples, 2
+// sums go through shared memory (13 FP64 instructions per sum and block of 8
+// warps instead of 40 by shuffles).  2 blocks of 8 warps per SM.  10^6 samples, 2
 // components, us an iteration: two passes with a one-thread sum of the block
-// partials 1154, one pass in FP64 instructions 131, as written 68.
+// partials 1154, one pass in FP64 instructions 131, as written 55
+// (4 blocks of 4 warps 62, 4 of 8 60, 2 of 16 60); the FP64 pipe is busy 74 % of
+// the time its SM works.
 // part: 3K sums, product, rest (doubles) and exponents, [3K + 3][blocks].
 template <int K>
 __global__ void __launch_bounds__(STEP_THREADS)
@@ -213,7 +215,7 @@ k_em_step(const double *__restrict__ x, long long m, EmParams *__restrict__ pp, 
         return t;
     };
     for (int c = warp; c < W; c += NW) {
-        const double t = column(c, [&](int q) { return sh[c][q]; }, STEP_THREADS);  // product: 128 factors up to 2
+        const double t = column(c, [&](int q) { return sh[c][q]; }, STEP_THREADS);  // product: 256 factors up to 2
         if (lane == 0) {
             __stcg(part + (long long)c * nb + blockIdx.x, t);
             __threadfence();
@@ -224,7 +226,7 @@ k_em_step(const double *__restrict__ x, long long m, EmParams *__restrict__ pp, 
     __syncthreads();
     if (!last) return;
     __threadfence();
-    long long moved = 0;  // exponents taken off the blocks' products (then 2^nb bounds theirs, nb <= 608)
+    long long moved = 0;  // exponents taken off the blocks' products (then 2^nb bounds theirs, nb <= 304)
     for (int c = warp; c < W; c += NW) {
         const double *p = part + (long long)c * nb;
         const double t = column(

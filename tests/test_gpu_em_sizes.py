@@ -1,4 +1,4 @@
-"""The one-launch EM iteration at the edges of its blocks (128 samples, 608
+"""The one-launch EM iteration at the edges of its blocks (256 samples, 304
 blocks), for every number of components, and where its variance update would
 cancel and the two-pass iteration takes over.  Against the FP64 oracle: sums
 in another order, so 1e-9 relative as in test_gpu_em.py."""
@@ -27,7 +27,7 @@ def check(pkg, orc, x, init, iters):
         assert a[4] == pytest.approx(b[4], rel=1e-12)
 
 
-@pytest.mark.parametrize("m,k", [(127, 1), (128, 1), (129, 2), (1000, 8), (4096, 5), (77823, 2), (77824, 3),
+@pytest.mark.parametrize("m,k", [(127, 1), (128, 1), (129, 2), (255, 2), (256, 3), (257, 1), (1000, 8), (4096, 5), (77823, 2), (77824, 3),
                                  (77825, 4), (200001, 6), (130000, 7)])
 def test_block_edges_and_components(pkg, orc, m, k):
     rng = np.random.default_rng(m + k)
