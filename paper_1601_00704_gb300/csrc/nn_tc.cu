@@ -1405,7 +1405,11 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     int segs = int(nsm / units);
     int l = (h + segs - 1) / segs;
     l += l & 1;  // even: row pairs never straddle two segments
-    if (l < (g_tc_variant == 5 ? 2 : 16)) return false;
+    // short segments repeat their halo rows: from 16 rows on, or from 4 where the
+    // bits are the tile kernel's whichever runs (256^2 128 -> 128 channels, 8
+    // rows: 37 us there, 31 here; 128 x 256, 4 rows: 25 / 22; 128^2, 2 rows: equal)
+    const int least = p->rowwise || (p->groups > 1 && kchunks(cin) == 1) ? 4 : 16;
+    if (l < (g_tc_variant == 5 ? 2 : least)) return false;
     p->L = l;
     p->nseg = (h + l - 1) / l;
     p->wstream = !resident;

@@ -57,7 +57,8 @@ def test_grouped_streaming_layer(lib, n, h, w, c0, c1, cout, variant):
 
 @pytest.mark.parametrize("n,h,w,c0,c1,cout,variant", [
     (1, 640, 256, 128, 0, 128, 0), (1, 611, 130, 64, 0, 128, 0), (1, 37, 200, 32, 64, 192, 5),
-    (2, 2, 128, 64, 64, 256, 5), (1, 65, 129, 32, 0, 128, 5)])
+    (2, 2, 128, 64, 64, 256, 5), (1, 65, 129, 32, 0, 128, 5), (1, 256, 256, 128, 0, 128, 0),
+    (1, 128, 256, 64, 0, 128, 0), (2, 101, 130, 32, 0, 192, 0)])
 def test_resident_groups_sum_in_the_tile_kernels_order(lib, n, h, w, c0, c1, cout, variant):
     """Up to 128 input channels the groups add taps and channels in the order of
     the tile kernel (variant 1): the outputs are its bits."""
