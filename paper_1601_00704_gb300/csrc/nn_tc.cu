@@ -568,17 +568,13 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // so that each adds only its part.  The weights of one (chunk, dx) sit as
 // [0 0 W(+1) W(0) W(-1) 0 0] in shared memory, neighbours sharing their
 // zero tiles.
-// With 64 output channels the ring has 8 slots of 64 columns.  Where the
-// stacked weights with their zero tiles fit in shared memory (STK), each
-// input row takes one N = 192 MMA per tap and K step as above; otherwise
-// three N = 64 MMAs, one per output row (no stacking, so no ring wrap inside
-// an MMA).  Issue has a cost per MMA whatever its size, so fewer, larger MMAs
-// win.  Groups of two
-// input rows leave the epilogue two groups of slack in the 4 pair slots.
-// Where the weights do not fit in shared memory (wstream), each stage brings
-// the nine weight tiles of its chunk along with its input rows (stacked: in
-// the 17-tile layout with its zero tiles; else four-row groups, so that each
-// weight tile serves four rows per load).
+// With 64 output channels the ring has 8 slots of 64 columns and the weights
+// lie without zero tiles: a row that wraps the ring takes its MMAs in two
+// parts, of N = 64 and N = 128.  Issue has a cost per MMA whatever its size,
+// so fewer, larger MMAs win.  Groups of two input rows leave the epilogue two
+// groups of slack in the 4 pair slots.  Where the weights do not fit beside
+// four stages (wstream), each stage brings the nine weight tiles of its chunk
+// along with its input rows.
 // Layers with 128, 192 or 256 output channels run as groups of 64, one CTA per
 // group, strip and segment: a ring of 128-column slots would hold only two row
 // pairs, and reading the input once per group from L2 costs less than the tile
@@ -597,10 +593,10 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // these layers most: the MMA warp runs as a whole with one lane issuing, so
 // that descriptors stay in uniform registers, and counts its ring position
 // instead of dividing 64-bit stage numbers.
-// us before (16-byte pieces, divisions, one-lane branch) / now, tile kernel in
-// brackets: 512^2 64 -> 128 48 / 46 (78), 128 -> 128 92 / 70 (117), 256 -> 128
-// 158 / 131 (192); 1024^2 128 -> 128 326 / 240 (375), 64 -> 64 85 / 72,
-// 192 -> 64 210 / 195; 2048^2 32 -> 32 137 / 103, 96 -> 32 310 / 240.
+// us before (16-byte pieces, divisions, one-lane branch, zero tiles) / now, tile
+// kernel in brackets: 512^2 64 -> 128 48 / 46 (78), 128 -> 128 92 / 70 (117),
+// 256 -> 128 158 / 105 (192); 1024^2 128 -> 128 326 / 240 (375), 64 -> 64
+// 85 / 68, 192 -> 64 210 / 154; 2048^2 32 -> 32 137 / 103, 96 -> 32 310 / 236.
 // With up2 the epilogue writes the
 // output 2x nearest-upsampled by TMA stores from a staged row pair.
 // Roles: warp 0 TMA (G input rows of one 32-channel chunk per stage: boxes
@@ -642,19 +638,19 @@ struct StreamArgs {
     uint32_t wofs;
 };
 
-template <int G, int COUT, bool STK>
+template <int G, int COUT>
 __global__ void __launch_bounds__(ST_THREADS, 1)
 k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
                  const __grid_constant__ CUtensorMap mapB, const __grid_constant__ CUtensorMap mapY0,
                  const __grid_constant__ CUtensorMap mapY1, const StreamArgs a) {
-    constexpr bool STACK = STK;  // dy taps stacked along N (N = 3 COUT)
+    constexpr bool ZEROS = COUT == 32;  // zero tiles between the stacked weights
     constexpr int NS = 512 / COUT;      // TMEM row slots
     constexpr int NP = NS / 2;          // row pair slots
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int ntile_w = 9 * a.nchunk;
-    const bool rowwise = STACK && COUT == 64 && a.rowwise;
-    const int nslot_w = a.wstream ? 0 : (STACK && !rowwise ? 15 * a.nchunk + 2 : ntile_w);  // stacked: with zero tiles
+    const bool rowwise = COUT == 64 && a.rowwise;
+    const int nslot_w = a.wstream ? 0 : ZEROS ? 15 * a.nchunk + 2 : ntile_w;
     uint8_t *sW = smem;
     uint8_t *sA = smem + size_t(nslot_w) * a.wtile;
     // up2: two buffers of a staged row pair after the stages
@@ -691,17 +687,13 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
             a.head_y && threadIdx.x < a.head_out * 32 ? __bfloat162float(a.head_w[threadIdx.x]) : 0.0f;
     if (a.head_y && threadIdx.x < a.head_out) shead_b[threadIdx.x] = a.head_b[threadIdx.x];
     for (int j = threadIdx.x; j < 4096 / 16; j += blockDim.x) reinterpret_cast<uint4 *>(szero)[j] = make_uint4(0, 0, 0, 0);
-    if (STACK && !rowwise) {
-        // the zero tiles: 0, 1 and 5 + 5k, 6 + 5k around (chunk, dx) group k,
-        // in the resident weights or, with wstream, in every stage's 17 tiles
+    if (ZEROS) {
+        // the zero tiles: 0, 1 and 5 + 5k, 6 + 5k around (chunk, dx) group k
         const int per = int(a.wtile / 16);
-        const int nw = a.wstream ? 17 : nslot_w;
-        for (int st = 0; st < (a.wstream ? a.stages : 1); ++st) {
-            uint4 *wz = reinterpret_cast<uint4 *>(a.wstream ? sA + size_t(st) * a.stage_bytes + a.wofs : sW);
-            for (int j = threadIdx.x; j < nw * per; j += blockDim.x) {
-                const int t = j / per;
-                if (t < 2 || (t - 2) % 5 >= 3) wz[j] = make_uint4(0, 0, 0, 0);
-            }
+        uint4 *wz = reinterpret_cast<uint4 *>(sW);
+        for (int j = threadIdx.x; j < nslot_w * per; j += blockDim.x) {
+            const int t = j / per;
+            if (t < 2 || (t - 2) % 5 >= 3) wz[j] = make_uint4(0, 0, 0, 0);
         }
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -734,10 +726,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                 for (int tap = 0; tap < 9; ++tap)
                     for (int ch = 0; ch < a.nchunk; ++ch)
                         tma_load_3d(
-                            sW + size_t(rowwise ? 3 * (ch * 3 + tap % 3) + (2 - tap / 3)
-                                        : STACK ? 2 + 5 * (ch * 3 + tap % 3) + (2 - tap / 3)
-                                                : tap * a.nchunk + ch) *
-                                     a.wtile,
+                            sW + size_t((ZEROS ? 2 : 0) + (ZEROS ? 5 : 3) * (ch * 3 + tap % 3) + (2 - tap / 3)) * a.wtile,
                             &mapB, &wfull, ch * TC_KC, o0, tap);
             }
             int i = 0;
@@ -759,9 +748,8 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                     tma_load_4d(dst, first ? &mapA0 : &mapA1, &full[s], c0, x0 - 1, y, img);
                     if (a.wstream)
                         for (int tap = 0; tap < 9; ++tap)
-                            tma_load_3d(dst + a.wofs +
-                                            size_t(STACK ? 2 + 5 * (tap % 3) + (2 - tap / 3) : tap) * a.wtile,
-                                        &mapB, &full[s], ch * TC_KC, o0, tap);
+                            tma_load_3d(dst + a.wofs + size_t(3 * (tap % 3) + (2 - tap / 3)) * a.wtile, &mapB, &full[s],
+                                        ch * TC_KC, o0, tap);
                 }
             if (!a.wstream) mbar_drain(&wfull, 0);
             drain_ring(full, S, i);
@@ -769,9 +757,9 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
     } else if (warp == 1) {
         {
             const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
-            // MMA shapes: the main N (3 COUT stacked, else COUT) and the clearing
+            // MMA shapes: the main N (three output rows) and the clearing
             // of a row pair's two slots
-            const uint32_t idN = idesc_bf16(STACK ? 3 * COUT : COUT), idZ = idesc_bf16(STACK ? 2 * COUT : COUT);
+            const uint32_t idN = idesc_bf16(3 * COUT), idZ = idesc_bf16(2 * COUT);
             bool ok = a.wstream || mbar_wait(&wfull, 0, &abort_flag, a.err, 22);
             tc_fence_after();
             const uint64_t zdesc = sdesc_nosw(smem_u32(szero), 2048u, 128u);
@@ -794,12 +782,7 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                         break;
                     }
                     tc_fence_after();
-                    if (STACK) {
-                        umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
-                    } else {
-                        umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
-                        umma_bf16_if(one, tmem + uint32_t((2 * ps + 1) * COUT), zdesc, zdesc, idZ, 0u);
-                    }
+                    umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
                 }
                 for (int ri = 0; ri < G && ok && rowwise; ++ri) {
                     const int row = G * g + ri, s0 = row % NS, st0 = at.s;
@@ -836,37 +819,33 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
                     }
                     tc_fence_after();
                     const uint64_t a0 = sdesc_k64(sA + size_t(s) * a.stage_bytes);
-                    if (!STACK) {
-                        // input row G g + ri adds W(dy) to output row G g + ri + 1 - dy; the
-                        // weight tile of (tap, chunk) is resident or in this stage
-                        const uint64_t wbase = a.wstream ? sdesc_k64(sA + size_t(s) * a.stage_bytes + a.wofs) : wdesc;
+                    if (!ZEROS) {
+                        // the weights of a dx are [W(+1) W(0) W(-1)], resident or in this stage
+                        const uint64_t b0 = a.wstream ? sdesc_k64(sA + size_t(s) * a.stage_bytes + a.wofs)
+                                                      : wdesc + uint64_t(uint32_t(9 * ch) * wt16);
 #pragma unroll 1
                         for (int ri = 0; ri < G; ++ri) {
                             const uint64_t arow = a0 + uint64_t(ri * kRow);
+                            const int s0 = (G * g + ri) % NS, head = min(3, NS - s0);
+                            // slots s0 .. s0 + 2, or those up to the ring's end and then the rest
+                            for (int part = 0; part < (head < 3 ? 2 : 1); ++part) {
+                                const uint32_t d = tmem + uint32_t(part ? 0 : s0 * COUT);
+                                const uint32_t id = idesc_bf16((part ? 3 - head : head) * COUT);
+                                const uint64_t bp = b0 + uint64_t((part ? head : 0) * wt16);
 #pragma unroll
-                            for (int o = 0; o < 3; ++o) {
-                                const uint32_t d = tmem + uint32_t(((G * g + ri + o) % NS) * COUT);
-#pragma unroll
-                                for (int dxi = 0; dxi < 3; ++dxi) {
-                                    const int tap = (2 - o) * 3 + dxi;
-                                    const uint64_t bt =
-                                        wbase + uint64_t(a.wstream ? tap : tap * a.nchunk + ch) * wt16;
+                                for (int dxi = 0; dxi < 3; ++dxi)
 #pragma unroll
                                     for (int kk = 0; kk < 2; ++kk)
                                         if (kk < kks)
-                                            umma_bf16_if(one, d, arow + uint64_t(dxi * kPx + kk * kStep), bt + uint64_t(kk * 2),
-                                                      idN, 1u);
-                                }
+                                            umma_bf16_if(one, d, arow + uint64_t(dxi * kPx + kk * kStep),
+                                                         bp + uint64_t(3 * dxi * wt16 + kk * 2), id, 1u);
                             }
                         }
                         umma_commit_if(one, &empty[s]);
                         continue;
                     }
-                    // B of (chunk, dx) group k starts at tile 2 + 5k: [W(+1) W(0) W(-1)];
-                    // with wstream the stage holds this chunk's 17 tiles
-                    const uint64_t b0 = a.wstream
-                                            ? sdesc_k64(sA + size_t(s) * a.stage_bytes + a.wofs) + uint64_t(2 * wt16)
-                                            : sdesc_k64(sW) + uint64_t((2 + 15 * ch) * wt16);
+                    // B of (chunk, dx) group k starts at tile 2 + 5k: [W(+1) W(0) W(-1)]
+                    const uint64_t b0 = wdesc + uint64_t((2 + 15 * ch) * wt16);
 #pragma unroll 1
                     for (int ri = 0; ri < G; ++ri) {
                         // input row G g + ri feeds the slots of rows G g + ri .. + 2
@@ -1356,7 +1335,6 @@ glbm_status launch_band(const void *x0, int c0, const void *x1, int c1, int n, i
 // is then no worse) or the weights and two stages do not fit.
 struct StreamPlan {
     int L, nseg, G, stages;
-    bool stack;          // dy taps stacked along N (weights with zero tiles)
     int ystages;         // up2: staged row pairs (2, or 1 where two do not fit)
     size_t smem;
     bool wstream;        // weights travel with each stage (too many to keep resident)
@@ -1383,23 +1361,15 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     const size_t row1 = stage_rows(1);
     const size_t wplain = size_t(9) * kchunks(cin) * TC_KC * cout * 2;
     p->rowwise = p->groups > 1 && kchunks(cin) > 1 && 1024 + wplain + 2 * kchunks(cin) * row1 <= kStreamSmemLimit;
-    const bool resident = p->rowwise || wplain <= kBandMaxWeights;
-    // 32 output channels: resident weights only (the stacked tiles with
-    // their zero tiles); 64: resident, or nine tiles per stage
-    if (!resident && cout == 32) return false;
-    // stacked tiles with their zero tiles; 64 output channels stack where
-    // those fit with two stages of two rows (and with up2 two staged row
-    // pairs: a single staging buffer serialises the stores with the
-    // epilogue and cost more than stacking saved, d1b 116 -> 133 us), else
-    // the plain tiles; weights carried in each stage stack too (17 tiles per
-    // stage)
-    const size_t wstack = size_t(15 * kchunks(cin) + 2) * cout * TC_KC * 2;
-    const size_t stage2 = stage_rows(2);
     const size_t pair_y = size_t(2) * TC_M * cout * 2;
-    const int ystages = up2 ? 2 : 0;
-    const bool stack = cout == 32 || !resident || p->rowwise || 1024 + wstack + ystages * pair_y + 2 * stage2 <= 221 * 1024;
-    const size_t staged = size_t(ystages) * pair_y;
-    const size_t wbytes = !resident ? 0 : stack && !p->rowwise ? wstack : wplain;
+    // up2: two staged row pairs (one serialises the stores with the epilogue)
+    const size_t staged = up2 ? 2 * pair_y : 0;
+    // 32 output channels: resident weights only, with the zero tiles; 64:
+    // resident where four stages of two rows fit beside them, or nine tiles per stage
+    const bool resident = cout == 32 ? wplain <= kBandMaxWeights
+                                     : p->rowwise || 1024 + wplain + staged + 4 * stage_rows(2) <= kStreamSmemLimit;
+    if (wplain > kBandMaxWeights && (cout == 32 || up2)) return false;
+    const size_t wbytes = !resident ? 0 : cout == 32 ? size_t(15 * kchunks(cin) + 2) * cout * TC_KC * 2 : wplain;
     const long long units = (long long)n * ((w + TC_M - 1) / TC_M) * p->groups;
     if (units > nsm) return false;
     int segs = int(nsm / units);
@@ -1413,12 +1383,10 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     p->L = l;
     p->nseg = (h + l - 1) / l;
     p->wstream = !resident;
-    p->stack = stack;
-    p->ystages = ystages;
+    p->ystages = up2 ? 2 : 0;
     // the tallest group that leaves three stages: 6, 4 or 2 rows with 32
-    // output channels; 2 rows with 64 (the 4 pair slots need two groups of
-    // slack), 4 when each stage carries the weights (amortised over 4 rows)
-    const int g0 = cout == 32 ? 6 : (resident || stack ? 2 : 4);
+    // output channels; 2 rows with 64 (the 4 pair slots need two groups of slack)
+    const int g0 = cout == 32 ? 6 : 2;
     if (p->rowwise) {
         p->G = 2;
         p->stages = std::min(int((kStreamSmemLimit - 1024 - wbytes) / row1), ST_SMAX);
@@ -1429,7 +1397,7 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     }
     for (int g = g0; g >= 2; g -= 2) {
         const size_t arows = stage_rows(g);
-        const size_t stage = arows + (resident ? 0 : size_t(stack ? 17 : 9) * cout * TC_KC * 2);
+        const size_t stage = arows + (resident ? 0 : size_t(9) * cout * TC_KC * 2);
         if (1024 + wbytes + staged + 2 * stage > kStreamSmemLimit) continue;
         const size_t room = kStreamSmemLimit - 1024 - wbytes - staged;
         int st = int(room / stage);
@@ -1510,11 +1478,10 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
         mY0 = mA0;  // unused
         mY1 = mA0;
     }
-    const auto kern =
-        cout == 64 ? (pl.stack ? (G == 4 ? k_tc_conv_stream<4, 64, true> : k_tc_conv_stream<2, 64, true>)
-                               : (G == 4 ? k_tc_conv_stream<4, 64, false> : k_tc_conv_stream<2, 64, false>))
-                   : (G == 6 ? k_tc_conv_stream<6, 32, true>
-                             : (G == 4 ? k_tc_conv_stream<4, 32, true> : k_tc_conv_stream<2, 32, true>));
+    const auto kern = cout == 64 ? k_tc_conv_stream<2, 64>
+                      : G == 6   ? k_tc_conv_stream<6, 32>
+                      : G == 4   ? k_tc_conv_stream<4, 32>
+                                 : k_tc_conv_stream<2, 32>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv: shared memory attribute (streaming)");
     const unsigned grid = unsigned((long long)n * a.nbx * pl.groups * nseg);
