@@ -480,16 +480,21 @@ inline Pair2 make_pair2(const Phys<float> &p) {
     return c;
 }
 
-// node_velocity for a pair.
-template <bool FORCH>
+// node_velocity for a pair.  SCALED: populations as stored in FP16, g S with S
+// a power of two.  A power of two commutes with every rounding, so it enters
+// where the sums leave the populations (drho, 1 / rho) and where the update
+// returns to them (rho in collide_small2): 3 multiplications instead of one per
+// population on the way in and on the way out, and the same bits (2048^2 FP16
+// 27.0 -> 24.9 us a step).
+template <bool FORCH, bool SCALED = false>
 __device__ __forceinline__ void node_velocity2(const f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c, f2 &drho,
                                                f2 &rho, f2 &ux, f2 &uy) {
     drho = radd(radd(radd(g[0], radd(g[1], g[3])), radd(g[2], g[4])), radd(radd(g[5], g[7]), radd(g[6], g[8])));
+    rho = radd(c.one, SCALED ? rmul(drho, c.inv_s) : drho);
     const f2 d57 = rsub(g[5], g[7]), d86 = rsub(g[8], g[6]);
     const f2 mx = radd(radd(rsub(g[1], g[3]), d57), d86);
     const f2 my = rsub(radd(rsub(g[2], g[4]), d57), d86);
-    rho = radd(c.one, drho);
-    const f2 ir = rrcp(rho);
+    const f2 ir = SCALED ? rmul(rrcp(rho), c.inv_s) : rrcp(rho);
     const f2 vx = rfma(mx, ir, rmul(eps, c.hgx)), vy = rfma(my, ir, rmul(eps, c.hgy));
     f2 den;
     if (FORCH) {
@@ -539,11 +544,12 @@ __device__ __forceinline__ void collide2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, 
     g[0] = radd(g[0], radd(radd(l1, l2), radd(l5, l6)));
 }
 
-// collide_small for a pair.
-template <bool FORCH>
+// collide_small for a pair (SCALED: drho and rho carry the scale).
+template <bool FORCH, bool SCALED>
 __device__ __forceinline__ void collide_small2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c) {
     f2 drho, rho, ux, uy;
-    node_velocity2<FORCH>(g, alpha, eps, beta, c, drho, rho, ux, uy);
+    node_velocity2<FORCH, SCALED>(g, alpha, eps, beta, c, drho, rho, ux, uy);
+    if (SCALED) rho = rmul(rho, c.scale);
     f2 nFx = rfma(eps, c.ngx, rmul(alpha, ux)), nFy = rfma(eps, c.ngy, rmul(alpha, uy));  // -F
     const f2 uu = rfma(ux, ux, rmul(uy, uy));
     if (FORCH) {
@@ -921,7 +927,7 @@ k_step(const T *__restrict__ src, T *__restrict__ dst, const typename Store<T>::
 // FP32 runs best at 12 warps per SM (fewer DRAM streams), 16-bit at 16;
 // cp.async.cg, a barrier per row and 128-thread blocks were slower.
 // 4096^2, us a step: FP32 195 -> 107, BF16 112 -> 86; 2048^2: FP32 49.6 -> 28.1,
-// FP16 29.6 -> 27.0.  FP32 then moves 0.9 of the copy bandwidth.
+// FP16 29.6 -> 24.9.  FP32 then moves 0.9 of the copy bandwidth.
 //
 // Both steps round, and draw their stochastic-rounding words, exactly as the
 // one-step kernel does, so the results are its bits.
@@ -963,25 +969,18 @@ __host__ __device__ constexpr LcgStep lcg_step(int n) {
 }
 
 // Stored form of 4 nodes' population I of 16-bit storage, stochastically
-// rounded with states 2I+1 and 2I+2 of the LCG as in step_body.
+// rounded with states 2I+1 and 2I+2 of the LCG as in step_body (the FP16 scale
+// is in the values).
 template <typename T, int I>
-__device__ __forceinline__ uint2 round4(Quad q, f2 scale, uint32_t seed) {
+__device__ __forceinline__ uint2 round4(Quad q, uint32_t seed) {
     constexpr LcgStep s0 = lcg_step(2 * I + 1), s1 = lcg_step(2 * I + 2);
-    if (Store<T>::kScaled) q.p[0] = rmul(q.p[0], scale), q.p[1] = rmul(q.p[1], scale);
     return make_uint2(Store<T>::pack_sr(lo2(q.p[0]), hi2(q.p[0]), seed * s0.a + s0.c),
                       Store<T>::pack_sr(lo2(q.p[1]), hi2(q.p[1]), seed * s1.a + s1.c));
 }
-// Loaded 4 nodes of storage T as pairs.
+// Loaded 4 nodes of storage T as pairs (FP16: with their scale).
 template <typename T>
-__device__ __forceinline__ Quad unpack4(const T (&t)[4], f2 inv_s) {
-    Quad q;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        q.p[k] = mk2(Store<T>::ld(t[2 * k], 1.0f), Store<T>::ld(t[2 * k + 1], 1.0f));
-        if constexpr (Store<T>::kSmall)
-            if (Store<T>::kScaled) q.p[k] = rmul(q.p[k], inv_s);
-    }
-    return q;
+__device__ __forceinline__ Quad unpack4(const T (&t)[4]) {
+    return Quad{{mk2(Store<T>::ld(t[0], 1.0f), Store<T>::ld(t[1], 1.0f)), mk2(Store<T>::ld(t[2], 1.0f), Store<T>::ld(t[3], 1.0f))}};
 }
 
 // x shifts within a strip: RIGHT: node x takes x - 1; else node x takes x + 1.
@@ -1007,7 +1006,7 @@ __device__ __forceinline__ void collide4(Quad (&g)[9], const Quad &a, const Quad
         f2 n[9];
 #pragma unroll
         for (int i = 0; i < 9; ++i) n[i] = g[i].p[k];
-        if constexpr (Store<T>::kSmall) collide_small2<FORCH>(n, a.p[k], e.p[k], b.p[k], c);
+        if constexpr (Store<T>::kSmall) collide_small2<FORCH, Store<T>::kScaled>(n, a.p[k], e.p[k], b.p[k], c);
         else collide2<FORCH>(n, a.p[k], e.p[k], b.p[k], c);
 #pragma unroll
         for (int i = 0; i < 9; ++i) g[i].p[k] = n[i];
@@ -1112,7 +1111,7 @@ __device__ __forceinline__ void march_strip(StripSmem<T, FORCH> &sm, const T *__
             if (FORCH) memcpy(&b, &sm.coef[slot][FORCH ? 2 : 0][lane], 16);
             Quad f[9];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) f[i] = unpack4<T>(sm.f[i][lane].v, c.inv_s);
+            for (int i = 0; i < 9; ++i) f[i] = unpack4<T>(sm.f[i][lane].v);
             h[0] = f[0], h[2] = f[2], h[4] = f[4];
             h[1] = shift4<true>(f[1]);
             h[3] = shift4<false>(f[3]);
@@ -1126,10 +1125,10 @@ __device__ __forceinline__ void march_strip(StripSmem<T, FORCH> &sm, const T *__
             if constexpr (Store<T>::kSmall) {
                 const uint32_t seed = mix32(uint32_t((long long)rr * nx + x0) ^ ph.step_key);
                 for_pops([&](auto i) {
-                    const uint2 w = round4<T, i.value>(h[i.value], c.scale, seed);
+                    const uint2 w = round4<T, i.value>(h[i.value], seed);
                     T t[4];
                     memcpy(t, &w, 8);
-                    h[i.value] = unpack4<T>(t, c.inv_s);
+                    h[i.value] = unpack4<T>(t);
                 });
             }
             h0 = h[0], h2 = h[2], h4 = h[4];
@@ -1161,7 +1160,7 @@ __device__ __forceinline__ void march_strip(StripSmem<T, FORCH> &sm, const T *__
             for_pops([&](auto i) {
                 T *p = dst + (long long)i.value * geo.plane + n0;
                 if constexpr (Store<T>::kSmall) {
-                    const uint2 w = round4<T, i.value>(g[i.value], c.scale, seed);
+                    const uint2 w = round4<T, i.value>(g[i.value], seed);
                     if (store) __stcs(reinterpret_cast<uint2 *>(p), w);
                 } else {
                     uint4 w;
@@ -1233,10 +1232,10 @@ struct TilePlan {
 // Stored 16-bit form of one node as the one-step kernel with one node per
 // thread rounds it.
 template <typename T, int I>
-__device__ __forceinline__ T round1(float v, float scale, uint32_t hash) {
+__device__ __forceinline__ T round1(float v, uint32_t hash) {
     uint32_t r = (hash ^ (uint32_t(I >> 1) * 0x9E3779B9u)) * 0x2C1B3C6Du;
     r ^= r >> 15;
-    return Store<T>::st_sr(v, scale, (I & 1) ? (r >> 16) : r);
+    return Store<T>::st_sr(v, 1.0f, (I & 1) ? (r >> 16) : r);
 }
 
 template <typename T, bool WALLS, bool FORCH, bool ODD>
@@ -1318,7 +1317,7 @@ k_tile(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__
             } else {
                 ld16<T, 4>(p + col[0], t);
             }
-            f[i] = unpack4<T>(t, c.inv_s);
+            f[i] = unpack4<T>(t);
         }
         g[0] = f[0], g[2] = f[2], g[4] = f[4];
         g[1] = right(f[1]), g[3] = left(f[3]);
@@ -1345,12 +1344,12 @@ k_tile(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__
                         const Quad &q = g[i.value];
                         const float v[4] = {lo2(q.p[0]), hi2(q.p[0]), lo2(q.p[1]), hi2(q.p[1])};
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) stored[i.value][k] = round1<T, i.value>(v[k], ph.scale, hash[k]);
+                        for (int k = 0; k < 4; ++k) stored[i.value][k] = round1<T, i.value>(v[k], hash[k]);
                     });
                 } else {
                     const uint32_t seed = mix32(uint32_t(base + col[0]) ^ key);
                     for_pops([&](auto i) {
-                        const uint2 w = round4<T, i.value>(g[i.value], c.scale, seed);
+                        const uint2 w = round4<T, i.value>(g[i.value], seed);
                         memcpy(stored[i.value], &w, 8);
                     });
                 }
@@ -1375,7 +1374,7 @@ k_tile(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__
             }
             if constexpr (Store<T>::kSmall) {
 #pragma unroll
-                for (int i = 0; i < 9; ++i) g[i] = unpack4<T>(stored[i], c.inv_s);
+                for (int i = 0; i < 9; ++i) g[i] = unpack4<T>(stored[i]);
             }
             // slots: population set {2, 5, 6 | 4, 7, 8}, row + 1, lane
             float4 *buf = tile_smem + (s & 1) * 6 * (R + 2) * Q + qx;
