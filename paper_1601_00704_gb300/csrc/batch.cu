@@ -369,8 +369,8 @@ glbm_status bfail(glbm_batch *h, glbm_status s, const char *fmt, ...) {
     } while (0)
 
 // Rows of a segment of the two-step kernel: at least 4 (the table's size
-// counts on it), at most 32 (4 waves of the 24-medium sweep).
-constexpr int kBatchMinRows = 4, kBatchRows = 32;
+// counts on it), at most 64.
+constexpr int kBatchMinRows = 4, kBatchRows = 64;
 
 int vec_of(const glbm_batch *h) { return h->elem == 2 ? 4 : 4; }
 
@@ -421,20 +421,37 @@ glbm_status build_table(glbm_batch *h) {
             for (int bx = 0; bx < md.bpr; ++bx) tiles.push_back({m, y, bx, 0});
         md.ntiles = int(tiles.size()) - md.tile0;
     }
-    // segments of the two-step kernel: as long as one wave of resident warps
-    // allows, at most kBatchRows (beyond, several waves even out the media)
+    // segments of the two-step kernel.  Every segment takes its rows and the two
+    // it repeats, and a wave of resident warps lasts as long as its longest
+    // one, so the length is that of the least waves x (rows + 2): 24 media of
+    // 64 to 1024 nodes, FP32, us a step: 32 rows (1.16 waves) 64.8, 40 (0.93)
+    // 48.8, 20 (1.83) 51.0, 64 (0.60) 71.5
     std::vector<BSeg> segs;
-    long long nodes = 0, strip_rows = 0;
-    for (int m : act) {
-        nodes += (long long)h->med[m].nx * h->med[m].ny;
-        strip_rows += (long long)((h->med[m].nx + kStripCols - 1) / kStripCols) * h->med[m].ny;
-    }
+    long long nodes = 0;
+    for (int m : act) nodes += (long long)h->med[m].nx * h->med[m].ny;
     if (nodes >= kPairNodes) {
         const long long slots = (long long)h->nsm * (h->elem == 2 ? kPairWarps<__half> : kPairWarps<float>);
-        const int rows = int(std::min<long long>(kBatchRows, std::max<long long>(kBatchMinRows, (strip_rows + slots - 1) / slots)));
+        auto len_of = [](int ny, int rows) {  // of a medium's segments, even ones of at most `rows`
+            const int per = (ny + rows - 1) / rows;
+            return (ny + per - 1) / per;
+        };
+        int rows = kBatchMinRows;
+        long long least = -1;
+        for (int r = kBatchMinRows; r <= kBatchRows; ++r) {
+            long long count = 0;
+            int longest = 0;
+            for (int m : act) {
+                const BMed &md = h->med[m];
+                const int len = len_of(md.ny, r);
+                count += (long long)((md.ny + len - 1) / len) * ((md.nx + kStripCols - 1) / kStripCols);
+                longest = std::max(longest, len);
+            }
+            const long long cost = (count + slots - 1) / slots * (longest + 2);
+            if (least < 0 || cost < least) least = cost, rows = r;
+        }
         for (int m : act) {
             const BMed &md = h->med[m];
-            const int per = (md.ny + rows - 1) / rows, len = (md.ny + per - 1) / per;
+            const int len = len_of(md.ny, rows);
             for (int y = 0; y < md.ny; y += len)
                 for (int x = 0; x < md.nx; x += kStripCols) segs.push_back({m, x, y, std::min(y + len, md.ny)});
         }
