@@ -237,15 +237,15 @@ def source_hash():
     return h.hexdigest()[:16]
 
 
-def ncu_traffic(storage, nx, ny):
+def ncu_traffic(storage, nx, ny, kernel):
     """DRAM bytes per launch of the step kernel from the committed ncu summary,
     scaled to this lattice; None if absent or taken from other source code."""
-    path = os.path.join(ROOT, "profiles", f"k_step_{storage}.md")
+    path = os.path.join(ROOT, "profiles", f"{kernel}_{storage}.md")
     if not os.path.exists(path):
         return None
     text = open(path).read()
     m_src = re.search(r"source_sha256_16:\s*([0-9a-f]{16})", text)
-    m_b = re.search(r"dram_bytes_per_node_update:\s*([0-9.eE+-]+)", text)
+    m_b = re.search(r"dram_bytes_per_node_(?:update|launch):\s*([0-9.eE+-]+)", text)
     if not (m_src and m_b) or m_src.group(1) != source_hash():
         return None
     return float(m_b.group(1)) * nx * ny
@@ -658,11 +658,12 @@ def run_ours(a, world, rank, local):
     bpu = bytes_per_update(a.storage, launches, a.chunk * a.steps)
     per_launch_s = ms * 1e-3 / launches
     achieved = bpu * N * a.chunk * a.steps / (ms * 1e-3) / 1e9
+    pairs = launches * 3 < a.chunk * a.steps * 2
     peak, peak_kind = peaks()
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-            "frac": achieved / peak, "traffic": ncu_traffic(a.storage, a.nx, a.ny),
+            "frac": achieved / peak, "traffic": ncu_traffic(a.storage, a.nx, a.ny, "k_pair" if pairs else "k_step"),
             "peak_kind": peak_kind, "bytes_per_node_update": bpu,
-            "kernel": f"k_pair<{a.storage}> (two fused pull-stream + collide steps)" if launches * 3 < a.chunk * a.steps * 2
+            "kernel": f"k_pair<{a.storage}> (two fused pull-stream + collide steps)" if pairs
             else f"k_step<{a.storage}> (fused pull-stream + collide)",
             "steps_per_launch": a.chunk * a.steps / launches,
             "launch_us": per_launch_s * 1e6,
