@@ -1329,8 +1329,9 @@ glbm_status launch_band(const void *x0, int c0, const void *x1, int c1, int n, i
     return e == cudaSuccess ? GLBM_OK : tccuda(e, "nn_tc_conv launch (band)");
 }
 
-// Streaming plan for a 3x3 layer with 32 output channels: one CTA per
-// (image, 128-pixel strip, segment of L output rows), at most one CTA per SM;
+// Streaming plan for a 3x3 layer with 32, 64 or (grouped) more output channels:
+// one CTA per (image, group, 128-pixel strip, segment of L output rows), at most
+// one CTA per SM;
 // false where the segments would be short (the band kernel's edge overhead
 // is then no worse) or the weights and two stages do not fit.
 struct StreamPlan {
