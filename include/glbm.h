@@ -563,13 +563,13 @@ void glbm_nn_tc_debug_starve(int stage);
 /* Choice of tensor-core convolution kernel for glbm_nn_tc_conv and
  * glbm_nn_tc_conv_fused (process-wide):
  * 0 (default) = per layer: 3x3 layers with BF16 output, rows of >= 128
- * pixels and 32, 64, 128, 192 or 256 output channels (in groups of 64) where
- * one CTA per (image, 128-pixel strip, group) leaves segments of >= 16 rows
- * per SM run the streaming kernel (each
- * CTA walks down its strip, each input row multiplied once into a ring of
- * row accumulators in tensor memory; the three vertical taps stacked into
- * one MMA of 96 or 192 columns where the weights fit shared memory with
- * their zero tiles; 64-channel layers whose weights exceed it take them
+ * pixels and 32 or 64 output channels, or 128, 192 or 256 (in groups of 64) of
+ * at most 128 input channels, run the streaming kernel where one CTA per
+ * (image, 128-pixel strip, group) leaves segments of >= 16 rows (groups: >= 4)
+ * per SM (each CTA walks down its strip, each input row multiplied once into a
+ * ring of row accumulators in tensor memory; the three vertical taps stacked
+ * into one MMA of 96 or 192 columns; groups add up in the order of the tile
+ * kernel and have its bits; 64-channel layers whose weights exceed shared memory take them
  * along with each stage); other such layers whose weights fit shared memory
  * run the band kernel (weights resident, each band's halo loaded once per
  * 32-channel chunk; stacked taps for 32 output channels); the rest run the

@@ -578,13 +578,16 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // Layers with 128, 192 or 256 output channels run as groups of 64, one CTA per
 // group, strip and segment: a ring of 128-column slots would hold only two row
 // pairs, and reading the input once per group from L2 costs less than the tile
-// kernel's nine loads of every pixel.  Where a group's weights stay resident
-// beside two input rows (32 to 128 input channels) a stage holds one row of
-// one chunk, and once a row's chunks are there they are multiplied tap by tap
-// (rowwise).  Every output is then summed in the tile kernel's order and has
-// its bits: an early layer of other rounding would move a whole network's
-// BF16 output by 1 %.  Rows whose three slots wrap the ring take two MMAs of
-// 64 and 128 columns, so no zero tiles are needed.
+// kernel's nine loads of every pixel.  A group's weights stay resident beside
+// two input rows, which limits it to 128 input channels.  A stage holds one row
+// of one chunk, and once a row's chunks are there they are multiplied tap by tap
+// (rowwise; a single chunk needs no such order).  Every output is then summed in
+// the tile kernel's order and has its bits: a layer of other rounding would
+// move a whole network's BF16 output by up to 1 %.  Wider inputs therefore stay
+// on the tile kernel: with weights travelling chunk by chunk 256 -> 128 takes 107 us
+// at 512^2 instead of 191, but sums in another order, and in the right order, 32
+// outputs per CTA beside one input row, 224 us.  Rows whose three slots wrap
+// the ring take two MMAs of 64 and 128 columns, so no zero tiles are needed.
 //
 // Input rows lie in shared memory as [row][130 pixels][32 channels] in the
 // 64-byte swizzle: the A operand of a tap starts dx pixels (64 dx bytes) in,
@@ -594,8 +597,8 @@ k_tc_conv_band(const __grid_constant__ CUtensorMap mapA0, const __grid_constant_
 // that descriptors stay in uniform registers, and counts its ring position
 // instead of dividing 64-bit stage numbers.
 // us before (16-byte pieces, divisions, one-lane branch, zero tiles) / now, tile
-// kernel in brackets: 512^2 64 -> 128 48 / 46 (78), 128 -> 128 92 / 70 (117),
-// 256 -> 128 158 / 105 (192); 1024^2 128 -> 128 326 / 240 (375), 64 -> 64
+// kernel in brackets: 512^2 64 -> 128 48 / 46 (78), 128 -> 128 92 / 70 (117);
+// 1024^2 128 -> 128 326 / 240 (375), 64 -> 64
 // 85 / 68, 192 -> 64 210 / 154; 2048^2 32 -> 32 137 / 103, 96 -> 32 310 / 236.
 // With up2 the epilogue writes the
 // output 2x nearest-upsampled by TMA stores from a staged row pair.
@@ -1345,7 +1348,8 @@ struct StreamPlan {
     bool rowwise;        // stages of one row; every output summed in the tile kernel's order
 };
 
-// grouped: cout may be 128, 192 or 256, split into groups of 64.
+// grouped: cout may be 128, 192 or 256, split into groups of 64 whose outputs
+// have the tile kernel's bits.
 bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p, bool up2 = false,
                  bool grouped = false) {
     if (w < TC_M || g_tc_variant == 1 || g_tc_variant == 3 || g_tc_variant == 4) return false;
@@ -1355,13 +1359,14 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
         cout = 64;
     }
     if (cout != 32 && cout != 64) return false;
-    // groups whose weights stay resident beside two rows of input sum in the
-    // tile kernel's order (one chunk: they do so anyway)
     constexpr size_t kStreamSmemLimit = 221 * 1024;  // the 227 KB per block less ~5 KB of static shared memory
     auto stage_rows = [](int g) { return (size_t(g) * BAND_PX * TC_KC * 2 + 1023) / 1024 * 1024; };  // bytes
     const size_t row1 = stage_rows(1);
     const size_t wplain = size_t(9) * kchunks(cin) * TC_KC * cout * 2;
-    p->rowwise = p->groups > 1 && kchunks(cin) > 1 && 1024 + wplain + 2 * kchunks(cin) * row1 <= kStreamSmemLimit;
+    // groups keep the tile kernel's order of summation (one chunk: they do so
+    // anyway), for which a group's weights lie beside two rows of input
+    if (p->groups > 1 && 1024 + wplain + 2 * kchunks(cin) * row1 > kStreamSmemLimit) return false;
+    p->rowwise = p->groups > 1 && kchunks(cin) > 1;
     const size_t pair_y = size_t(2) * TC_M * cout * 2;
     // up2: two staged row pairs (one serialises the stores with the epilogue)
     const size_t staged = up2 ? 2 * pair_y : 0;
@@ -1376,10 +1381,10 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     int segs = int(nsm / units);
     int l = (h + segs - 1) / segs;
     l += l & 1;  // even: row pairs never straddle two segments
-    // short segments repeat their halo rows: from 16 rows on, or from 4 where the
-    // bits are the tile kernel's whichever runs (256^2 128 -> 128 channels, 8
+    // short segments repeat their halo rows: from 16 rows on, or from 4 for groups,
+    // whose bits are the tile kernel's whichever runs (256^2 128 -> 128 channels, 8
     // rows: 37 us there, 31 here; 128 x 256, 4 rows: 25 / 22; 128^2, 2 rows: equal)
-    const int least = p->rowwise || (p->groups > 1 && kchunks(cin) == 1) ? 4 : 16;
+    const int least = p->groups > 1 ? 4 : 16;
     if (l < (g_tc_variant == 5 ? 2 : least)) return false;
     p->L = l;
     p->nseg = (h + l - 1) / l;
