@@ -616,7 +616,9 @@ struct StreamArgs {
     int groups;  // groups of COUT output channels, one CTA each (1, or cout / 64)
     int rowwise;  // 1 (64 channels, stacked): stages of one row, a row's chunks multiplied tap by tap
     int starve;  // test hook: stage number + 1 the first CTA leaves unloaded
-    int kks;               // K steps of 16 channels per chunk: 2, or 1 for a 16-channel input
+    // K steps of 16 channels per chunk: 2, or 1 for a 16-channel input (of 48, 80,
+    // ... channels only the last chunk is half empty, and its loads are zero-filled)
+    int kks;
     uint32_t stage_bytes;
     uint32_t tx_bytes;     // bytes the TMA loads of a stage deliver
     uint32_t wtile;        // bytes of one weight slice (32 rows x 64 B)
@@ -1454,7 +1456,7 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
     a.w = w;
     a.nchunk0 = kchunks(c0);
     a.nchunk = a.nchunk0 + c1 / TC_KC;
-    a.kks = c0 % TC_KC ? 1 : 2;  // 16 input channels: one K step per tap
+    a.kks = a.nchunk == 1 && c0 % TC_KC ? 1 : 2;  // 16 input channels: one K step per tap
     a.nbx = (w + TC_M - 1) / TC_M;
     a.nseg = nseg;
     a.groups = pl.groups;
