@@ -332,11 +332,13 @@ glbm_status launch_tile_t(glbm *h, int n, long long clock_off) {
     for (int i = 0; i < n; ++i) refused = injected_failure() || refused;  // the test hook counts time steps
     if (refused) return fail(h, GLBM_ECUDA, "step launch: injected failure (test hook)");
     const int Q = 1 << pl.q_log2;
-    const size_t smem = sizeof(float4) * 2 * 6 * (pl.rows + 2) * Q;
+    const size_t smem = tile_bytes(pl.rows, Q);
+    // the limit belongs to the function, for every handle and thread: always the
+    // most that any plan takes, so that no launch is refused what another set
     cudaError_t err = cudaSuccess;
     if (smem > 48 * 1024)
         err = cudaFuncSetAttribute(k_tile<T, WALLS, FORCH, ODD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   int(smem));
+                                   int(kTileSmem));
     if (err == cudaSuccess)
         err = launch_kernel_smem(
             k_tile<T, WALLS, FORCH, ODD>, dim3(unsigned(pl.nx_tiles) * unsigned(pl.ny_tiles)),

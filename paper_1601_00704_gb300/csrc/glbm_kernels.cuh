@@ -1220,6 +1220,12 @@ k_pair(const T *__restrict__ src, T *__restrict__ dst, const float *__restrict__
 // of 4 for whole vectors, per node otherwise), so the results are its bits.
 // ---------------------------------------------------------------------------
 constexpr int kTileThreads = 640;  // most per block: 96 registers a thread
+constexpr int kTileQ = 16;         // most lanes of a row
+// Shared memory of a tile of `rows` rows (with halo) and q lanes: two buffers of
+// six populations, with a row beyond each edge; and the most of any plan.
+constexpr size_t tile_bytes(int rows, int q) { return sizeof(float4) * 2 * 6 * size_t(rows + 2) * size_t(q); }
+constexpr size_t kTileSmem = tile_bytes(kTileThreads / kTileQ, kTileQ);
+static_assert(tile_bytes(kTileThreads / 8, 8) <= kTileSmem, "narrow tiles");
 
 struct TilePlan {
     int steps;     // T: most steps per launch; 0: not used
