@@ -1235,8 +1235,9 @@ bool map_act_band(CUtensorMap *m, const void *ptr, int c, int w, int h, int n, i
 
 // dynamic shared memory budget: the 227 KB opt-in limit less room for the
 // kernels' static shared memory
-constexpr size_t kSmemLimit = 226 * 1024;
 constexpr size_t kBandMaxWeights = 80 * 1024;  // larger weight sets: tile kernel
+// band and streaming kernels: the 227 KB per block less ~5 KB of static shared memory
+constexpr size_t kStreamSmemLimit = 221 * 1024;
 // 32-channel K chunks of c input channels (a last partial chunk of 16: the
 // loads fill its missing channels with zeros)
 inline int kchunks(int c) { return (c + TC_KC - 1) / TC_KC; }
@@ -1322,7 +1323,7 @@ glbm_status launch_band(const void *x0, int c0, const void *x1, int c1, int n, i
     a.relu = relu ? 1 : 0;
     a.err = err;
     if (a.tmem_cols > 512) return tcfail(GLBM_EINVAL, "nn_tc_conv: band accumulators exceed tensor memory");
-    cudaError_t e = cudaFuncSetAttribute(k_tc_conv_band, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(k_tc_conv_band, kStreamSmemLimit);
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv: shared memory attribute (band)");
     int dev = 0, nsm = 0;
     e = cudaGetDevice(&dev);
@@ -1361,7 +1362,6 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
         cout = 64;
     }
     if (cout != 32 && cout != 64) return false;
-    constexpr size_t kStreamSmemLimit = 221 * 1024;  // the 227 KB per block less ~5 KB of static shared memory
     auto stage_rows = [](int g) { return (size_t(g) * BAND_PX * TC_KC * 2 + 1023) / 1024 * 1024; };  // bytes
     const size_t row1 = stage_rows(1);
     const size_t wplain = size_t(9) * kchunks(cin) * TC_KC * cout * 2;
@@ -1490,7 +1490,7 @@ glbm_status launch_stream(const void *x0, int c0, const void *x1, int c1, int n,
                       : G == 6   ? k_tc_conv_stream<6, 32>
                       : G == 4   ? k_tc_conv_stream<4, 32>
                                  : k_tc_conv_stream<2, 32>;
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(kern, kStreamSmemLimit);
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv: shared memory attribute (streaming)");
     const unsigned grid = unsigned((long long)n * a.nbx * pl.groups * nseg);
     kern<<<grid, ST_THREADS, smem, st>>>(mA0, mA1, mB, mY0, mY1, a);
@@ -1593,7 +1593,7 @@ extern "C" glbm_status glbm_nn_tc_conv(const void *x0, int c0, const void *x1, i
     const size_t smem = 1024 + size_t(ring) * (size_t(mt) * TC_STAGE_A + size_t(cout) * TC_KC * 2);
     const auto kern = mt == 2 ? (deep ? k_tc_conv<2, TC_STAGES_DEEP> : k_tc_conv<2, TC_STAGES>)
                               : (deep ? k_tc_conv<1, TC_STAGES_DEEP> : k_tc_conv<1, TC_STAGES>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    cudaError_t e = allow_smem(kern, kSmemLimit);
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv: shared memory attribute");
     kern<<<grid, TC_THREADS, smem, static_cast<cudaStream_t>(stream)>>>(mA0, mA1, mB, a);
     e = cudaGetLastError();

@@ -476,7 +476,7 @@ glbm_status launch_wgrad_band(const void *x, int cx, int cin, const void *dy, in
     splits = (a.units + a.units_per_cta - 1) / a.units_per_cta;
     // the stages also hold the epilogue's 32 x 32 x 9 FP32 gather
     const size_t smem = 1024 + std::max(size_t(a.stages) * a.stage_bytes, size_t(32 * 32 * 9 * 4));
-    e = cudaFuncSetAttribute(k_tc_wgrad_band, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    e = allow_smem(k_tc_wgrad_band, kSmemLimit);
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv_wgrad: shared memory attribute");
     k_tc_wgrad_band<<<dim3(unsigned(groups), unsigned(splits)), WG_THREADS, smem, stream>>>(mX, mDY, a);
     e = cudaGetLastError();
@@ -532,7 +532,7 @@ extern "C" glbm_status glbm_nn_tc_conv_wgrad(const void *x, int cx, int cin, con
     a.rows_per_cta = int((rows + splits - 1) / splits);
     splits = (rows + a.rows_per_cta - 1) / a.rows_per_cta;
     const size_t smem = 1024 + size_t(WG_STAGES) * a.stage_bytes;
-    e = cudaFuncSetAttribute(k_tc_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+    e = allow_smem(k_tc_wgrad, kSmemLimit);
     if (e != cudaSuccess) return tccuda(e, "nn_tc_conv_wgrad: shared memory attribute");
     k_tc_wgrad<<<dim3(unsigned(mtiles), unsigned(splits)), WG_THREADS, smem, static_cast<cudaStream_t>(stream)>>>(
         mX, mDY, a);

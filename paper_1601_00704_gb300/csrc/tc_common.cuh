@@ -123,6 +123,17 @@ struct RingPos {
     }
 };
 
+// Dynamic shared memory of one block: 227 KB less what the kernels hold statically.
+constexpr size_t kSmemLimit = 226 * 1024;
+// Let launches of `kern` take up to `most` bytes of dynamic shared memory.  The
+// limit belongs to the function, for every thread of the process: `most` is the
+// same at each call of a kernel and at least what any of its launches takes (set
+// to what one launch takes it would refuse another thread's larger one).
+template <typename K>
+inline cudaError_t allow_smem(K kern, size_t most) {
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(most));
+}
+
 // Test hook (glbm_nn_tc_debug_starve): stage number + 1 whose copies the
 // first CTA of the next tensor-core launch leaves unissued, 0 for none.
 inline int take_starve() {

@@ -65,3 +65,54 @@ def test_solvers_of_different_tiles(pkg, storage):
     for a, b in zip(alone, _together(jobs)):
         assert isinstance(b, np.ndarray), b
         assert np.array_equal(a, b)
+
+
+# (kernel, two layers of it: n, h, w, input channels, output channels) that take different amounts of shared memory
+LAYERS = {"streaming": ((1, 600, 256, 32, 64), (1, 600, 256, 64, 64)), "band": ((1, 16, 256, 32, 64), (1, 16, 256, 64, 64)),
+          "tile": ((2, 40, 40, 32, 256), (2, 40, 40, 32, 96)), "weight gradient": ((2, 16, 16, 32, 32), (2, 64, 64, 64, 64))}
+
+
+@pytest.mark.parametrize("kernel", LAYERS)
+def test_layers_of_different_sizes(pkg, kernel):
+    import ctypes as C
+
+    import torch
+    lib = pkg.load()
+
+    def vp(t):
+        return C.c_void_p(t.data_ptr())
+
+    def job(n, h, w, ci, co):
+        g = torch.Generator(device="cuda").manual_seed(ci + co)
+        x = torch.randn((n, h, w, ci), generator=g, device="cuda").to(torch.bfloat16)
+        dy = torch.randn((n, h, w, co), generator=g, device="cuda").to(torch.bfloat16)
+        wt = torch.randn((9, co, ci), generator=g, device="cuda").to(torch.bfloat16)
+        b = torch.randn(co, generator=g, device="cuda")
+        y = torch.empty((n, h, w, co), dtype=torch.bfloat16, device="cuda")
+        dw = torch.zeros((co, ci, 3, 3), device="cuda")
+        err = torch.zeros(1, dtype=torch.int32, device="cuda")
+        stream = torch.cuda.Stream()
+        st = C.c_void_p(stream.cuda_stream)
+        torch.cuda.synchronize()
+
+        def layer():
+            torch.cuda.set_device(0)  # the thread's CUDA context, which encoding a tensor map needs
+            torch.cuda.synchronize()
+            for _ in range(1500):
+                if kernel == "weight gradient":
+                    rc = lib.glbm_nn_tc_conv_wgrad(vp(x), ci, ci, vp(dy), co, co, n, h, w, 3, vp(dw), vp(err), st)
+                else:
+                    rc = lib.glbm_nn_tc_conv(vp(x), ci, None, 0, n, h, w, 3, vp(wt), vp(b), co, vp(y), co, 1, 0, 0,
+                                             vp(err), st)
+                if rc != 0:
+                    raise pkg.GLBMError(rc, lib.glbm_last_error(None).decode())
+            stream.synchronize()
+            assert int(err) == 0
+            return y.clone()
+        return layer
+
+    jobs = [job(*shape) for shape in LAYERS[kernel]]
+    alone = [j() for j in jobs]
+    for a, b in zip(alone, _together(jobs)):
+        assert isinstance(b, torch.Tensor), b
+        assert kernel == "weight gradient" or torch.equal(a, b)
