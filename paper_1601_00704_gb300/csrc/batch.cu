@@ -333,6 +333,7 @@ struct glbm_batch {
     long long tstep = 0;
     bool reduced = false;
     double gx = 0.0, gy = 0.0;
+    OddConstants<float> odd{};
     int threads = 128, order = 0;
     bool persistent = false;  // one cooperative launch per chunk (k_batch_persist)
     int patience = 1;         // consecutive passing checks for a medium to converge
@@ -481,6 +482,7 @@ Phys<float> batch_phys(const glbm_batch *h) {
     ph.inv_scale = 1.0f;
     ph.step_key = 0;
     ph.sr = 1;
+    ph.odd = h->odd;
     return ph;
 }
 
@@ -730,6 +732,7 @@ glbm_status glbm_batch_create(int count, const int *nx, const int *ny, double ta
     if (!h) return bfail(nullptr, GLBM_ENOMEM, "glbm_batch_create: out of host memory");
     h->count = count;
     h->tau = tau;
+    if (storage == GLBM_F32) h->odd = odd_constants(float(1.0 / tau));
     h->storage = storage;
     h->flags = flags;
     h->elem = storage == GLBM_F32 ? 4 : 2;

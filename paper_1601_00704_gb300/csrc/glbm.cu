@@ -69,6 +69,7 @@ struct glbm {
     glbm_guard::Table guards; // every device buffer above, with its guard zones
     bool has_medium = false, forch = false, reduced = false;
     double feps_mode = 0.0, gx = 0.0, gy = 0.0;
+    OddConstants<double> odd{};  // of the collision's type
     double scale = 1.0;       // FP16 storage scale S (stored = g*S)
     bool sr = true;           // 16-bit storage: stochastic rounding
     bool at_rest = false;     // state is f_eq(1, 0) (zero deviations)
@@ -144,6 +145,7 @@ Phys<R> make_phys(const glbm *h) {
     p.tstep = uint32_t(h->tstep);
     p.sr = h->sr ? 1 : 0;
     p.seed = h->seed;
+    p.odd = {R(h->odd.c), R(h->odd.a), R(h->odd.b)};
     return p;
 }
 
@@ -668,6 +670,11 @@ glbm_status glbm_create(int nx, int ny, double tau, glbm_storage storage, unsign
     h->elem = storage == GLBM_F64 ? 8 : (storage == GLBM_F32 ? 4 : 2);
     h->celem = storage == GLBM_F64 ? 8 : 4;
     h->sr = !(flags & GLBM_NEAREST16);
+    if (storage == GLBM_F64) h->odd = odd_constants(1.0 / tau);
+    else if (storage == GLBM_F32) {
+        const OddConstants<float> o = odd_constants(float(1.0 / tau));
+        h->odd = {o.c, o.a, o.b};
+    }
     cudaError_t e = cudaGetDevice(&h->dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
     if (e == cudaSuccess) h->tile = plan_tiles(h);
@@ -1233,6 +1240,13 @@ extern "C" glbm_status glbm_step_reduce_noalloc(const float *g_src, float *g_dst
     ph.inv_scale = 1.0f;
     ph.step_key = 0;
     ph.sr = 0;
+    {
+        // a program that steps in a loop passes one tau again and again
+        thread_local float omega = 0.0f;
+        thread_local OddConstants<float> odd{};
+        if (omega != ph.omega) omega = ph.omega, odd = odd_constants(omega);
+        ph.odd = odd;
+    }
     // the status keeps the previous call's values: start it from zero
     cudaError_t e = cudaMemsetAsync(st, 0, sizeof(DevStatus), cs);
     if (e != cudaSuccess) return noalloc_fail(GLBM_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));

@@ -37,6 +37,8 @@
 
 #pragma once
 
+#include "odd_constants.h"
+
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
@@ -197,6 +199,7 @@ struct Phys {
     uint32_t seed = 0;
     uint32_t step_key2 = 0;  // key of the following step, for k_pair
     uint32_t tstep = 0;      // the step itself, for kernels that form several keys
+    OddConstants<R> odd{};   // FP32 and FP64 storage: the odd half's constants
 };
 
 // Stochastic-rounding key of time step t (host and device agree).
@@ -307,15 +310,13 @@ __device__ __forceinline__ void node_velocity(const R (&g)[9], R alpha, R eps, R
 //
 // Operation count: with H = 1.5 u/tau + 3A F, J = 3 u/tau + 3A F and
 // A = 1 - 1/(2 tau) the direction sums of Eqs. 30 and 31 collapse to
-//     even = (3 rho/eps) [ (e.u)(e.H) - (u.H)/3 ],   odd = rho (e.J),
+//     w even = w (3 rho/eps) [ (e.u)(e.H) - (u.H)/3 ],   w odd = w rho (e.J),
 // shared by opposite directions: 106 FP32 operations per node with the mass
 // closure below.  The form before it (separate f_eq and F_i terms, and TwoSum
 // sums of the populations before and after the collision) took 241 and was
 // bound by them where the lattice fits L2: 1024^2 FP32 10.8 -> 8.8 us a step.
-// The factor 3 sits in J, not in the weight, because fl(1/9) is 4x nearer to
-// its value than fl(1/3) or fl(1/6), and F, ten times u in shale, shows it:
-// with 1/6 in the weight the velocity error against FP64 was 5 % larger, as
-// written it is 1 % smaller than the separate terms' (192^2, 200 steps).
+// w rho J is c rho (a u + b F) with constants whose rounding loses no momentum
+// (odd_constants.h); H goes with the same b, so that w (3/eps) becomes 3c/eps.
 template <typename R>
 __device__ __forceinline__ R collide_pair(R &gi, R &gj, R w, R d, R k1, R eu, R eH, R eJ, R q, R we, R wo) {
     const R ev = rmul(we, rfma(eu, eH, -q));
@@ -337,14 +338,14 @@ __device__ __forceinline__ void collide(R (&g)[9], R alpha, R eps, R beta,
     if (FORCH) drag = rfma(beta, rsqrt_(rfma(ux, ux, rmul(uy, uy))), alpha);
     const R Fx = rfma(-drag, ux, rmul(eps, ph.gx));
     const R Fy = rfma(-drag, uy, rmul(eps, ph.gy));
-    const R k1 = R(1) - ph.omega, omH = R(1.5) * ph.omega, omJ = R(3) * ph.omega, A3 = R(3) * ph.A;
-    const R AFx = rmul(A3, Fx), AFy = rmul(A3, Fy);
+    const R k1 = R(1) - ph.omega, omJ = ph.odd.a, omH = R(0.5) * omJ;
+    const R AFx = rmul(ph.odd.b, Fx), AFy = rmul(ph.odd.b, Fy);
     const R Hx = rfma(omH, ux, AFx), Hy = rfma(omH, uy, AFy);
     const R Jx = rfma(omJ, ux, AFx), Jy = rfma(omJ, uy, AFy);
     const R q = rmul(R(1.0 / 3.0), rfma(ux, Hx, rmul(uy, Hy)));
     // weights of the axis class (w = 1/9) and the diagonal class (1/36)
-    const R we1 = rmul(R(1.0 / 3.0), rmul(rrcp(eps), rho)), we2 = rmul(R(0.25), we1);
-    const R wo1 = rmul(wgt<R>(1), rho), wo2 = rmul(R(0.25), wo1);
+    const R we1 = rmul(R(3) * ph.odd.c, rmul(rrcp(eps), rho)), we2 = rmul(R(0.25), we1);
+    const R wo1 = rmul(ph.odd.c, rho), wo2 = rmul(R(0.25), wo1);
     const R w1 = wgt<R>(1), w2 = R(0.25) * wgt<R>(1);
     // Mass closure: the collision conserves each node's mass exactly in
     // arithmetic, but rounding the nine stored populations does not, and the
@@ -352,10 +353,12 @@ __device__ __forceinline__ void collide(R (&g)[9], R alpha, R eps, R beta,
     // steps.  The rest population therefore takes up exactly what the eight
     // moving ones lose, g0* = g0 + sum_i (g_i - g_i*): each difference is of
     // neighbouring densities (exact by Sterbenz's lemma once within a factor
-    // of two), so one rounding per node remains instead of nine.  Measured
-    // against FP64 over 10 000 steps (128^2; Darcy, clear and mixed media) the
-    // velocity and density errors equal those of TwoSum sums, 30x below the
-    // unclosed update's.
+    // of two), so one rounding per node remains instead of nine: errors 30x below
+    // the unclosed update's.  Against FP64, relative to the separate f_eq and F_i
+    // terms with TwoSum sums before and after (geometric means over tau = 0.55 .. 2,
+    // 3000 to 10 000 steps): two-phase media velocity 0.75, density 0.56; clear and
+    // porous blocks velocity 0.79, density 1.02 +- 0.04 (with TwoSum sums 0.92); a
+    // clear channel, where rounding scatters, velocity 0.97, density 0.64.
     const R l1 = collide_pair<R>(g[1], g[3], w1, drho, k1, ux, Hx, Jx, q, we1, wo1);
     const R l2 = collide_pair<R>(g[2], g[4], w1, drho, k1, uy, Hy, Jy, q, we1, wo1);
     const R l5 = collide_pair<R>(g[5], g[7], w2, drho, k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), q, we2, wo2);
@@ -461,7 +464,7 @@ __device__ __forceinline__ f2 rsqrt_(f2 a) { return mk2(rsqrt_(lo2(a)), rsqrt_(h
 // constant bank.
 struct Pair2 {
     f2 one, half, quarter, hgx, hgy, ngx, ngy, k1;
-    f2 omH, omJ, nA3, nthird, third, w1, nw1, w2, nw2;   // 32-bit storage
+    f2 omH, omJ, nA3, nthird, we, wo, nwo, w1, nw1, w2, nw2;  // 32-bit storage
     f2 cA, cO, ncO, w1om, four, cO3, ncA3, cO2, ncA;     // 16-bit storage
     f2 scale, inv_s;
 };
@@ -471,8 +474,9 @@ inline Pair2 make_pair2(const Phys<float> &p) {
     c.one = bc2(1.0f), c.half = bc2(0.5f), c.quarter = bc2(0.25f);
     c.hgx = bc2(0.5f * p.gx), c.hgy = bc2(0.5f * p.gy), c.ngx = bc2(-p.gx), c.ngy = bc2(-p.gy);
     c.k1 = bc2(1.0f - om);
-    c.omH = bc2(1.5f * om), c.omJ = bc2(3.0f * om), c.nA3 = bc2(-(3.0f * p.A));
-    c.nthird = bc2(-(1.0f / 3.0f)), c.third = bc2(1.0f / 3.0f), c.w1 = bc2(w1), c.nw1 = bc2(-w1);
+    c.omH = bc2(0.5f * p.odd.a), c.omJ = bc2(p.odd.a), c.nA3 = bc2(-p.odd.b);
+    c.nthird = bc2(-(1.0f / 3.0f)), c.we = bc2(3.0f * p.odd.c), c.wo = bc2(p.odd.c), c.nwo = bc2(-p.odd.c);
+    c.w1 = bc2(w1), c.nw1 = bc2(-w1);
     c.w2 = bc2(0.25f * w1), c.nw2 = bc2(-0.25f * w1);
     c.cA = bc2(cA), c.ncA = bc2(-cA), c.cO = bc2(cO), c.ncO = bc2(-cO), c.w1om = bc2(w1 * om), c.four = bc2(4.0f);
     c.cO3 = bc2(3.0f * cO), c.ncA3 = bc2(-(3.0f * cA)), c.cO2 = bc2(2.0f * cO);
@@ -532,9 +536,9 @@ __device__ __forceinline__ void collide2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, 
     const f2 Hx = rfma(c.omH, ux, AFx), Hy = rfma(c.omH, uy, AFy);
     const f2 Jx = rfma(c.omJ, ux, AFx), Jy = rfma(c.omJ, uy, AFy);
     const f2 nq = rmul(c.nthird, rfma(ux, Hx, rmul(uy, Hy)));
-    const f2 we1 = rmul(c.third, rmul(rrcp(eps), rho)), we2 = rmul(c.quarter, we1);
-    const f2 wo1 = rmul(c.w1, rho), wo2 = rmul(c.quarter, wo1);
-    const f2 nwo1 = rmul(c.nw1, rho), nwo2 = rmul(c.quarter, nwo1);
+    const f2 we1 = rmul(c.we, rmul(rrcp(eps), rho)), we2 = rmul(c.quarter, we1);
+    const f2 wo1 = rmul(c.wo, rho), wo2 = rmul(c.quarter, wo1);
+    const f2 nwo1 = rmul(c.nwo, rho), nwo2 = rmul(c.quarter, nwo1);
     const f2 l1 = collide_pair2(g[1], g[3], c.w1, c.nw1, drho, c.k1, ux, Hx, Jx, nq, we1, wo1, nwo1);
     const f2 l2 = collide_pair2(g[2], g[4], c.w1, c.nw1, drho, c.k1, uy, Hy, Jy, nq, we1, wo1, nwo1);
     const f2 l5 = collide_pair2(g[5], g[7], c.w2, c.nw2, drho, c.k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), nq, we2,
