@@ -152,7 +152,10 @@ glbm_status glbm_mean_velocity(glbm_t h, double out[2]);
 glbm_status glbm_permeability(glbm_t h, double *kxx);
 
 /* The Eq. 34 velocity field of the last completed step, [ny][nx] FP64 each
- * (recomputed from the pre-step state with the step's own arithmetic). */
+ * (recomputed from the pre-step state with the step's own arithmetic).
+ * GLBM_ESTATE after a glbm_step that failed where that state could not be
+ * restored (a launch advances several steps, and the device was out of memory
+ * or the error persisted). */
 glbm_status glbm_get_velocity(glbm_t h, double *ux, double *uy,
                               int device_ptrs);
 

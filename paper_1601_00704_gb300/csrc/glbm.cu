@@ -58,6 +58,7 @@ struct glbm {
     size_t celem = 4;    // bytes per coefficient
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;         // buffer holding the current state
+    int behind = 1;      // steps by which the other one lies behind it (see settle); 0: neither
     void *coef[3] = {nullptr, nullptr, nullptr};  // alpha, eps, beta
     double *partial = nullptr;
     float *pmax = nullptr;  // 16-bit storage: block maxima of |stored|
@@ -86,7 +87,7 @@ struct glbm {
     int nsm = 0;              // SMs of the device
     TilePlan tile{};          // multi-step tiles of small or odd lattices
     struct Graph {
-        int parity, end_parity;
+        int parity, end_parity, end_behind;
         long long launches, chunk;
         int reduce, test, patience;
         double tol, scale;
@@ -243,6 +244,7 @@ glbm_status launch_step_t(glbm *h, bool reduce, long long clock_off) {
     h->launches++;
     h->tstep++;
     h->cur ^= 1;
+    h->behind = 1;
     return GLBM_OK;
 }
 
@@ -296,6 +298,7 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
     h->launches++;
     h->tstep += 2;
     h->cur ^= 1;
+    h->behind = 2;
     return GLBM_OK;
 }
 
@@ -352,6 +355,7 @@ glbm_status launch_tile_t(glbm *h, int n, long long clock_off) {
     h->launches++;
     h->tstep += n;
     h->cur ^= 1;
+    h->behind = n;
     return GLBM_OK;
 }
 
@@ -452,12 +456,13 @@ glbm_status run_chunk(glbm *h, long long chunk, bool reduce, double tol) {
                 h->launches += g.launches;
                 h->tstep += chunk;
                 h->cur = g.end_parity;
+                h->behind = g.end_behind;
                 if (reduce) h->reduced = true;
                 return GLBM_OK;
             }
         }
         if (h->ngraphs == 8) drop_graphs(h);
-        const int p0 = h->cur;
+        const int p0 = h->cur, b0 = h->behind;
         const long long t0 = h->tstep, l0 = h->launches;
         const bool r0 = h->reduced;
         cudaGraph_t graph = nullptr;
@@ -478,12 +483,13 @@ glbm_status run_chunk(glbm *h, long long chunk, bool reduce, double tol) {
         if (st) {
             (void)cudaGetLastError();  // drop the capture's error state
             h->cur = p0;
+            h->behind = b0;
             h->tstep = t0;
             h->launches = l0;
             h->reduced = r0;
             return st;
         }
-        h->graphs[h->ngraphs++] = {p0, h->cur, h->launches - l0, chunk, int(reduce), test, h->patience, tol, h->scale, exec};
+        h->graphs[h->ngraphs++] = {p0, h->cur, h->behind, h->launches - l0, chunk, int(reduce), test, h->patience, tol, h->scale, exec};
         CU(h, cudaGraphLaunch(exec, h->stream));
         return GLBM_OK;
     }
@@ -493,6 +499,37 @@ glbm_status run_chunk(glbm *h, long long chunk, bool reduce, double tol) {
     // keep the device step counter in step for later graph replays
     if (graph_eligible(h)) return clock_op(h, h->tstep, false);
     return GLBM_OK;
+}
+
+// After a failed chunk the last launch may have advanced several steps, and the
+// velocity export recomputes the last step from the state before it: bring the
+// other buffer from `behind` steps to one step behind, with the same steps
+// once more, one by one, through a buffer allocated for that.
+void settle(glbm *h) {
+    if (h->behind <= 1) return;
+    const int n = h->behind, c = h->cur;
+    const long long t0 = h->tstep, l0 = h->launches;
+    const size_t fbytes = size_t(9) * h->plane * h->elem;
+    void *const current = h->buf[c];
+    h->behind = 0;
+    void *tmp = nullptr;
+    bool ok = cudaMalloc(&tmp, fbytes) == cudaSuccess;
+    if (ok) {
+        h->buf[c] = tmp;
+        h->cur = c ^ 1;
+        h->tstep -= n;
+        for (int i = 1; i < n && ok; ++i) ok = do_step(h, false) == GLBM_OK;
+        if (h->cur == c)
+            ok = ok && cudaMemcpyAsync(h->buf[c ^ 1], tmp, fbytes, cudaMemcpyDeviceToDevice, h->stream) == cudaSuccess;
+        ok = cudaStreamSynchronize(h->stream) == cudaSuccess && ok;
+        cudaFree(tmp);
+        h->buf[c] = current;
+        h->cur = c;
+        h->tstep = t0;
+        h->launches = l0;
+    }
+    (void)cudaGetLastError();
+    h->behind = ok ? 1 : 0;
 }
 
 double pow2_floor(double x) { return std::ldexp(1.0, int(std::floor(std::log2(x)))); }
@@ -742,6 +779,7 @@ glbm_status glbm_set_medium(glbm_t h, const double *eps, const double *K, double
     CU(h, cudaMemsetAsync(h->dclock, 0, sizeof(unsigned), h->stream));
     if (h->forch != (F_eps != 0.0)) drop_graphs(h);  // another kernel instantiation
     h->cur = 0;
+    h->behind = 1;
     h->steps = 0;
     h->tstep = 0;
     h->at_rest = true;
@@ -801,6 +839,7 @@ glbm_status glbm_init_equilibrium(glbm_t h, const double *rho, const double *ux,
         else h->scale = fp16_scale_for(16.0 * (std::fabs(h->gx) + std::fabs(h->gy)));
     }
     h->cur = 0;
+    h->behind = 1;
     init_eq_dispatch(h, d[0], d[1], d[2]);
     if (glbm_status s = launch_error(h)) return s;
     if (glbm_status s = reset_status(h)) return s;
@@ -811,8 +850,8 @@ glbm_status glbm_init_equilibrium(glbm_t h, const double *rho, const double *ux,
     return GLBM_OK;
 }
 
-glbm_status glbm_step(glbm_t h, long long n, double tol, int check_every, long long *steps_done,
-                      int *converged) {
+static glbm_status step(glbm_t h, long long n, double tol, int check_every, long long *steps_done,
+                        int *converged) {
     glbm_trace::Range trace_range("glbm_step");
     if (steps_done) *steps_done = 0;
     if (converged) *converged = 0;
@@ -853,6 +892,18 @@ glbm_status glbm_step(glbm_t h, long long n, double tol, int check_every, long l
     return GLBM_OK;
 }
 
+glbm_status glbm_step(glbm_t h, long long n, double tol, int check_every, long long *steps_done,
+                      int *converged) {
+    const glbm_status st = step(h, n, tol, check_every, steps_done, converged);
+    if (st && h) {
+        char why[sizeof(h->err)];  // settle's own failures are not the caller's
+        memcpy(why, h->err, sizeof(why));
+        settle(h);
+        memcpy(h->err, why, sizeof(why));
+    }
+    return st;
+}
+
 glbm_status glbm_set_convergence(glbm_t h, int patience) {
     if (glbm_status s = check(h)) return s;
     if (patience < 1 || patience > 1000000)
@@ -888,6 +939,8 @@ glbm_status glbm_get_velocity(glbm_t h, double *ux, double *uy, int device_ptrs)
     if (glbm_status s = check(h)) return s;
     if (!ux || !uy) return fail(h, GLBM_EINVAL, "get_velocity: ux and uy are required");
     if (h->steps == 0) return fail(h, GLBM_ESTATE, "get_velocity: no step has completed since the last reset");
+    if (h->behind == 0)
+        return fail(h, GLBM_ESTATE, "get_velocity: the state before the last step was lost in a failed step call");
     double *dbuf = nullptr;
     double *dx = ux, *dy = uy;
     if (!device_ptrs) {
@@ -1084,6 +1137,7 @@ glbm_status glbm_load(glbm_t h, const char *path) {
     if (bool(hd.forch) != h->forch) drop_graphs(h);
     if (hd.gx != h->gx || hd.gy != h->gy || hd.scale != h->scale) drop_graphs(h);
     h->cur = 0;
+    h->behind = 1;
     h->forch = hd.forch;
     h->feps_mode = hd.feps_mode;
     h->at_rest = hd.at_rest;
