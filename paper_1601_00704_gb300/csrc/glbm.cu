@@ -289,7 +289,14 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
     const int segs = std::max(1, h->nsm * kPairWarps<T> / strips);
     const int rows = std::max(2, (h->ny + segs - 1) / segs);
     const dim3 grid(unsigned(strips) * unsigned((h->ny + rows - 1) / rows));
-    const cudaError_t err = launch_kernel_smem(
+    // FP32 kernels that fit 16 blocks per SM by their registers would be given so
+    // much shared memory that L1 no longer holds the rows that neighbouring strips
+    // and segments share (Forchheimer with walls: 2048^2 53 -> 33 us a step, 4096^2
+    // 191 -> 116); 132 KB is what the driver gives the others
+    cudaError_t err = cudaSuccess;
+    if (sizeof(T) == 4)
+        err = cudaFuncSetAttribute(k_pair<T, WALLS, FORCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 58);
+    if (err == cudaSuccess) err = launch_kernel_smem(
         k_pair<T, WALLS, FORCH>, grid, dim3(kPairThreads), sizeof(StripSmem<T, FORCH>), h->stream,
         h->stream != nullptr, static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
         static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
