@@ -85,7 +85,8 @@ struct glbm {
     // non-legacy stream): key = (buffer parity at start, steps, reduce at
     // end, test, tol, FP16 scale)
     int nsm = 0;              // SMs of the device
-    TilePlan tile{};          // multi-step tiles of small or odd lattices
+    TilePlan tile{};          // multi-step tiles of small or odd lattices (steps = 0: not used)
+    bool pairs = false;       // two steps per launch (k_pair)
     struct Graph {
         int parity, end_parity, end_behind;
         long long launches, chunk;
@@ -152,60 +153,158 @@ Phys<R> make_phys(const glbm *h) {
 
 bool injected_failure() { return glbm_injected_failure(); }
 
-// Tile shape for k_tile: the one with the fewest microseconds a step, if that
-// beats the one-step kernel.  A launch takes
-//     A + rounds (blocks in turn on an SM) x T (B + C x warps per scheduler),
-// fitted to 900 launches over lattices of 64^2 to 768^2, tiles of 32 and 64
-// columns and T = 2 .. 12 (median error 5 %): A = 1.85 us launch, loads and
-// stores, B = 0.28 us the latency of a step, C = 0.37 us its issue.  The
-// one-step kernel takes max(1.7, 1.3 + 7e-6 N) us from a graph; on the legacy
-// stream, where nothing is captured, no launch takes less than about 5 us.
-//   FP32, us a step before / after: 128^2 1.74 / 0.97 (T = 8), 256^2 2.22 / 1.33
-//   (T = 4), 512 x 384 2.96 / 2.17, 640^2 5.16 / 3.99, 768^2 5.78 / 5.4;
-//   BF16: 128^2 1.85 / 1.02, 512 x 384 2.57 / 2.18.
-// Above kTileNodes a wave of blocks no longer covers the lattice and the halo
-// is pure loss: 1024^2 8.4 / 8.8.  Odd row lengths keep gaining in FP32, whose
-// one-step kernel loads one node per thread (2221 x 2000: 57.7 / 44.9, best with
-// two blocks per SM that overlap loads and steps); in 16-bit storage rounding
-// node by node dominates and large lattices stay on it (61.4 / 61.9).
-TilePlan plan_tiles(const glbm *h) {
+// Microseconds of a launch, by which the kernel of a lattice is chosen: fitted to
+// some 900 measurements, 2 to 4096 columns (a few of 1e5 and more) and 2e3 to
+// 1.6e7 nodes; median error 5 %.
+//   one step    t0 + block x blocks + node x nodes (blocks of 128 threads, so
+//               that narrow rows cost what wide ones do), and at least `full` where
+//               a launch fills more than half of the SMs' slots and the next one's
+//               blocks have no room beside its own; up to 1.25 times that (odd
+//               rows: 1.45) as the lattice outgrows L2, then its bytes at 6.5 TB/s
+//   k_tile      A + rounds (blocks in turn on an SM) x T (step + warp x warps per
+//               scheduler): launch, loads and stores, latency of a step and its issue
+//   k_pair      2 (rows of a segment + 2) x pair, per wave of warps, or its bytes
+// On the legacy stream nothing is captured, and launches take multiples of 2 us.
+// Forchheimer's square roots lengthen the latency of a step most; node-by-node
+// rounding in odd rows of 16-bit storage doubles its issue.
+struct LaunchCost {
+    double t0, block, node, full, step, warp, pair;
+};
+constexpr LaunchCost kCost[3][2][2] = {
+    // FP32: whole vectors without and with Forchheimer, odd rows likewise
+    {{{1.65, 1.96e-3, 2.15e-6, 5.0, 0.31, 0.39, 1.16}, {2.18, 2.42e-3, 1.92e-6, 5.7, 0.62, 0.45, 1.43}},
+     {{1.47, 0.47e-3, 5.67e-6, 3.0, 0.22, 0.52, 0.0}, {1.44, 0.68e-3, 3.92e-6, 3.1, 0.72, 0.58, 0.0}}},
+    // BF16
+    {{{1.65, 2.33e-3, 2.6e-7, 3.7, 0.35, 0.39, 1.375}, {2.08, 2.82e-3, 2.6e-7, 4.5, 0.77, 0.41, 1.75}},
+     {{1.44, 1.00e-3, 3.9e-6, 3.5, 0.52, 0.78, 0.0}, {1.50, 1.36e-3, 2.3e-6, 3.6, 0.82, 0.89, 0.0}}},
+    // FP16
+    {{{1.92, 2.55e-3, 1.0e-7, 4.5, 0.45, 0.39, 1.375}, {2.33, 3.04e-3, 1.0e-7, 5.4, 1.08, 0.37, 1.75}},
+     {{1.60, 1.10e-3, 3.9e-6, 3.8, 0.69, 0.73, 0.0}, {1.65, 1.48e-3, 2.1e-6, 3.8, 1.27, 0.74, 0.0}}}};
+constexpr double kHbm = 6.5e6;      // bytes a microsecond
+
+double launch_us(const glbm *h, double t) { return h->stream ? t : 2.06 * std::ceil((t + 0.8) / 2.06); }
+
+const LaunchCost &cost_of(const glbm *h) {
+    const int st = h->storage == GLBM_BF16DEV ? 1 : (h->storage == GLBM_F16DEV ? 2 : 0);
+    return kCost[st][h->nx % 4 != 0][h->forch];
+}
+
+// Bytes of a launch: the populations in and out, and the coefficients.
+double launch_bytes(const glbm *h) { return double(h->N) * (18.0 * h->elem + (h->forch ? 12.0 : 8.0)); }
+
+double one_step_us(const glbm *h) {
+    const LaunchCost &c = cost_of(h);
+    const int vec = vec_width(h);
+    const double blocks = double(make_geo(h, vec).bpr) * h->ny;
+    const double busy = double(h->N) / (blocks * kThreads * vec);  // share of threads with nodes
+    const int slots = h->nsm * (h->storage == GLBM_BF16DEV ? kMinBlocks<__nv_bfloat16> : kMinBlocks<float>);
+    const double bytes = launch_bytes(h);
+    double t = c.t0 + c.block * blocks + c.node * double(h->N);
+    if (blocks > slots / 2) t = std::max(t, c.full * std::min(1.0, 1.5 * busy));
+    t *= 1.0 + (vec == 1 ? 0.45 : 0.25) * std::min(1.0, std::max(0.0, (bytes - 60e6) / 60e6));
+    if (bytes > 160e6) t = std::max(t, bytes / kHbm);
+    return t;
+}
+
+TilePlan tile_of(const glbm *h, int T, int q, int R) {
+    TilePlan p;
+    p.steps = T;
+    p.q_log2 = q;
+    p.rows = R;
+    p.hx = (T + 3) / 4 * 4;
+    p.hy = T - 1;
+    const int w = (4 << q) - 2 * p.hx, l = R - 2 * p.hy;
+    p.nx_tiles = (h->nx + w - 1) / w;
+    p.ny_tiles = (h->ny + l - 1) / l;
+    return p;
+}
+
+// us of a launch whose steps take `step` + `warp` per warp and scheduler
+double tile_us(const glbm *h, const TilePlan &p, double step, double warp) {
+    const int Q = 1 << p.q_log2, R = p.rows;
+    const int fit = std::min(65536 / (96 * R * Q), 227 * 1024 / (192 * (R + 2) * Q + 1024));
+    const long long tiles = (long long)p.nx_tiles * p.ny_tiles;
+    const long long per_sm = (tiles + h->nsm - 1) / h->nsm, side = std::min<long long>(per_sm, std::max(1, fit));
+    const long long rounds = (per_sm + side - 1) / side;
+    // rows of the halo drop out as their reach shrinks
+    const double warps = double(side) * R * Q / 128.0 * (R - p.hy) / R;
+    return (h->elem == 2 ? 1.71 : 1.85) + double(rounds) * p.steps * (step + warp * warps);
+}
+
+struct PairPlan {
+    int strips, rows, segs;
+};
+
+// Segments as long as one wave of resident warps allows: the fewest rows are
+// computed twice.
+PairPlan pair_plan(const glbm *h) {
+    const int slots = h->nsm * (h->elem == 2 ? kPairWarps<__half> : kPairWarps<float>);
+    PairPlan p;
+    p.strips = (h->nx + kStripCols - 1) / kStripCols;
+    const int segs = std::max(1, slots / p.strips);
+    p.rows = std::max(2, (h->ny + segs - 1) / segs);
+    p.segs = (h->ny + p.rows - 1) / p.rows;
+    return p;
+}
+
+// us a step
+double pair_us(const glbm *h) {
+    const PairPlan p = pair_plan(h);
+    const int slots = h->nsm * (h->elem == 2 ? kPairWarps<__half> : kPairWarps<float>);
+    const double waves = std::max(1.0, double(p.strips) * p.segs / slots);
+    // a segment from wall to wall repeats no rows
+    const bool periodic = h->flags & GLBM_PERIODIC_Y;
+    const double rows = p.rows + (p.segs == 1 && !periodic ? 0.7 : 2.0);
+    return std::max((periodic ? 0.93 : 1.0) * cost_of(h).pair * rows * waves, launch_bytes(h) / kHbm / 2);
+}
+
+// Which kernel advances the lattice: one step per launch, two (k_pair) or several
+// (k_tile), whichever takes the fewest microseconds a step by the costs above.
+// k_pair is not for FP64 or round-to-nearest, needs whole vectors, and is taken
+// from 1.3 million nodes on; k_tile up to 600 000, and beyond that for FP32 in
+// odd rows, whose one-step kernel loads one node per thread.  us a step, one step /
+// several (the rule before this one, by node count alone, took several throughout):
+//   FP32   128^2 1.74 / 0.92, 512 x 384 2.96 / 2.03, 100 x 3000 8.4 / 3.5,
+//          1021 x 391 5.2 / 5.0 (Forchheimer 5.1 / 6.2), 4096^2 191 / 108
+//   BF16   512 x 384 2.57 / 2.03, 1000 x 500 3.95 / 4.54, 1021 x 587 8.8 / 11.7,
+//          1024 x 1367 8.6 / 10.9, 256 x 5468 15 / 12.4, 4096^2 110 / 87
+// On the legacy stream two steps per launch save half of what a launch there
+// takes beyond its kernel, and k_pair is left only for segments of 6 rows and
+// more where it loses by more than that (1024 x 1367 BF16 11.1 / 12.4,
+// Forchheimer 12.4 / 15.5); shorter ones tie or gain (2044 x 643 10.4 / 10.4,
+// 1160 x 1131 12.5 / 10.4).
+void plan_launches(glbm *h) {
     constexpr long long kTileNodes = 600000;
+    const bool odd = h->nx % 4 != 0, small = h->elem == 2;
+    h->pairs = false;
+    h->tile = TilePlan{};
+    if (h->storage == GLBM_F64 || (small && !h->sr)) return;
+    const double one = one_step_us(h);
+    if (!odd && h->N >= kPairNodes) {
+        const PairPlan p = pair_plan(h);
+        h->pairs = pair_us(h) < one + (h->stream ? 0.0 : 2.0) || (!h->stream && (p.rows < 6 || p.segs == 1));
+        return;
+    }
+    if (h->N > kTileNodes) {
+        if (odd && !small) h->tile = tile_of(h, 4, 4, 20);  // two blocks per SM that overlap loads and steps
+        return;
+    }
+    // the shape by the costs of whole vectors without Forchheimer (others pick
+    // worse ones); two steps do not pay for odd rows' loads one by one where a
+    // block is alone on its SM (1021 x 587 FP32 7.0 / 10.2)
     TilePlan best{};
-    const bool small = h->elem == 2, odd = h->nx % 4 != 0;
-    if (h->storage == GLBM_F64 || (small && !h->sr)) return best;
-    auto shape = [&](int T, int q, int R) {
-        TilePlan p;
-        p.steps = T;
-        p.q_log2 = q;
-        p.rows = R;
-        p.hx = (T + 3) / 4 * 4;
-        p.hy = T - 1;
-        const int w = (4 << q) - 2 * p.hx, l = R - 2 * p.hy;
-        p.nx_tiles = (h->nx + w - 1) / w;
-        p.ny_tiles = (h->ny + l - 1) / l;
-        return p;
-    };
-    if (h->N > kTileNodes) return odd && !small ? shape(4, 4, 20) : best;
-    const double A = small ? 1.71 : 1.85, B = small ? 0.31 : 0.28, C = small ? 0.405 : 0.37;
-    const double launch = h->stream ? 0.0 : 5.0;
-    double least = std::max(launch, std::max(1.7, small ? 1.2 + 7.4e-6 * double(h->N) : 1.3 + 7e-6 * double(h->N)));
+    double least = 1e30;
     for (int T : {2, 3, 4, 6, 8})
-        for (int q : {3, 4}) {
-            const int Q = 1 << q;
-            for (int R = 2 * (T - 1) + 1; R * Q <= kTileThreads; ++R) {
-                if (R * Q % 32) continue;
-                const TilePlan p = shape(T, q, R);
-                const int fit = std::min(65536 / (96 * R * Q), 227 * 1024 / (192 * (R + 2) * Q + 1024));
-                const long long tiles = (long long)p.nx_tiles * p.ny_tiles;
-                const long long per_sm = (tiles + h->nsm - 1) / h->nsm, side = std::min<long long>(per_sm, std::max(1, fit));
-                const long long rounds = (per_sm + side - 1) / side;
-                // rows of the halo drop out as their reach shrinks
-                const double warps = double(side) * R * Q / 128.0 * (R - (T - 1)) / R;
-                const double t = std::max(launch, A + double(rounds) * T * (B + C * warps)) / T;
+        for (int q : {3, 4})
+            for (int R = 2 * (T - 1) + 1; R << q <= kTileThreads; ++R) {
+                if ((R << q) % 32 || (odd && T == 2 && R << q > kTileThreads / 2)) continue;
+                const TilePlan p = tile_of(h, T, q, R);
+                const double l = tile_us(h, p, small ? 0.31 : 0.28, small ? 0.405 : 0.37);
+                const double t = (h->stream ? l : std::max(5.0, l)) / T;
                 if (t < least) least = t, best = p;
             }
-        }
-    return best;
+    const LaunchCost &c = cost_of(h);
+    if (launch_us(h, tile_us(h, best, c.step, c.warp)) / best.steps < launch_us(h, one)) h->tile = best;
 }
 
 int grid_1d(long long N) {
@@ -271,8 +370,7 @@ glbm_status do_step(glbm *h, bool reduce, long long clock_off = -1) {
     return GLBM_EINVAL;
 }
 
-// Two steps in one launch (k_pair), segments as long as one wave of resident
-// warps allows: the fewest rows are computed twice.
+// Two steps in one launch (k_pair).
 template <typename T, bool WALLS, bool FORCH>
 glbm_status launch_pair_t(glbm *h, long long clock_off) {
     const Geo geo = make_geo(h, 4);
@@ -285,10 +383,8 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
     bool refused = injected_failure();
     refused = injected_failure() || refused;
     if (refused) return fail(h, GLBM_ECUDA, "step launch: injected failure (test hook)");
-    const int strips = (h->nx + kStripCols - 1) / kStripCols;
-    const int segs = std::max(1, h->nsm * kPairWarps<T> / strips);
-    const int rows = std::max(2, (h->ny + segs - 1) / segs);
-    const dim3 grid(unsigned(strips) * unsigned((h->ny + rows - 1) / rows));
+    const PairPlan pl = pair_plan(h);
+    const dim3 grid(unsigned(pl.strips) * unsigned(pl.segs));
     // FP32 kernels that fit 16 blocks per SM by their registers would be given so
     // much shared memory that L1 no longer holds the rows that neighbouring strips
     // and segments share (Forchheimer with walls: 2048^2 53 -> 33 us a step, 4096^2
@@ -296,11 +392,12 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
     cudaError_t err = cudaSuccess;
     if (sizeof(T) == 4)
         err = cudaFuncSetAttribute(k_pair<T, WALLS, FORCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 58);
-    if (err == cudaSuccess) err = launch_kernel_smem(
-        k_pair<T, WALLS, FORCH>, grid, dim3(kPairThreads), sizeof(StripSmem<T, FORCH>), h->stream,
-        h->stream != nullptr, static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
-        static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
-        static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), strips, rows);
+    if (err == cudaSuccess)
+        err = launch_kernel_smem(
+            k_pair<T, WALLS, FORCH>, grid, dim3(kPairThreads), sizeof(StripSmem<T, FORCH>), h->stream,
+            h->stream != nullptr, static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
+            static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
+            static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), pl.strips, pl.rows);
     if (err != cudaSuccess) return fail(h, GLBM_ECUDA, "step launch: %s", cudaGetErrorString(err));
     h->launches++;
     h->tstep += 2;
@@ -314,12 +411,6 @@ glbm_status launch_pair(glbm *h, long long co) {
     if (!(h->flags & GLBM_PERIODIC_Y))
         return h->forch ? launch_pair_t<T, true, true>(h, co) : launch_pair_t<T, true, false>(h, co);
     return h->forch ? launch_pair_t<T, false, true>(h, co) : launch_pair_t<T, false, false>(h, co);
-}
-
-// Rows of whole vectors, a storage that k_pair knows (not FP64, not
-// round-to-nearest) and a lattice large enough for it.
-bool pair_eligible(const glbm *h) {
-    return h->nx % 4 == 0 && h->storage != GLBM_F64 && (h->elem == 4 || h->sr) && h->N >= kPairNodes;
 }
 
 glbm_status do_pair(glbm *h, long long clock_off = -1) {
@@ -387,7 +478,7 @@ glbm_status do_tile(glbm *h, int n, long long co) {
 // its own: the velocity export reads the state before it.
 glbm_status do_steps(glbm *h, long long chunk, bool reduce, bool clocked) {
     const long long plain = chunk - (reduce ? 1 : 0);
-    const bool pairs = pair_eligible(h);
+    const bool pairs = h->pairs;
     for (long long s = 0; s < chunk;) {
         const long long co = clocked ? s : -1;
         const int n = pairs ? 2 : int(std::min<long long>(h->tile.steps, plain - s));
@@ -721,7 +812,7 @@ glbm_status glbm_create(int nx, int ny, double tau, glbm_storage storage, unsign
     }
     cudaError_t e = cudaGetDevice(&h->dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
-    if (e == cudaSuccess) h->tile = plan_tiles(h);
+    if (e == cudaSuccess) plan_launches(h);
     const size_t fbytes = size_t(9) * h->plane * h->elem;
     const size_t cbytes = size_t(h->plane) * h->celem;
     // the scalar grid has the most blocks
@@ -793,7 +884,10 @@ glbm_status glbm_set_medium(glbm_t h, const double *eps, const double *K, double
     if (h->storage == GLBM_F16DEV) h->scale = fp16_scale_for(16.0 * (std::fabs(h->gx) + std::fabs(h->gy)));
     h->has_medium = true;
     h->feps_mode = F_eps;
-    h->forch = F_eps != 0.0;
+    if (h->forch != (F_eps != 0.0)) {
+        h->forch = F_eps != 0.0;
+        plan_launches(h);
+    }
     return GLBM_OK;
 }
 
@@ -1158,6 +1252,7 @@ glbm_status glbm_load(glbm_t h, const char *path) {
     h->tstep = hd.tstep;
     h->steps = hd.steps;
     h->has_medium = true;
+    plan_launches(h);
     return GLBM_OK;
 }
 

@@ -939,10 +939,10 @@ k_step(const T *__restrict__ src, T *__restrict__ dst, const typename Store<T>::
 constexpr int kPairThreads = 32;
 template <typename T>
 constexpr int kPairWarps = sizeof(T) == 2 ? 16 : 12;  // resident warps per SM
-// Fewest nodes for which k_pair is used: below, the lattice stays in L2, there
+// Fewest nodes for which k_pair is considered: below, the lattice stays in L2, there
 // is less than a warp's worth of rows per segment and the one-step kernel is
 // faster (1024^2: FP32 8.4 against 8.9 us a step, BF16 6.9 against 8.4; 1280^2:
-// 16.4 against 15.6 and 11.4 against 10.6).
+// 16.4 against 11.6 and 11.5 against 10.9).
 constexpr long long kPairNodes = 5ll << 18;
 constexpr int kStripLanes = 30;              // lanes of a strip that store
 constexpr int kStripCols = 4 * kStripLanes;  // columns of a strip
