@@ -465,31 +465,34 @@ __device__ __forceinline__ f2 rsqrt_(f2 a) { return mk2(rsqrt_(lo2(a)), rsqrt_(h
 struct Pair2 {
     f2 one, half, quarter, hgx, hgy, ngx, ngy, k1;
     f2 omH, omJ, nA3, nthird, we, wo, nwo, w1, nw1, w2, nw2;  // 32-bit storage
-    f2 cA, cO, ncO, w1om, four, cO3, ncA3, cO2, ncA;     // 16-bit storage
-    f2 scale, inv_s;
+    f2 cA, ncO, w1om, four, cO3, ncA3, cO2, ncA;     // 16-bit storage
+    f2 inv_s;
 };
 inline Pair2 make_pair2(const Phys<float> &p) {
     Pair2 c;
     const float w1 = 1.0f / 9.0f, om = p.omega, cA = (3.0f * w1) * p.A, cO = (1.5f * w1) * om;
     c.one = bc2(1.0f), c.half = bc2(0.5f), c.quarter = bc2(0.25f);
-    c.hgx = bc2(0.5f * p.gx), c.hgy = bc2(0.5f * p.gy), c.ngx = bc2(-p.gx), c.ngy = bc2(-p.gy);
+    const float gx = p.gx * p.scale, gy = p.gy * p.scale;  // FP16: with the storage scale (else 1)
+    c.hgx = bc2(0.5f * gx), c.hgy = bc2(0.5f * gy), c.ngx = bc2(-gx), c.ngy = bc2(-gy);
     c.k1 = bc2(1.0f - om);
     c.omH = bc2(0.5f * p.odd.a), c.omJ = bc2(p.odd.a), c.nA3 = bc2(-p.odd.b);
     c.nthird = bc2(-(1.0f / 3.0f)), c.we = bc2(3.0f * p.odd.c), c.wo = bc2(p.odd.c), c.nwo = bc2(-p.odd.c);
     c.w1 = bc2(w1), c.nw1 = bc2(-w1);
     c.w2 = bc2(0.25f * w1), c.nw2 = bc2(-0.25f * w1);
-    c.cA = bc2(cA), c.ncA = bc2(-cA), c.cO = bc2(cO), c.ncO = bc2(-cO), c.w1om = bc2(w1 * om), c.four = bc2(4.0f);
+    c.cA = bc2(cA), c.ncA = bc2(-cA), c.ncO = bc2(-cO), c.w1om = bc2(w1 * om), c.four = bc2(4.0f);
     c.cO3 = bc2(3.0f * cO), c.ncA3 = bc2(-(3.0f * cA)), c.cO2 = bc2(2.0f * cO);
-    c.scale = bc2(p.scale), c.inv_s = bc2(p.inv_scale);
+    c.inv_s = bc2(p.inv_scale);
     return c;
 }
 
 // node_velocity for a pair.  SCALED: populations as stored in FP16, g S with S
-// a power of two.  A power of two commutes with every rounding, so it enters
-// where the sums leave the populations (drho, 1 / rho) and where the update
-// returns to them (rho in collide_small2): 3 multiplications instead of one per
-// population on the way in and on the way out, and the same bits (2048^2 FP16
-// 27.0 -> 24.9 us a step).
+// a power of two.  A power of two commutes with every rounding, so the whole
+// update runs on S drho, S u and S F (the launch constants bring S G) and S
+// leaves only rho, the products of two of them (rho / eps in collide_small2) and
+// the square roots' arguments: 2 multiplications (4 with Forchheimer) instead of
+// one per population on the way in and on the way out, and the same bits (2048^2
+// FP16 27.0 -> 25.2 us a step).  Nothing is multiplied by S rho / eps, which
+// leaves FP32's range where eps^2 G is below 1e-35.
 template <bool FORCH, bool SCALED = false>
 __device__ __forceinline__ void node_velocity2(const f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c, f2 &drho,
                                                f2 &rho, f2 &ux, f2 &uy) {
@@ -498,12 +501,13 @@ __device__ __forceinline__ void node_velocity2(const f2 (&g)[9], f2 alpha, f2 ep
     const f2 d57 = rsub(g[5], g[7]), d86 = rsub(g[8], g[6]);
     const f2 mx = radd(radd(rsub(g[1], g[3]), d57), d86);
     const f2 my = rsub(radd(rsub(g[2], g[4]), d57), d86);
-    const f2 ir = SCALED ? rmul(rrcp(rho), c.inv_s) : rrcp(rho);
+    const f2 ir = rrcp(rho);
     const f2 vx = rfma(mx, ir, rmul(eps, c.hgx)), vy = rfma(my, ir, rmul(eps, c.hgy));
     f2 den;
     if (FORCH) {
         const f2 c0 = rfma(c.quarter, alpha, c.half), c1 = rmul(c.half, beta);
-        const f2 vmag = rsqrt_(rfma(vx, vx, rmul(vy, vy)));
+        f2 vmag = rsqrt_(rfma(vx, vx, rmul(vy, vy)));
+        if (SCALED) vmag = rmul(vmag, c.inv_s);
         den = radd(c0, rsqrt_(rfma(c1, vmag, rmul(c0, c0))));
     } else {
         den = rfma(c.half, alpha, c.one);
@@ -548,20 +552,20 @@ __device__ __forceinline__ void collide2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, 
     g[0] = radd(g[0], radd(radd(l1, l2), radd(l5, l6)));
 }
 
-// collide_small for a pair (SCALED: drho and rho carry the scale).
+// collide_small for a pair (SCALED: see node_velocity2).
 template <bool FORCH, bool SCALED>
 __device__ __forceinline__ void collide_small2(f2 (&g)[9], f2 alpha, f2 eps, f2 beta, const Pair2 &c) {
     f2 drho, rho, ux, uy;
     node_velocity2<FORCH, SCALED>(g, alpha, eps, beta, c, drho, rho, ux, uy);
-    if (SCALED) rho = rmul(rho, c.scale);
     f2 nFx = rfma(eps, c.ngx, rmul(alpha, ux)), nFy = rfma(eps, c.ngy, rmul(alpha, uy));  // -F
     const f2 uu = rfma(ux, ux, rmul(uy, uy));
     if (FORCH) {
-        const f2 bu = rmul(beta, rsqrt_(uu));
+        const f2 umag = SCALED ? rmul(rsqrt_(uu), c.inv_s) : rsqrt_(uu);
+        const f2 bu = rmul(beta, umag);
         nFx = rfma(bu, ux, nFx);
         nFy = rfma(bu, uy, nFy);
     }
-    const f2 ier = rmul(rrcp(eps), rho);
+    const f2 ier = rmul(rrcp(eps), SCALED ? rmul(rho, c.inv_s) : rho);
     const f2 nuF = rfma(ux, nFx, rmul(uy, nFy));
     const f2 C1 = rfma(c.w1om, drho, rmul(ier, rfma(c.ncO, uu, rmul(c.cA, nuF))));
     const f2 P1 = rmul(c.cO3, ier), Q1 = rmul(c.ncA3, ier);
