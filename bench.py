@@ -217,10 +217,13 @@ def peaks():
     return 6800.0, "fallback"
 
 
-def step_launches(launches, chunks, storage):
-    """Step kernels among `launches`: a chunk also takes a finalize and, in
-    16-bit storage, a step counter update."""
-    return launches - chunks * (2 if ELEM[storage] == 2 else 1)
+def other_launches(steps, storage, check_every=100, tested=False):
+    """Launches of one ``Solver.step`` call that are not step kernels (on a user
+    stream, rescaling of FP16 aside): a finalize per chunk with a convergence
+    test or FP16's range check, else one for the last chunk, and in 16-bit
+    storage a step counter update per chunk."""
+    chunks = -(-steps // check_every)
+    return (chunks if tested or storage == "f16" else 1) + (chunks if ELEM[storage] == 2 else 0)
 
 
 def bytes_per_update(storage, launches, steps):
@@ -316,7 +319,7 @@ def format_throughput(a, eps, K, steps=300):
         e1.record(stream)
         e1.synchronize()
         us = e0.elapsed_time(e1) * 1e3 / steps
-        bpu = bytes_per_update(st, step_launches(s.counters()[1] - l0, 1, st), steps)
+        bpu = bytes_per_update(st, s.counters()[1] - l0 - other_launches(steps, st), steps)
         out[st] = {"glups": a.nx * a.ny / us / 1e3, "us_per_step": us,
                    "bytes_per_node_update": bpu,
                    "frac_of_measured_hbm": bpu * a.nx * a.ny / us / 1e3 / peaks()[0]}
@@ -537,7 +540,7 @@ def sweep(a):
             sec = e0.elapsed_time(e1) * 1e-3
             glups = a.nx * a.ny * done / sec / 1e9
             bytes_per = bytes_per_update(
-                a.storage, step_launches(s.counters()[1] - l0, -(-done // 1000), a.storage), done)
+                a.storage, s.counters()[1] - l0 - other_launches(done, a.storage, 1000, tested=True), done)
             cells.append({"om_fraction": om, "corr_len": cl, "steps": done, "converged": bool(conv),
                           "glups": glups, "frac_of_measured_hbm": glups * bytes_per / peak,
                           "k_app": s.permeability()})
@@ -654,7 +657,7 @@ def run_ours(a, world, rank, local):
     value = world * updates / (ms * 1e-3) / 1e9
     # dominant kernel: the fused step, of which large lattices take two per
     # launch (the finalize kernel adds ~3 us per chunk, included here)
-    launches = step_launches(l1 - l0, a.steps, a.storage)
+    launches = l1 - l0 - a.steps * other_launches(a.chunk, a.storage)
     bpu = bytes_per_update(a.storage, launches, a.chunk * a.steps)
     per_launch_s = ms * 1e-3 / launches
     achieved = bpu * N * a.chunk * a.steps / (ms * 1e-3) / 1e9
