@@ -127,6 +127,9 @@ __device__ const fx::Table g_exp_table = fx::make_table();
 // partials 1154, one pass in FP64 instructions 131, as written 55
 // (4 blocks of 4 warps 62, 4 of 8 60, 2 of 16 60); the FP64 pipe is busy 74 % of
 // the time its SM works.
+// K = 7 and 8 hold 50 and 56 KB of static shared memory, more than 48, which CUDA 13
+// admits for sm_103a; at 188 and 210 registers one block fits an SM, and the grid
+// runs in two waves (10^6 samples, 8 components: 222 us an iteration, two passes 2610).
 // part: 3K sums, product, rest (doubles) and exponents, [3K + 3][blocks].
 template <int K>
 __global__ void __launch_bounds__(STEP_THREADS)
@@ -419,7 +422,7 @@ extern "C" glbm_status glbm_em_gmm1d(const double *x, long long m, int k, double
             k_em_finalize<<<1, EM_THREADS, 0, st>>>(part, nb, m, 2, tol, &dh->p, &dh->s, dh->sw);
         } else {
             for (int i = 0; i < n; ++i) launch_em_step<1>(k, nbs, st, xs, m, &dh->p, &dh->s, tol, part);
-            batch = std::min(2 * batch, 16);
+            batch = 2 * std::min(batch, 8);
         }
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&hs, &dh->s, sizeof(EmState), cudaMemcpyDeviceToHost, st);

@@ -81,12 +81,12 @@ struct glbm {
     // 16-bit storage: device copy of tstep, read by the step kernels of
     // replayed graphs for their stochastic-rounding key
     unsigned *dclock = nullptr;
-    // chunks replayed from captured CUDA graphs (any storage, on a
-    // non-legacy stream): key = (buffer parity at start, steps, reduce at
-    // end, test, tol, FP16 scale)
     int nsm = 0;              // SMs of the device
     TilePlan tile{};          // multi-step tiles of small or odd lattices (steps = 0: not used)
     bool pairs = false;       // two steps per launch (k_pair)
+    // chunks replayed from captured CUDA graphs (any storage, on a
+    // non-legacy stream): key = (buffer parity at start, steps, reduce at
+    // end, test, tol, FP16 scale)
     struct Graph {
         int parity, end_parity, end_behind;
         long long launches, chunk;

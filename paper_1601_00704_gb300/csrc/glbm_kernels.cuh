@@ -928,14 +928,16 @@ k_step(const T *__restrict__ src, T *__restrict__ dst, const typename Store<T>::
 // columns (6 %).  Rows y0 - 1 and y1 of a segment [y0, y1) are recomputed by
 // its neighbours' warps (2/rows).  One warp per block and no barriers.
 //
-// The arithmetic runs on packed pairs because issue, not HBM, is the next
-// bound (scalar: 147 instructions per node and step, packed: 107).  Registers
+// The arithmetic runs on packed pairs because issue would be the next bound
+// (scalar: 147 instructions per node and step, packed: 107).  Registers
 // are what is scarce: with the upward rows and the next row's loads in
 // registers, or at 5 warps per scheduler, the loop spills and loses 20 %.
 // FP32 runs best at 12 warps per SM (fewer DRAM streams), 16-bit at 16;
 // cp.async.cg, a barrier per row and 128-thread blocks were slower.
-// 4096^2, us a step: FP32 195 -> 107, BF16 112 -> 86; 2048^2: FP32 49.6 -> 28.1,
-// FP16 29.6 -> 24.9.  FP32 then moves 0.9 of the copy bandwidth.
+// 4096^2, us a step: FP32 191 -> 108 (Forchheimer 201 -> 116), BF16 110 -> 87;
+// 2048^2: FP32 49.5 -> 28.0, FP16 30.0 -> 25.2.  FP32 then moves 0.9 of the copy
+// bandwidth; 16-bit storage is bound by latency at 4 warps per scheduler (issue
+// active 60 % of the time, 0.64 of the copy bandwidth).
 //
 // Both steps round, and draw their stochastic-rounding words, exactly as the
 // one-step kernel does, so the results are its bits.

@@ -118,27 +118,25 @@ k_tc_conv(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUt
             drain_ring(full, S, i);
         }
     } else if (warp == 1) {
-        {
-            const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
-            const uint32_t idesc = idesc_bf16(a.cout);
-            for (int i = 0; i < iters; ++i) {
-                const int s = i % S, use = i / S;
-                if (!mbar_wait(&full[s], use & 1, &abort_flag, a.err, 2)) break;
-                tc_fence_after();
-                const uint64_t bd = sdesc_k64(sB + s * stage_b);
+        const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
+        const uint32_t idesc = idesc_bf16(a.cout);
+        for (int i = 0; i < iters; ++i) {
+            const int s = i % S, use = i / S;
+            if (!mbar_wait(&full[s], use & 1, &abort_flag, a.err, 2)) break;
+            tc_fence_after();
+            const uint64_t bd = sdesc_k64(sB + s * stage_b);
 #pragma unroll
-                for (int t = 0; t < MT; ++t) {
-                    const uint64_t ad = sdesc_k64(sA + (s * MT + t) * TC_STAGE_A);
+            for (int t = 0; t < MT; ++t) {
+                const uint64_t ad = sdesc_k64(sA + (s * MT + t) * TC_STAGE_A);
 #pragma unroll
-                    for (int kk = 0; kk < TC_KC / 16; ++kk)  // K = 16 per MMA: 32 bytes along the row
-                        umma_bf16_if(one, tmem + uint32_t(t) * a.acc_cols, ad + uint64_t((kk * 32) >> 4),
-                                  bd + uint64_t((kk * 32) >> 4), idesc, (i > 0 || kk > 0) ? 1u : 0u);
-                }
-                umma_commit_if(one, &empty[s]);
+                for (int kk = 0; kk < TC_KC / 16; ++kk)  // K = 16 per MMA: 32 bytes along the row
+                    umma_bf16_if(one, tmem + uint32_t(t) * a.acc_cols, ad + uint64_t((kk * 32) >> 4),
+                              bd + uint64_t((kk * 32) >> 4), idesc, (i > 0 || kk > 0) ? 1u : 0u);
             }
-            umma_commit_if(one, &done);  // after a timeout too: the wait below retires every MMA issued
-            mbar_drain(&done, 0);
+            umma_commit_if(one, &empty[s]);
         }
+        umma_commit_if(one, &done);  // after a timeout too: the wait below retires every MMA issued
+        mbar_drain(&done, 0);
     } else {
         const int q = warp & 3;  // TMEM lanes 32q..32q+31 belong to this warp
         // after a timeout the MMA warp still commits `done` (to retire its MMAs):
@@ -760,136 +758,134 @@ k_tc_conv_stream(const __grid_constant__ CUtensorMap mapA0, const __grid_constan
             drain_ring(full, S, i);
         }
     } else if (warp == 1) {
-        {
-            const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
-            // MMA shapes: the main N (three output rows) and the clearing
-            // of a row pair's two slots
-            const uint32_t idN = idesc_bf16(3 * COUT), idZ = idesc_bf16(2 * COUT);
-            bool ok = a.wstream || mbar_wait(&wfull, 0, &abort_flag, a.err, 22);
-            tc_fence_after();
-            const uint64_t zdesc = sdesc_nosw(smem_u32(szero), 2048u, 128u);
-            const uint64_t wdesc = sdesc_k64(sW);
-            const uint32_t wt16 = a.wtile >> 4;
-            const int kks = a.kks;
-            // A in 16-byte units: a pixel is 4, a K step of 16 channels 2
-            constexpr uint32_t kRow = BAND_PX * 4, kPx = 4, kStep = 2;
-            const uint32_t d13 = uint32_t((NS - 3) * COUT);
-            RingPos at;
-            for (int g = 0; g < ngroups && ok; ++g) {
-                // pairs hg g + 1 .. hg g + hg enter their slots: wait until the
-                // epilogue has drained each one's last stored occupant, then
-                // clear them
-                for (int pn = hg * g + 1; pn <= hg * g + hg && ok; ++pn) {
-                    const int ps = pn % NP, prev = pn - NP;
-                    if (prev >= 1 && prev <= npairs &&
-                        !mbar_wait(&pempty[ps], uint32_t((prev - 1) / NP) & 1u, &abort_flag, a.err, 23)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
+        const uint32_t one = lane == 0;  // this lane issues; the waits and addresses are the warp's
+        // MMA shapes: the main N (three output rows) and the clearing
+        // of a row pair's two slots
+        const uint32_t idN = idesc_bf16(3 * COUT), idZ = idesc_bf16(2 * COUT);
+        bool ok = a.wstream || mbar_wait(&wfull, 0, &abort_flag, a.err, 22);
+        tc_fence_after();
+        const uint64_t zdesc = sdesc_nosw(smem_u32(szero), 2048u, 128u);
+        const uint64_t wdesc = sdesc_k64(sW);
+        const uint32_t wt16 = a.wtile >> 4;
+        const int kks = a.kks;
+        // A in 16-byte units: a pixel is 4, a K step of 16 channels 2
+        constexpr uint32_t kRow = BAND_PX * 4, kPx = 4, kStep = 2;
+        const uint32_t d13 = uint32_t((NS - 3) * COUT);
+        RingPos at;
+        for (int g = 0; g < ngroups && ok; ++g) {
+            // pairs hg g + 1 .. hg g + hg enter their slots: wait until the
+            // epilogue has drained each one's last stored occupant, then
+            // clear them
+            for (int pn = hg * g + 1; pn <= hg * g + hg && ok; ++pn) {
+                const int ps = pn % NP, prev = pn - NP;
+                if (prev >= 1 && prev <= npairs &&
+                    !mbar_wait(&pempty[ps], uint32_t((prev - 1) / NP) & 1u, &abort_flag, a.err, 23)) {
+                    ok = false;
+                    break;
                 }
-                for (int ri = 0; ri < G && ok && rowwise; ++ri) {
-                    const int row = G * g + ri, s0 = row % NS, st0 = at.s;
-                    RingPos w = at;
-                    for (int ch = 0; ch < a.nchunk && ok; ++ch, w.next(S))
-                        ok = mbar_wait(&full[w.s], w.parity, &abort_flag, a.err, 24);
-                    if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t a0 = sdesc_k64(sA);
-                    // slots s0 .. s0 + 2, or those up to the ring's end and then the rest
-                    const int head = min(3, NS - s0);
-                    for (int part = 0; part < (head < 3 ? 2 : 1); ++part) {
-                        const uint32_t d = tmem + uint32_t(part ? 0 : s0 * COUT);
-                        const uint32_t id = idesc_bf16((part ? 3 - head : head) * COUT);
-                        const uint64_t b0 = wdesc + uint64_t((part ? head : 0) * wt16);
+                tc_fence_after();
+                umma_bf16_if(one, tmem + uint32_t(2 * ps * COUT), zdesc, zdesc, idZ, 0u);
+            }
+            for (int ri = 0; ri < G && ok && rowwise; ++ri) {
+                const int row = G * g + ri, s0 = row % NS, st0 = at.s;
+                RingPos w = at;
+                for (int ch = 0; ch < a.nchunk && ok; ++ch, w.next(S))
+                    ok = mbar_wait(&full[w.s], w.parity, &abort_flag, a.err, 24);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t a0 = sdesc_k64(sA);
+                // slots s0 .. s0 + 2, or those up to the ring's end and then the rest
+                const int head = min(3, NS - s0);
+                for (int part = 0; part < (head < 3 ? 2 : 1); ++part) {
+                    const uint32_t d = tmem + uint32_t(part ? 0 : s0 * COUT);
+                    const uint32_t id = idesc_bf16((part ? 3 - head : head) * COUT);
+                    const uint64_t b0 = wdesc + uint64_t((part ? head : 0) * wt16);
 #pragma unroll 1
-                        for (int dxi = 0; dxi < 3; ++dxi)
+                    for (int dxi = 0; dxi < 3; ++dxi)
 #pragma unroll 1
-                            for (int ch = 0; ch < a.nchunk; ++ch) {
-                                const int s = st0 + ch < S ? st0 + ch : st0 + ch - S;
-                                const uint64_t ar = a0 + uint64_t(uint32_t(s) * (a.stage_bytes >> 4) + uint32_t(dxi) * kPx);
-                                const uint64_t br = b0 + uint64_t(uint32_t(3 * (3 * ch + dxi)) * wt16);
-                                umma_bf16_if(one, d, ar, br, id, 1u);
-                                umma_bf16_if(one, d, ar + kStep, br + 2, id, 1u);
-                            }
-                    }
-                    for (int ch = 0; ch < a.nchunk; ++ch, at.next(S)) umma_commit_if(one, &empty[at.s]);
-                }
-                for (int ch = 0; ch < a.nchunk && ok && !rowwise; ++ch, at.next(S)) {
-                    const int s = at.s;
-                    if (!mbar_wait(&full[s], at.parity, &abort_flag, a.err, 24)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint64_t a0 = sdesc_k64(sA + size_t(s) * a.stage_bytes);
-                    if (!ZEROS) {
-                        // the weights of a dx are [W(+1) W(0) W(-1)], resident or in this stage
-                        const uint64_t b0 = a.wstream ? sdesc_k64(sA + size_t(s) * a.stage_bytes + a.wofs)
-                                                      : wdesc + uint64_t(uint32_t(9 * ch) * wt16);
-#pragma unroll 1
-                        for (int ri = 0; ri < G; ++ri) {
-                            const uint64_t arow = a0 + uint64_t(ri * kRow);
-                            const int s0 = (G * g + ri) % NS, head = min(3, NS - s0);
-                            // slots s0 .. s0 + 2, or those up to the ring's end and then the rest
-                            for (int part = 0; part < (head < 3 ? 2 : 1); ++part) {
-                                const uint32_t d = tmem + uint32_t(part ? 0 : s0 * COUT);
-                                const uint32_t id = idesc_bf16((part ? 3 - head : head) * COUT);
-                                const uint64_t bp = b0 + uint64_t((part ? head : 0) * wt16);
-#pragma unroll
-                                for (int dxi = 0; dxi < 3; ++dxi)
-#pragma unroll
-                                    for (int kk = 0; kk < 2; ++kk)
-                                        if (kk < kks)
-                                            umma_bf16_if(one, d, arow + uint64_t(dxi * kPx + kk * kStep),
-                                                         bp + uint64_t(3 * dxi * wt16 + kk * 2), id, 1u);
-                            }
+                        for (int ch = 0; ch < a.nchunk; ++ch) {
+                            const int s = st0 + ch < S ? st0 + ch : st0 + ch - S;
+                            const uint64_t ar = a0 + uint64_t(uint32_t(s) * (a.stage_bytes >> 4) + uint32_t(dxi) * kPx);
+                            const uint64_t br = b0 + uint64_t(uint32_t(3 * (3 * ch + dxi)) * wt16);
+                            umma_bf16_if(one, d, ar, br, id, 1u);
+                            umma_bf16_if(one, d, ar + kStep, br + 2, id, 1u);
                         }
-                        umma_commit_if(one, &empty[s]);
-                        continue;
-                    }
-                    // B of (chunk, dx) group k starts at tile 2 + 5k: [W(+1) W(0) W(-1)]
-                    const uint64_t b0 = wdesc + uint64_t((2 + 15 * ch) * wt16);
+                }
+                for (int ch = 0; ch < a.nchunk; ++ch, at.next(S)) umma_commit_if(one, &empty[at.s]);
+            }
+            for (int ch = 0; ch < a.nchunk && ok && !rowwise; ++ch, at.next(S)) {
+                const int s = at.s;
+                if (!mbar_wait(&full[s], at.parity, &abort_flag, a.err, 24)) {
+                    ok = false;
+                    break;
+                }
+                tc_fence_after();
+                const uint64_t a0 = sdesc_k64(sA + size_t(s) * a.stage_bytes);
+                if (!ZEROS) {
+                    // the weights of a dx are [W(+1) W(0) W(-1)], resident or in this stage
+                    const uint64_t b0 = a.wstream ? sdesc_k64(sA + size_t(s) * a.stage_bytes + a.wofs)
+                                                  : wdesc + uint64_t(uint32_t(9 * ch) * wt16);
 #pragma unroll 1
                     for (int ri = 0; ri < G; ++ri) {
-                        // input row G g + ri feeds the slots of rows G g + ri .. + 2
-                        const int s0 = (G * g + ri) % NS;
                         const uint64_t arow = a0 + uint64_t(ri * kRow);
-                        if (s0 <= NS - 3) {
-                            const uint32_t d0 = tmem + uint32_t(s0 * COUT);
+                        const int s0 = (G * g + ri) % NS, head = min(3, NS - s0);
+                        // slots s0 .. s0 + 2, or those up to the ring's end and then the rest
+                        for (int part = 0; part < (head < 3 ? 2 : 1); ++part) {
+                            const uint32_t d = tmem + uint32_t(part ? 0 : s0 * COUT);
+                            const uint32_t id = idesc_bf16((part ? 3 - head : head) * COUT);
+                            const uint64_t bp = b0 + uint64_t((part ? head : 0) * wt16);
 #pragma unroll
                             for (int dxi = 0; dxi < 3; ++dxi)
 #pragma unroll
                                 for (int kk = 0; kk < 2; ++kk)
                                     if (kk < kks)
-                                        umma_bf16_if(one, d0, arow + uint64_t(dxi * kPx + kk * kStep),
-                                                  b0 + uint64_t(5 * dxi * wt16 + kk * 2), idN, 1u);
-                        } else {
-                            // slots 13-15 take B shifted by 1 (s0 = 14: [0 W(+1) W(0)]) or
-                            // 2 (s0 = 15: [0 0 W(+1)]) tiles; slots 0-2 the rest, shifted
-                            // the other way ([W(-1) 0 0] or [W(0) W(-1) 0])
-                            const uint32_t sh = uint32_t(s0 - (NS - 3));  // 1 or 2
-#pragma unroll
-                            for (int dxi = 0; dxi < 3; ++dxi)
-#pragma unroll
-                                for (int kk = 0; kk < 2; ++kk) {
-                                    if (kk >= kks) break;
-                                    const uint64_t ad = arow + uint64_t(dxi * kPx + kk * kStep);
-                                    const uint64_t bk = b0 + uint64_t(5 * dxi * wt16 + kk * 2);
-                                    umma_bf16_if(one, tmem + d13, ad, bk - uint64_t(sh * wt16), idN, 1u);
-                                    umma_bf16_if(one, tmem, ad, bk + uint64_t((3 - sh) * wt16), idN, 1u);
-                                }
+                                        umma_bf16_if(one, d, arow + uint64_t(dxi * kPx + kk * kStep),
+                                                     bp + uint64_t(3 * dxi * wt16 + kk * 2), id, 1u);
                         }
                     }
                     umma_commit_if(one, &empty[s]);
+                    continue;
                 }
-                for (int pc = hg * g; pc < hg * g + hg && ok; ++pc)
-                    if (pc >= 1 && pc <= npairs) umma_commit_if(one, &pfull[pc % NP]);
+                // B of (chunk, dx) group k starts at tile 2 + 5k: [W(+1) W(0) W(-1)]
+                const uint64_t b0 = wdesc + uint64_t((2 + 15 * ch) * wt16);
+#pragma unroll 1
+                for (int ri = 0; ri < G; ++ri) {
+                    // input row G g + ri feeds the slots of rows G g + ri .. + 2
+                    const int s0 = (G * g + ri) % NS;
+                    const uint64_t arow = a0 + uint64_t(ri * kRow);
+                    if (s0 <= NS - 3) {
+                        const uint32_t d0 = tmem + uint32_t(s0 * COUT);
+#pragma unroll
+                        for (int dxi = 0; dxi < 3; ++dxi)
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk)
+                                if (kk < kks)
+                                    umma_bf16_if(one, d0, arow + uint64_t(dxi * kPx + kk * kStep),
+                                              b0 + uint64_t(5 * dxi * wt16 + kk * 2), idN, 1u);
+                    } else {
+                        // slots 13-15 take B shifted by 1 (s0 = 14: [0 W(+1) W(0)]) or
+                        // 2 (s0 = 15: [0 0 W(+1)]) tiles; slots 0-2 the rest, shifted
+                        // the other way ([W(-1) 0 0] or [W(0) W(-1) 0])
+                        const uint32_t sh = uint32_t(s0 - (NS - 3));  // 1 or 2
+#pragma unroll
+                        for (int dxi = 0; dxi < 3; ++dxi)
+#pragma unroll
+                            for (int kk = 0; kk < 2; ++kk) {
+                                if (kk >= kks) break;
+                                const uint64_t ad = arow + uint64_t(dxi * kPx + kk * kStep);
+                                const uint64_t bk = b0 + uint64_t(5 * dxi * wt16 + kk * 2);
+                                umma_bf16_if(one, tmem + d13, ad, bk - uint64_t(sh * wt16), idN, 1u);
+                                umma_bf16_if(one, tmem, ad, bk + uint64_t((3 - sh) * wt16), idN, 1u);
+                            }
+                    }
+                }
+                umma_commit_if(one, &empty[s]);
             }
-            umma_commit_if(one, &drainbar);  // retire every MMA issued, also after a timeout
-            mbar_drain(&drainbar, 0);
+            for (int pc = hg * g; pc < hg * g + hg && ok; ++pc)
+                if (pc >= 1 && pc <= npairs) umma_commit_if(one, &pfull[pc % NP]);
         }
+        umma_commit_if(one, &drainbar);  // retire every MMA issued, also after a timeout
+        mbar_drain(&drainbar, 0);
     } else if (warp >= 4) {
         const int q = warp & 3;  // TMEM lanes 32q..32q+31 belong to this warp
         const int px = x0 + q * 32 + lane;
