@@ -355,10 +355,11 @@ __device__ __forceinline__ void collide(R (&g)[9], R alpha, R eps, R beta,
     // neighbouring densities (exact by Sterbenz's lemma once within a factor
     // of two), so one rounding per node remains instead of nine: errors 30x below
     // the unclosed update's.  Against FP64, relative to the separate f_eq and F_i
-    // terms with TwoSum sums before and after (geometric means over tau = 0.55 .. 2,
-    // 3000 to 10 000 steps): two-phase media velocity 0.75, density 0.56; clear and
-    // porous blocks velocity 0.79, density 1.02 +- 0.04 (with TwoSum sums 0.92); a
-    // clear channel, where rounding scatters, velocity 0.97, density 0.64.
+    // terms with TwoSum sums before and after, geometric means over tau = 0.55 .. 2:
+    // four two-phase media velocity 0.65, density 0.46; blocks of clear and porous
+    // rock (35 lattices of 24 to 48 nodes a side) 0.66 and 0.88 +- 0.02, with TwoSum
+    // sums 0.77; clear channels, where rounding scatters tenfold from tau to tau,
+    // 0.95 and 0.63.
     const R l1 = collide_pair<R>(g[1], g[3], w1, drho, k1, ux, Hx, Jx, q, we1, wo1);
     const R l2 = collide_pair<R>(g[2], g[4], w1, drho, k1, uy, Hy, Jy, q, we1, wo1);
     const R l5 = collide_pair<R>(g[5], g[7], w2, drho, k1, radd(ux, uy), radd(Hx, Hy), radd(Jx, Jy), q, we2, wo2);
