@@ -568,8 +568,8 @@ void glbm_nn_tc_debug_starve(int stage);
  * 0 (default) = per layer: 3x3 layers with BF16 output, rows of >= 128
  * pixels and 32 or 64 output channels, or 128, 192 or 256 (in groups of 64) of
  * at most 128 input channels, run the streaming kernel where one CTA per
- * (image, 128-pixel strip, group) leaves segments of >= 16 rows (groups: >= 4)
- * per SM (each CTA walks down its strip, each input row multiplied once into a
+ * (image, 128-pixel strip, group) leaves segments of >= 16 rows (groups: >= 4,
+ * and CTAs for 0.65 of the SMs) per SM (each CTA walks down its strip, each input row multiplied once into a
  * ring of row accumulators in tensor memory; the three vertical taps stacked
  * into one MMA of 96 or 192 columns; groups add up in the order of the tile
  * kernel and have its bits; 64-channel layers whose weights exceed shared memory take them

@@ -388,7 +388,7 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
     // FP32 kernels that fit 16 blocks per SM by their registers would be given so
     // much shared memory that L1 no longer holds the rows that neighbouring strips
     // and segments share (Forchheimer with walls: 2048^2 53 -> 33 us a step, 4096^2
-    // 191 -> 116); 132 KB is what the driver gives the others
+    // 191 -> 116); 132 KB is what the others get
     cudaError_t err = cudaSuccess;
     if (sizeof(T) == 4)
         err = cudaFuncSetAttribute(k_pair<T, WALLS, FORCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 58);

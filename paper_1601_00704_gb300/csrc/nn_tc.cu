@@ -1386,6 +1386,9 @@ bool stream_plan(int w, int h, int n, int cin, int cout, int nsm, StreamPlan *p,
     if (l < (g_tc_variant == 5 ? 2 : least)) return false;
     p->L = l;
     p->nseg = (h + l - 1) / l;
+    // groups take about 0.65 of the tile kernel's time on all SMs, so fewer CTAs
+    // than that lose to it (128 -> 256, 4 x 356 x 697, 96 CTAs: 717 us, there 680)
+    if (p->groups > 1 && g_tc_variant != 5 && units * p->nseg * 20 < (long long)nsm * 13) return false;
     p->wstream = !resident;
     p->ystages = up2 ? 2 : 0;
     // the tallest group that leaves three stages: 6, 4 or 2 rows with 32

@@ -26,7 +26,8 @@ def _vp(t):
 @pytest.mark.parametrize("n,h,w,c0,c1,cout,variant", [
     (1, 512, 512, 128, 128, 128, 0), (1, 611, 130, 128, 64, 128, 0), (1, 700, 128, 96, 64, 256, 0),
     (1, 37, 300, 224, 0, 192, 5), (2, 33, 130, 128, 128, 256, 5), (1, 2, 128, 160, 0, 128, 5), (1, 65, 129, 96, 96, 128, 5),
-    (1, 40, 256, 128, 128, 192, 5), (1, 600, 128, 160, 128, 128, 0), (1, 300, 256, 64, 64, 128, 0)])
+    (1, 40, 256, 128, 128, 192, 5), (1, 600, 128, 160, 128, 128, 0), (1, 300, 256, 64, 64, 128, 0),
+    (4, 24, 650, 64, 64, 256, 0), (3, 24, 650, 32, 0, 192, 0)])
 def test_grouped_layers_have_the_tile_kernels_bits(lib, n, h, w, c0, c1, cout, variant):
     import torch
     g = torch.Generator(device="cuda").manual_seed(h * w + c0 + cout)
