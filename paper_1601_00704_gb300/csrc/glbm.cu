@@ -83,6 +83,7 @@ struct glbm {
     unsigned *dclock = nullptr;
     int nsm = 0;              // SMs of the device
     TilePlan tile{};          // multi-step tiles of small or odd lattices (steps = 0: not used)
+    int tile_least = 0;       // fewest steps that pay for a tile's launch
     bool pairs = false;       // two steps per launch (k_pair)
     // chunks replayed from captured CUDA graphs (any storage, on a
     // non-legacy stream): key = (buffer parity at start, steps, reduce at
@@ -219,8 +220,8 @@ TilePlan tile_of(const glbm *h, int T, int q, int R) {
     return p;
 }
 
-// us of a launch whose steps take `step` + `warp` per warp and scheduler
-double tile_us(const glbm *h, const TilePlan &p, double step, double warp) {
+// us of a launch of n steps that take `step` + `warp` per warp and scheduler
+double tile_us(const glbm *h, const TilePlan &p, int n, double step, double warp) {
     const int Q = 1 << p.q_log2, R = p.rows;
     const int fit = std::min(65536 / (96 * R * Q), 227 * 1024 / (192 * (R + 2) * Q + 1024));
     const long long tiles = (long long)p.nx_tiles * p.ny_tiles;
@@ -228,7 +229,7 @@ double tile_us(const glbm *h, const TilePlan &p, double step, double warp) {
     const long long rounds = (per_sm + side - 1) / side;
     // rows of the halo drop out as their reach shrinks
     const double warps = double(side) * R * Q / 128.0 * (R - p.hy) / R;
-    return (h->elem == 2 ? 1.71 : 1.85) + double(rounds) * p.steps * (step + warp * warps);
+    return (h->elem == 2 ? 1.71 : 1.85) + double(rounds) * n * (step + warp * warps);
 }
 
 struct PairPlan {
@@ -278,6 +279,7 @@ void plan_launches(glbm *h) {
     const bool odd = h->nx % 4 != 0, small = h->elem == 2;
     h->pairs = false;
     h->tile = TilePlan{};
+    h->tile_least = 0;
     if (h->storage == GLBM_F64 || (small && !h->sr)) return;
     const double one = one_step_us(h);
     if (!odd && h->N >= kPairNodes) {
@@ -299,12 +301,17 @@ void plan_launches(glbm *h) {
             for (int R = 2 * (T - 1) + 1; R << q <= kTileThreads; ++R) {
                 if ((R << q) % 32 || (odd && T == 2 && R << q > kTileThreads / 2)) continue;
                 const TilePlan p = tile_of(h, T, q, R);
-                const double l = tile_us(h, p, small ? 0.31 : 0.28, small ? 0.405 : 0.37);
+                const double l = tile_us(h, p, T, small ? 0.31 : 0.28, small ? 0.405 : 0.37);
                 const double t = (h->stream ? l : std::max(5.0, l)) / T;
                 if (t < least) least = t, best = p;
             }
+    // the rest of a chunk may be too few steps for a launch with the halo of many
     const LaunchCost &c = cost_of(h);
-    if (launch_us(h, tile_us(h, best, c.step, c.warp)) / best.steps < launch_us(h, one)) h->tile = best;
+    for (int n = best.steps; n >= 2; --n) {
+        if (launch_us(h, tile_us(h, best, n, c.step, c.warp)) >= n * launch_us(h, one)) break;
+        h->tile = best;
+        h->tile_least = n;
+    }
 }
 
 int grid_1d(long long N) {
@@ -370,9 +377,19 @@ glbm_status do_step(glbm *h, bool reduce, long long clock_off = -1) {
     return GLBM_EINVAL;
 }
 
-// Two steps in one launch (k_pair).
+// Two steps in one launch (k_pair).  `prepare`: only set what the function keeps
+// for the process.
 template <typename T, bool WALLS, bool FORCH>
-glbm_status launch_pair_t(glbm *h, long long clock_off) {
+glbm_status launch_pair_t(glbm *h, long long clock_off, bool prepare) {
+    if (prepare) {
+        // FP32 kernels that fit 16 blocks per SM by their registers would be given so
+        // much shared memory that L1 no longer holds the rows that neighbouring strips
+        // and segments share (Forchheimer with walls: 2048^2 53 -> 33 us a step, 4096^2
+        // 191 -> 116); 132 KB is what the others get
+        if (sizeof(T) == 4)
+            CU(h, cudaFuncSetAttribute(k_pair<T, WALLS, FORCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 58));
+        return GLBM_OK;
+    }
     const Geo geo = make_geo(h, 4);
     Phys<float> ph = make_phys<float>(h);
     if (Store<T>::kSmall && clock_off >= 0) {
@@ -385,19 +402,11 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
     if (refused) return fail(h, GLBM_ECUDA, "step launch: injected failure (test hook)");
     const PairPlan pl = pair_plan(h);
     const dim3 grid(unsigned(pl.strips) * unsigned(pl.segs));
-    // FP32 kernels that fit 16 blocks per SM by their registers would be given so
-    // much shared memory that L1 no longer holds the rows that neighbouring strips
-    // and segments share (Forchheimer with walls: 2048^2 53 -> 33 us a step, 4096^2
-    // 191 -> 116); 132 KB is what the others get
-    cudaError_t err = cudaSuccess;
-    if (sizeof(T) == 4)
-        err = cudaFuncSetAttribute(k_pair<T, WALLS, FORCH>, cudaFuncAttributePreferredSharedMemoryCarveout, 58);
-    if (err == cudaSuccess)
-        err = launch_kernel_smem(
-            k_pair<T, WALLS, FORCH>, grid, dim3(kPairThreads), sizeof(StripSmem<T, FORCH>), h->stream,
-            h->stream != nullptr, static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
-            static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
-            static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), pl.strips, pl.rows);
+    const cudaError_t err = launch_kernel_smem(
+        k_pair<T, WALLS, FORCH>, grid, dim3(kPairThreads), sizeof(StripSmem<T, FORCH>), h->stream,
+        h->stream != nullptr, static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
+        static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
+        static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), pl.strips, pl.rows);
     if (err != cudaSuccess) return fail(h, GLBM_ECUDA, "step launch: %s", cudaGetErrorString(err));
     h->launches++;
     h->tstep += 2;
@@ -407,24 +416,32 @@ glbm_status launch_pair_t(glbm *h, long long clock_off) {
 }
 
 template <typename T>
-glbm_status launch_pair(glbm *h, long long co) {
+glbm_status launch_pair(glbm *h, long long co, bool prepare) {
     if (!(h->flags & GLBM_PERIODIC_Y))
-        return h->forch ? launch_pair_t<T, true, true>(h, co) : launch_pair_t<T, true, false>(h, co);
-    return h->forch ? launch_pair_t<T, false, true>(h, co) : launch_pair_t<T, false, false>(h, co);
+        return h->forch ? launch_pair_t<T, true, true>(h, co, prepare) : launch_pair_t<T, true, false>(h, co, prepare);
+    return h->forch ? launch_pair_t<T, false, true>(h, co, prepare) : launch_pair_t<T, false, false>(h, co, prepare);
 }
 
-glbm_status do_pair(glbm *h, long long clock_off = -1) {
+glbm_status do_pair(glbm *h, long long clock_off, bool prepare = false) {
     switch (h->storage) {
-        case GLBM_F16DEV: return launch_pair<__half>(h, clock_off);
-        case GLBM_BF16DEV: return launch_pair<__nv_bfloat16>(h, clock_off);
-        default: return launch_pair<float>(h, clock_off);
+        case GLBM_F16DEV: return launch_pair<__half>(h, clock_off, prepare);
+        case GLBM_BF16DEV: return launch_pair<__nv_bfloat16>(h, clock_off, prepare);
+        default: return launch_pair<float>(h, clock_off, prepare);
     }
 }
 
-// Several steps of every tile in one launch (k_tile), `n` <= plan.steps.
+// Several steps of every tile in one launch (k_tile), `n` <= plan.steps.  n = 0:
+// only set what the function keeps for the process.
 template <typename T, bool WALLS, bool FORCH, bool ODD>
 glbm_status launch_tile_t(glbm *h, int n, long long clock_off) {
     const TilePlan &pl = h->tile;
+    if (n == 0) {
+        // the limit belongs to the function, for every handle and thread: always the
+        // most that any plan takes, so that no launch is refused what another set
+        CU(h, cudaFuncSetAttribute(k_tile<T, WALLS, FORCH, ODD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   int(kTileSmem)));
+        return GLBM_OK;
+    }
     const Geo geo = make_geo(h, 4);
     Phys<float> ph = make_phys<float>(h);
     if (Store<T>::kSmall && clock_off >= 0) {
@@ -436,19 +453,12 @@ glbm_status launch_tile_t(glbm *h, int n, long long clock_off) {
     if (refused) return fail(h, GLBM_ECUDA, "step launch: injected failure (test hook)");
     const int Q = 1 << pl.q_log2;
     const size_t smem = tile_bytes(pl.rows, Q);
-    // the limit belongs to the function, for every handle and thread: always the
-    // most that any plan takes, so that no launch is refused what another set
-    cudaError_t err = cudaSuccess;
-    if (smem > 48 * 1024)
-        err = cudaFuncSetAttribute(k_tile<T, WALLS, FORCH, ODD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   int(kTileSmem));
-    if (err == cudaSuccess)
-        err = launch_kernel_smem(
-            k_tile<T, WALLS, FORCH, ODD>, dim3(unsigned(pl.nx_tiles) * unsigned(pl.ny_tiles)),
-            dim3(unsigned(Q * pl.rows)), smem, h->stream, h->stream != nullptr,
-            static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
-            static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
-            static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), pl, n);
+    const cudaError_t err = launch_kernel_smem(
+        k_tile<T, WALLS, FORCH, ODD>, dim3(unsigned(pl.nx_tiles) * unsigned(pl.ny_tiles)),
+        dim3(unsigned(Q * pl.rows)), smem, h->stream, h->stream != nullptr,
+        static_cast<const T *>(h->buf[h->cur]), static_cast<T *>(h->buf[h->cur ^ 1]),
+        static_cast<const float *>(h->coef[0]), static_cast<const float *>(h->coef[1]),
+        static_cast<const float *>(h->coef[2]), geo, ph, make_pair2(ph), pl, n);
     if (err != cudaSuccess) return fail(h, GLBM_ECUDA, "step launch: %s", cudaGetErrorString(err));
     h->launches++;
     h->tstep += n;
@@ -474,6 +484,13 @@ glbm_status do_tile(glbm *h, int n, long long co) {
     }
 }
 
+// Choose the kernels (plan_launches) and set their functions up.
+glbm_status plan(glbm *h) {
+    plan_launches(h);
+    if (h->pairs) return do_pair(h, -1, true);
+    return h->tile.steps ? do_tile(h, 0, -1) : GLBM_OK;
+}
+
 // `chunk` steps, the last one reducing when `reduce`.  That one is a launch of
 // its own: the velocity export reads the state before it.
 glbm_status do_steps(glbm *h, long long chunk, bool reduce, bool clocked) {
@@ -485,7 +502,7 @@ glbm_status do_steps(glbm *h, long long chunk, bool reduce, bool clocked) {
         glbm_status st;
         int done = n;
         if (pairs && s + 2 <= plain) st = do_pair(h, co);
-        else if (!pairs && n >= 2) st = do_tile(h, n, co);
+        else if (!pairs && n >= std::max(2, h->tile_least)) st = do_tile(h, n, co);
         else st = do_step(h, reduce && s == chunk - 1, co), done = 1;
         if (st) return st;
         s += done;
@@ -812,7 +829,6 @@ glbm_status glbm_create(int nx, int ny, double tau, glbm_storage storage, unsign
     }
     cudaError_t e = cudaGetDevice(&h->dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->dev);
-    if (e == cudaSuccess) plan_launches(h);
     const size_t fbytes = size_t(9) * h->plane * h->elem;
     const size_t cbytes = size_t(h->plane) * h->celem;
     // the scalar grid has the most blocks
@@ -841,6 +857,12 @@ glbm_status glbm_create(int nx, int ny, double tau, glbm_storage storage, unsign
         return s;
     }
     memset(h->hstat, 0, sizeof(DevStatus));
+    if (glbm_status s = plan(h)) {
+        fail(nullptr, s, "glbm_create: %s", h->err);
+        release(h);
+        delete h;
+        return s;
+    }
     *out = h;
     return GLBM_OK;
 }
@@ -886,7 +908,7 @@ glbm_status glbm_set_medium(glbm_t h, const double *eps, const double *K, double
     h->feps_mode = F_eps;
     if (h->forch != (F_eps != 0.0)) {
         h->forch = F_eps != 0.0;
-        plan_launches(h);
+        return plan(h);
     }
     return GLBM_OK;
 }
@@ -1252,8 +1274,7 @@ glbm_status glbm_load(glbm_t h, const char *path) {
     h->tstep = hd.tstep;
     h->steps = hd.steps;
     h->has_medium = true;
-    plan_launches(h);
-    return GLBM_OK;
+    return plan(h);
 }
 
 void glbm_destroy(glbm_t h) {
